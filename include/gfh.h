@@ -135,17 +135,17 @@ typedef struct gfh_peaks {
 } gfh_peaks;
 
 /* Tile shape of the Hough kernel; zero fields pick the library default (16 x 3072, 512).  The
- * tile (rows x (cols + 2) int32 plus the candidate keys) must fit in 227 KB of shared memory.
- * form chooses how a warp draws its 32 peaks: 0 = each peak in its own form (interior peaks, clear
- * of the tile's edges on every row, in a shorter form than peaks near an edge; a warp holding both
- * runs both), 1 = one form per warp (the edge-following form for all 32 as soon as one needs it).
- * The maps are identical; 1 pays where many warps mix the two kinds of peak (narrow tiles, tall
- * maps).  The coarse-tile search always draws one form per warp. */
+ * default stands for tiles planned by the library: their rows and columns follow each region's
+ * estimated work, and heavy tiles are split until every block has its share.  Any other shape is
+ * taken as it is, drawn in strips of half its columns (a cell has two counts while it is drawn).  A
+ * shape of which rows x (cols + 2) int32 plus the candidate keys exceed 227 KB is refused.
+ * form is accepted for compatibility (0 or 1) and selects nothing: every warp draws edge event by
+ * edge event.  The maps do not depend on the shape. */
 typedef struct gfh_tile_config {
   int32_t rows;     /* k rows per tile: 4, 8, 16 or 32 */
   int32_t cols;     /* x0 columns per tile: multiple of 128, at most 4096 */
   int32_t threads;  /* threads per block: 256 or 512, or 1024 with 16 or 32 rows */
-  int32_t form;     /* drawing form: 0 or 1 */
+  int32_t form;     /* 0 or 1, no effect */
 } gfh_tile_config;
 
 /* Context: binds a device and a stream (cudaStream_t passed as void*; NULL = legacy default). */
@@ -299,9 +299,9 @@ int gfh_plan_execute(gfh_plan* plan, const gfh_peaks* peaks);
 /*
  * Autotuner: times gfh_plan_execute on these peaks (reps runs each, CUDA events on the context's
  * stream) for the current tile shape and for every shape of rows {4, 8, 16} x cols {1024, 2048,
- * 3072, 4096} x threads {256, 512} (and 1024 threads for 16 rows) that fits in shared memory,
- * then the fastest shape with the other drawing form, and rebuilds the plan with the fastest.  The results are unchanged by the shape (the maps are
- * exact).  Synchronises; writes the bound outputs.  h_best / h_best_ms (may be NULL) receive the
+ * 3072, 4096} x threads {256, 512} (and 1024 threads for 16 rows) that fits in shared memory, the
+ * planned tiles of the default shape among them, and rebuilds the plan with the fastest.  The
+ * results are unchanged by the shape (the maps are exact).  Synchronises; writes the bound outputs.  h_best / h_best_ms (may be NULL) receive the
  * chosen shape and its time.
  * The choice is cached for the life of the process, keyed by the plan's signature: the device
  * (compute capability, SM count), whether candidates are selected, and per map its k rows, x0
@@ -586,9 +586,9 @@ int gfh_conv3x3(gfh_ctx* ctx, int32_t mode, int32_t cin, int32_t cout, int32_t s
  * -1 where no cell of the band was computed).  cr and the statistics come from sums over the
  * computed cells only (a cell computed twice counts twice) with the map's full cell count: they
  * are comparable with those of gfh_plan_execute only for maps searched in full.  A peak list whose
- * bins hold their peaks in FFT order (as gfh_peakmap emits them) lets narrow fine tiles read only
- * the peaks of the FFTs that can meet them; any other bin-sorted list is read in full, with the
- * same results.  Asynchronous, allocation-free, capturable.
+ * bins hold their peaks in FFT order (as gfh_peakmap emits them) lets tiles read only the peaks of
+ * the FFTs that can have an edge in them; any other bin-sorted list is read in full, with the same
+ * results.  Asynchronous, allocation-free, capturable.
  */
 int gfh_plan_set_coarse(gfh_plan* plan, int32_t coarse_k, int32_t coarse_x, int32_t max_sel);
 int gfh_plan_execute_tiles(gfh_plan* plan, const gfh_peaks* peaks, const int32_t* d_coarse,

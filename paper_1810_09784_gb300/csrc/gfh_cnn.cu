@@ -32,7 +32,6 @@
 namespace {
 
 constexpr int kImg = 256;
-constexpr size_t kSmemPerSm = 228 * 1024;   // shared memory of one SM
 constexpr int kTiles = 64;
 constexpr int kClasses = kTiles * kTiles + 1;
 

@@ -370,12 +370,29 @@ extern "C" int gfh_tfft_portions(double n, double f_hi, double fdot_hi, double t
 
 namespace {
 
+// ceil(2^89 / s) (FftRow::D) for a shift per row s > 2^25, else 0.
+uint64_t rows_per_column(int64_t s) {
+  if (s <= (int64_t(1) << 25)) return 0;
+  const unsigned __int128 one = 1;
+  return (uint64_t)(((one << 89) + (uint64_t)s - 1) / (uint64_t)s);
+}
+
 struct HostMap {
   std::vector<int64_t> U, B, S;
   std::vector<int32_t> band;
   std::vector<double> f0, f0n;
   int64_t cells = 0;
+  int64_t ana_lo = 0, ana_hi = -1;   // first and last analysis column (contiguous: f0 falls with the column)
 };
+
+void find_analysis_columns(HostMap& hm) {
+  const int64_t n = (int64_t)hm.band.size();
+  int64_t a = 0, b = n - 1;
+  while (a < n && hm.band[a] < 0) ++a;
+  while (b >= a && hm.band[b] < 0) --b;
+  hm.ana_lo = a;
+  hm.ana_hi = b;
+}
 
 // Bin range [ja, jb] of the peaks that can touch columns [c0, c1) on rows [r0, r1) (tile planning).
 // For bin j (local jl) and shift s in [s_min, s_max]: lo >= (U[jl+1]-s_max)>>32 and
@@ -402,98 +419,189 @@ void tile_bins(const gfh_grid& g, const HostMap& hm, int64_t s_min, int64_t s_ma
   *jb = g.bin_lo + b;
 }
 
-// Bins per tile of the coarse-tile search's FFT sub-ranges (8 bytes each in shared memory) that
-// fit beside a tile of `base` bytes without lowering the blocks per SM (228 KB per SM, 1 KB of it
-// reserved per block, at most the Hough kernels' limit per block), at most 1024.
-int sub_capacity(size_t base, int threads) {
-  constexpr size_t kSmemSM = 228 * 1024, kReserve = 1024, kOwn = kMaxSmemBytes - kHoughSmemLimit;
-  const int blocks = (int)std::min<size_t>(kSmemSM / (base + kOwn + kReserve), (size_t)(2048 / threads));
-  if (blocks < 1) return 0;
-  const size_t room = std::min(kSmemSM / blocks - kReserve - kOwn, kHoughSmemLimit);
-  if (room <= base + 16) return 0;
-  const size_t cap = std::min<size_t>((room - base - 16) / 8, 1024);
-  return cap >= 32 ? (int)cap : 0;
+// Candidate bands of columns [c0, c1) (bands follow the columns): lo > hi when there is none.
+void column_bands(const HostMap& hm, int64_t c0, int64_t c1, int32_t* lo, int32_t* hi) {
+  const int64_t a = std::max(c0, hm.ana_lo), b = std::min(c1 - 1, hm.ana_hi);
+  *lo = 0;
+  *hi = -1;
+  if (a > b) return;
+  *lo = std::min(hm.band[a], hm.band[b]);
+  *hi = std::max(hm.band[a], hm.band[b]);
 }
 
-// Number of FFTs whose interval of bin jl (local) meets columns c0 .. ub on some of the R rows
-// from row0 (B_i + r S_i does not fall as i grows when k_min >= 0: two bisections).
-int64_t window_ffts(const gfh_grid& g, const HostMap& hm, int jl, int row0, int R, int64_t c0,
-                    int64_t ub) {
-  const int64_t x_hi = hm.U[jl] - 1 - (c0 << GFH_FRAC_BITS);
-  const int64_t y_lo = hm.U[jl + 1] - ((ub + 1) << GFH_FRAC_BITS);
-  const int64_t r_last = (int64_t)row0 + R - 1;
-  int lo = 0, hi = g.n_fft;
-  while (lo < hi) {
-    const int mid = (lo + hi) / 2;
-    if (hm.B[mid] + (int64_t)row0 * hm.S[mid] <= x_hi) lo = mid + 1; else hi = mid;
+TileDev make_tile(const gfh_grid& g, const HostMap& hm, int m, int r0, int nr, int64_t c0, int nc) {
+  // With k_min >= 0, B and S are non-decreasing in i (dk > 0, t_i non-decreasing), so the smallest
+  // shift of the rows is at (i = 0, r0) and the largest at (last i, last row).  With k_min < 0
+  // (n = 0 only) the shift of FFT i on row r is (k_min + r dk) t_i up to its rounding: its extremes
+  // are at the first and last FFT and row, one lattice unit per row aside.
+  const int last = g.n_fft - 1, r1 = r0 + nr - 1;
+  int64_t s_min = hm.B[0] + (int64_t)r0 * hm.S[0], s_max = hm.B[last] + (int64_t)r1 * hm.S[last];
+  if (g.k_min < 0.0) {
+    for (int i : {0, last})
+      for (int r : {r0, r1}) {
+        const int64_t v = hm.B[i] + (int64_t)r * hm.S[i];
+        s_min = std::min(s_min, v - 2 - r1);
+        s_max = std::max(s_max, v + 2 + r1);
+      }
   }
-  const int last = lo - 1;
-  lo = 0;
-  hi = last + 1;
-  while (lo < hi) {
-    const int mid = (lo + hi) / 2;
-    if (hm.B[mid] + r_last * hm.S[mid] > y_lo) hi = mid; else lo = mid + 1;
-  }
-  return last - lo + 1;
+  TileDev t{};
+  t.map = m;
+  t.row0 = r0;
+  t.nrows = nr;
+  t.col0 = c0;
+  t.ncols = nc;
+  tile_bins(g, hm, s_min, s_max, c0, c0 + nc, &t.bin_a, &t.bin_b);
+  column_bands(hm, c0, c0 + nc, &t.band_lo, &t.band_hi);
+  return t;
 }
 
-// Whether a tile of the coarse-tile search walks only its bins' FFT sub-ranges: they fit
-// (sub_cap), the shifts grow with the FFT (k_min >= 0) and, over up to 8 bins sampled across the
-// tile's bin range, at most half the (FFT, bin) pairs read meet the tile.
-bool tile_walks_sub_ranges(const gfh_grid& g, const HostMap& hm, const TileDev& t, int R,
-                           int sub_cap) {
+// Work of a tile, in warp instructions: measured costs of the kernel's parts (an empty tile, one
+// with edges, its cells, a run of 32 peaks and its two events per column moved), with the peaks that
+// have an edge in it estimated from up to 8 of its bins along the line that the shifts follow, at
+// the density of noise peaks.
+double tile_work(const gfh_grid& g, const HostMap& hm, const TileDev& t) {
+  const double cells = (double)t.nrows * t.ncols;
   const int nb = t.bin_b - t.bin_a + 1;
-  if (sub_cap <= 0 || nb <= 0 || nb > sub_cap || g.k_min < 0.0 || g.n_fft < 1) return false;
-  const int64_t c0 = t.col0;
-  const int64_t ub = std::min<int64_t>(c0 + t.ncols - 1, g.n_x0 - 1);
+  const double fill = 2500.0 + cells / 128.0 * 3.0;
+  if (nb <= 0) return fill;
+  const int n = g.n_fft;
+  const double one = 1.0 / 4294967296.0;
+  const int64_t r0 = t.row0, r1 = r0 + t.nrows - 1;
+  const double b0 = (double)(hm.B[0] + r0 * hm.S[0]) * one, b1 = (double)(hm.B[0] + r1 * hm.S[0]) * one;
+  const double e0 = (double)(hm.B[n - 1] + r0 * hm.S[n - 1]) * one,
+               e1 = (double)(hm.B[n - 1] + r1 * hm.S[n - 1]) * one;
+  const double s0 = n > 1 ? (e0 - b0) / (n - 1) : 0.0, s1 = n > 1 ? (e1 - b1) / (n - 1) : 0.0;
   const int samples = std::min(nb, 8);
-  int64_t meet = 0;
+  double ffts = 0.0, moved = 0.0;
   for (int q = 0; q < samples; ++q) {
     const int jl = t.bin_a - g.bin_lo + (int)((int64_t)q * (nb - 1) / std::max(1, samples - 1));
-    meet += std::max<int64_t>(0, window_ffts(g, hm, jl, t.row0, R, c0, ub));
+    const double hi_x = (double)hm.U[jl] * one - (double)t.col0;              // right edge
+    const double lo_x = (double)hm.U[jl + 1] * one - (double)t.col0;          // left edge
+    double lo = 0.0, hi = n;
+    auto at_most = [&](double x, double b, double s) {                        // b + i s <= x
+      if (s > 0.0) hi = std::min(hi, (x - b) / s);
+      else if (s < 0.0) lo = std::max(lo, (x - b) / s);
+      else if (b > x) hi = lo;
+    };
+    at_most(hi_x, b0, s0);                                                    // reaches the first column
+    at_most(-(lo_x - t.ncols), -b1, -s1);                                     // not past the last
+    double len = std::max(0.0, hi - lo);
+    const double mid = 0.5 * (lo + hi);
+    if (hi_x - lo_x > t.ncols && len > 0.0) {                                 // FFTs that cover the tile
+      lo = 0.0;
+      hi = n;
+      at_most(-(lo_x - 1.0), -b0, -s0);
+      at_most(hi_x - t.ncols, b1, s1);
+      len = std::max(0.0, len - std::max(0.0, hi - lo));
+    }
+    const double i = std::min(std::max(mid, 0.0), (double)(n - 1));
+    const double shift = t.nrows > 1 ? ((b1 - b0) + i * (s1 - s0)) / (t.nrows - 1) : 0.0;
+    ffts += len;
+    moved += len * shift * (t.nrows - 1);
   }
-  return (double)meet <= 0.5 * (double)samples * (double)g.n_fft;
+  const double runs = 0.0755 / 32.0 * nb / samples;
+  if (ffts <= 0.0) return fill;
+  return 8000.0 + cells / 128.0 * 50.0 + 8.0 * nb + runs * (190.0 * ffts + 16.0 * moved);
 }
 
-// Tiles of map m covering rows [r0, r1) x columns [c_lo, c_hi) (c_lo, c_hi multiples of 4) with
-// the plan's tile shape; appended to `tiles`.
-void map_tiles(const gfh_grid& g, const HostMap& hm, int m, const gfh_tile_config& tc, int r0,
-               int r1, int64_t c_lo, int64_t c_hi, std::vector<TileDev>& tiles, int& max_bands) {
-  for (int rr = r0; rr < r1; rr += tc.rows) {
-    const int nr = std::min(tc.rows, r1 - rr);
-    // With k_min >= 0, B and S are non-decreasing in i (dk > 0, t_i non-decreasing), so the
-    // smallest shift of the row block is at (i = 0, rr) and the largest at (last i, last row).
-    // With k_min < 0 (n = 0 only) B falls with i: the shift of FFT i is linear in the row, so
-    // its extremes over the block are at the block's first and last rows, taken over every i.
-    int64_t s_min = hm.B[0] + (int64_t)rr * hm.S[0];
-    int64_t s_max = hm.B[g.n_fft - 1] + (int64_t)(rr + nr - 1) * hm.S[g.n_fft - 1];
-    if (g.k_min < 0.0) {
-      for (int i = 0; i < g.n_fft; ++i) {
-        const int64_t a = hm.B[i] + (int64_t)rr * hm.S[i];
-        const int64_t b = hm.B[i] + (int64_t)(rr + nr - 1) * hm.S[i];
-        s_min = std::min(s_min, std::min(a, b));
-        s_max = std::max(s_max, std::max(a, b));
+// Rows x columns of a tile with a given room (words of one of its two counts).
+int64_t tile_words(int rows, int cols) { return (int64_t)rows * (cols + kHoughPad); }
+int cols_for(int rows, int64_t words) {
+  return (int)std::min<int64_t>(4096, std::max<int64_t>(64, (words / rows - kHoughPad) / 64 * 64));
+}
+
+// Tiles of map m over rows [r0, r1) x columns [c_lo, c_hi) (both multiples of 4).  Chosen shapes: per
+// region of kTall rows by the columns of the flattest shape, the shape of least work.  Tall, narrow
+// tiles halve the peaks' fixed work with every doubling of the rows, flat wide ones suit regions with
+// few edges, whose cost is the cells'.
+void map_tiles(const gfh_grid& g, const HostMap& hm, int m, const TilePlan& tp, int r0, int r1,
+               int64_t c_lo, int64_t c_hi, std::vector<TileDev>& tiles) {
+  auto cut = [&](int a, int b, int64_t c, int64_t d, int rows, int cols, std::vector<TileDev>& out) {
+    for (int r = a; r < b; r += rows)
+      for (int64_t x = c; x < d; x += cols)
+        out.push_back(make_tile(g, hm, m, r, std::min(rows, b - r), x, (int)std::min<int64_t>(cols, d - x)));
+  };
+  if (tp.rows > 0) {
+    cut(r0, r1, c_lo, c_hi, tp.rows, tp.cols, tiles);
+    return;
+  }
+  constexpr int kTall = 128, kFlat = 8;
+  const int wide = cols_for(kFlat, tp.words);
+  std::vector<TileDev> best, cand;
+  for (int a = r0; a < r1; a += kTall) {
+    const int b = std::min(r1, a + kTall);
+    for (int64_t c = c_lo; c < c_hi; c += wide) {
+      const int64_t d = std::min(c_hi, c + wide);
+      double best_work = -1.0;
+      for (int rows = kFlat; rows <= kTall; rows *= 2) {
+        cand.clear();
+        cut(a, b, c, d, rows, cols_for(rows, tp.words), cand);
+        double work = 0.0;
+        for (const TileDev& t : cand) work += tile_work(g, hm, t);
+        if (best_work < 0.0 || work < best_work) { best_work = work; best.swap(cand); }
+        if (rows >= b - a) break;
       }
-    }
-    for (int64_t c0 = c_lo; c0 < c_hi; c0 += tc.cols) {
-      TileDev t{};
-      t.map = m;
-      t.row0 = rr;
-      t.nrows = nr;
-      t.col0 = c0;
-      t.ncols = (int32_t)std::min<int64_t>(tc.cols, c_hi - c0);
-      tile_bins(g, hm, s_min, s_max, c0, c0 + t.ncols, &t.bin_a, &t.bin_b);
-      t.band_lo = INT32_MAX;
-      t.band_hi = -1;
-      for (int64_t c = c0; c < c0 + t.ncols; ++c) {
-        const int32_t b = hm.band[c];
-        if (b >= 0) { t.band_lo = std::min(t.band_lo, b); t.band_hi = std::max(t.band_hi, b); }
-      }
-      if (t.band_hi < 0) t.band_lo = 0;
-      else max_bands = std::max(max_bands, t.band_hi - t.band_lo + 1);
-      tiles.push_back(t);
+      tiles.insert(tiles.end(), best.begin(), best.end());
     }
   }
+}
+
+// Halves the tiles that hold more than `most` work, across columns or rows as makes the least of it.
+void split_tiles(const std::vector<gfh_grid>& grids, const std::vector<HostMap>& hms, double most,
+                 std::vector<TileDev>& tiles, std::vector<double>& work) {
+  for (size_t q = 0; q < tiles.size(); ++q) {
+    while (work[q] > most) {
+      const TileDev t = tiles[q];
+      const gfh_grid& g = grids[t.map];
+      const HostMap& hm = hms[t.map];
+      TileDev a{}, b{};
+      double wa = 0.0, wb = 0.0;
+      bool found = false;
+      auto offer = [&](const TileDev& x, const TileDev& y) {
+        const double u = tile_work(g, hm, x), v = tile_work(g, hm, y);
+        if (!found || std::max(u, v) + 0.5 * (u + v) < std::max(wa, wb) + 0.5 * (wa + wb)) {
+          a = x; b = y; wa = u; wb = v;
+          found = true;
+        }
+      };
+      if (t.ncols >= 16) {
+        const int h = (t.ncols / 2 + 3) & ~3;
+        offer(make_tile(g, hm, t.map, t.row0, t.nrows, t.col0, h),
+              make_tile(g, hm, t.map, t.row0, t.nrows, t.col0 + h, t.ncols - h));
+      }
+      if (t.nrows >= 2) {
+        const int h = (t.nrows + 1) / 2;
+        offer(make_tile(g, hm, t.map, t.row0, h, t.col0, t.ncols),
+              make_tile(g, hm, t.map, t.row0 + h, t.nrows - h, t.col0, t.ncols));
+      }
+      if (!found || std::max(wa, wb) > 0.9 * work[q]) break;
+      tiles[q] = a;
+      work[q] = wa;
+      tiles.push_back(b);
+      work.push_back(wb);
+    }
+  }
+}
+
+// Most work first (ties by map, so that a block's consecutive tiles are often of one map).
+void sort_tiles(std::vector<TileDev>& tiles, const std::vector<double>& work) {
+  std::vector<int32_t> at(tiles.size());
+  std::iota(at.begin(), at.end(), 0);
+  std::stable_sort(at.begin(), at.end(), [&](int32_t x, int32_t y) { return work[x] > work[y]; });
+  std::vector<TileDev> out(tiles.size());
+  for (size_t q = 0; q < at.size(); ++q) out[q] = tiles[at[q]];
+  tiles.swap(out);
+}
+
+// Shared-memory bytes of the largest tile's counts (x: the x-direction form, whole tiles of `rows`),
+// and the most bands in a tile.
+size_t tile_bytes(const std::vector<TileDev>& tiles, int rows_x, int* bands) {
+  int64_t words = 0;
+  for (const TileDev& t : tiles) {
+    words = std::max(words, tile_words(rows_x > 0 ? rows_x : t.nrows, t.ncols));
+    *bands = std::max(*bands, t.band_hi - t.band_lo + 1);
+  }
+  return (size_t)words * 8;
 }
 
 }  // namespace
@@ -527,14 +635,21 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
       tc.cols > 4096 || !(tc.form == 0 || tc.form == 1) ||
       !(tc.threads == 256 || tc.threads == 512 || (tc.threads == 1024 && tc.rows >= 16)))
     return GFH_ERR_ARG;
+  // The default shape stands for tiles planned by their work (512 threads, two blocks per SM); any
+  // other is taken as it is, in strips of half its columns (a cell has two counts).
+  const bool planned = tc.rows == 16 && tc.cols == 3072 && tc.threads == 512 && tc.form == 0;
   const int nwarps = tc.threads / 32;
   if ((tc.cols / 128 + nwarps - 1) / nwarps > 4) return GFH_ERR_ARG;  // <= 4 chunks per warp
 
   std::vector<HostMap> hms(n_maps);
   std::vector<TileDev> tiles, tiles_x;
+  // (a strip leaves 24 KB of shared memory for the chunk sums, band keys and windows)
+  const TilePlan shape{tc.rows, std::min(tc.cols / 2, cols_for(tc.rows, (int64_t)(kHoughSmemLimit - 24 * 1024) / 8)), 0};
+  const TilePlan chosen{0, 0, kPlannedWords};
   std::vector<char> map_xd(n_maps, 0);
-  int max_tile_bands = 1;
-  size_t csr_entries = 0;
+  int max_tile_bands = 1, cfg_bands = 1;
+  std::map<int, ListDev> by_list;           // per list read: the bins and FFTs that its maps cover
+  std::map<int, int> list_ffts;
   for (int m = 0; m < n_maps; ++m) {
     const gfh_grid& g = grids[m];
     if (!grid_made(&g) || !h_maps[m]) return GFH_ERR_ARG;
@@ -548,52 +663,91 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
     int64_t ana_cols = 0;
     for (int64_t c = 0; c < g.n_x0; ++c) ana_cols += hm.band[c] >= 0;
     hm.cells = ana_cols * g.n_k;
-    csr_entries += (size_t)(g.bin_hi - g.bin_lo + 2);
+    auto ins = by_list.insert({g.list, ListDev{nullptr, nullptr, g.list, g.bin_lo, g.bin_hi + 1, 0, 0, 0}});
+    ListDev& ld = ins.first->second;             // n_bins holds the end of the bins for now
+    ld.bin_lo = std::min(ld.bin_lo, g.bin_lo);
+    ld.n_bins = std::max(ld.n_bins, g.bin_hi + 1);
+    list_ffts[g.list] = std::max(list_ffts[g.list], g.n_fft);
     if (((uintptr_t)h_maps[m]) % 16) return GFH_ERR_ARG;  // 16-byte vector stores
     // A line moving more than two columns per k row (coarse k steps, e.g. Eq. dkeqn's) costs
     // fewer events differenced along x0 on every row (2 per row) than along k (the columns it
     // crosses): such maps use the x-direction form.
     map_xd[m] = hm.S[g.n_fft - 1] > (int64_t(2) << GFH_FRAC_BITS);
-    map_tiles(g, hm, m, tc, 0, g.n_k, 0, g.ld_x0, map_xd[m] ? tiles_x : tiles, max_tile_bands);
+    find_analysis_columns(hm);
+    for (int64_t c = 0; c < g.ld_x0; c += tc.cols) {
+      int32_t lo, hi;
+      column_bands(hm, c, std::min<int64_t>(c + tc.cols, g.ld_x0), &lo, &hi);
+      cfg_bands = std::max(cfg_bands, hi - lo + 1);
+    }
+    map_tiles(g, hm, m, planned && !map_xd[m] ? chosen : shape, 0, g.n_k, 0, g.ld_x0, map_xd[m] ? tiles_x : tiles);
   }
-  // The tile must fit in shared memory (layout of k_hough: tile, chunk sums, band keys).
+  // The given tile must fit in shared memory (one count per cell, chunk sums, band keys).
   const bool select = h_cands != nullptr || d_stats != nullptr;
   const size_t smem = (size_t)tc.rows * (tc.cols + 2) * 4 + 32 * 4 * (tiles_x.empty() ? 1 : tc.rows) +
-                      (select ? (size_t)max_tile_bands * 8 : 0);
+                      (select ? (size_t)cfg_bands * 8 : 0);
   if (smem > kHoughSmemLimit) return GFH_ERR_SIZE;
-  // Longest work first: bins x rows; the x-direction tiles form a second list after the others.
-  auto by_work = [](const TileDev& a, const TileDev& b) {
-    const int64_t wa = (int64_t)std::max(0, a.bin_b - a.bin_a + 1) * a.nrows;
-    const int64_t wb = (int64_t)std::max(0, b.bin_b - b.bin_a + 1) * b.nrows;
-    return wa > wb;
-  };
-  std::stable_sort(tiles.begin(), tiles.end(), by_work);
-  std::stable_sort(tiles_x.begin(), tiles_x.end(), by_work);
+  // Most work first; the x-direction tiles form a second list after the others.
+  std::vector<double> work(tiles.size()), work_x(tiles_x.size());
+  double all = 0.0;
+  for (size_t q = 0; q < tiles.size(); ++q) all += work[q] = tile_work(grids[tiles[q].map], hms[tiles[q].map], tiles[q]);
+  for (size_t q = 0; q < tiles_x.size(); ++q)
+    work_x[q] = (double)std::max(0, tiles_x[q].bin_b - tiles_x[q].bin_a + 1) * tiles_x[q].nrows;
+  if (planned)      // enough tiles for every block to have some, and none that outlasts the others
+    split_tiles(std::vector<gfh_grid>(grids, grids + n_maps), hms, std::max(all / (6.0 * ctx->num_sms), 12000.0), tiles, work);
+  sort_tiles(tiles, work);
+  sort_tiles(tiles_x, work_x);
+  const size_t cells = tile_bytes(tiles, 0, &max_tile_bands);
+  const size_t cells_x = tile_bytes(tiles_x, tc.rows, &max_tile_bands);
   const int n_tiles_k = (int)tiles.size();
   tiles.insert(tiles.end(), tiles_x.begin(), tiles_x.end());
 
-  // One device buffer: map descriptors | tiles | csr map index | keys | per-map tables.
+  // FFT blocks of 64, or longer so that a bin has at most 256 of them
+  std::vector<ListDev> lists;
+  std::map<int, int> list_at;
+  int64_t csr_entries = 0;
+  for (auto& kv : by_list) {
+    ListDev ld = kv.second;
+    ld.n_bins -= ld.bin_lo;
+    ld.shift = 6;
+    while (((list_ffts[kv.first] - 1) >> ld.shift) + 1 > 256) ++ld.shift;
+    ld.nb1 = ((list_ffts[kv.first] - 1) >> ld.shift) + 2;
+    if (csr_entries + ld.n_bins > INT32_MAX) return GFH_ERR_SIZE;
+    ld.entry0 = (int32_t)csr_entries;
+    csr_entries += ld.n_bins;
+    list_at[kv.first] = (int)lists.size();
+    lists.push_back(ld);
+  }
+
+  // One device buffer: map descriptors | tiles | lists | index list of each bin | keys | per-map tables.
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   const size_t o_maps = take(sizeof(MapDev) * n_maps);
   const size_t o_tiles = take(sizeof(TileDev) * tiles.size());
+  const size_t o_lists = take(sizeof(ListDev) * lists.size());
   const size_t o_csrmap = take(sizeof(int32_t) * csr_entries);
+  std::vector<size_t> o_csr(lists.size()), o_blk(lists.size());
+  for (size_t l = 0; l < lists.size(); ++l) {
+    o_csr[l] = take(sizeof(int64_t) * ((size_t)lists[l].n_bins + 1));
+    o_blk[l] = take(sizeof(int32_t) * (size_t)lists[l].n_bins * lists[l].nb1);
+  }
   size_t key_words = 0;
   for (int m = 0; m < n_maps; ++m) key_words += grids[m].n_bands + 2;
-  const size_t o_keys = take(sizeof(unsigned long long) * key_words);
-  std::vector<size_t> o_U(n_maps), o_B(n_maps), o_S(n_maps), o_band(n_maps), o_f0(n_maps),
-      o_f0n(n_maps), o_csr(n_maps);
+  // (a launch takes at most 65535 lists)
+  int n_lists = 1;
+  for (int m = 0; m < n_maps; ++m) n_lists = std::max(n_lists, std::min(grids[m].list, 65535) + 1);
+  const size_t zeroed = sizeof(unsigned long long) * key_words + sizeof(int) * ((size_t)n_lists + 4);
+  const size_t o_keys = take(zeroed);
+  std::vector<size_t> o_U(n_maps), o_SD(n_maps), o_B(n_maps), o_band(n_maps), o_f0(n_maps),
+      o_f0n(n_maps);
   for (int m = 0; m < n_maps; ++m) {
     o_U[m] = take(2 * sizeof(int64_t) * (hms[m].U.size() - 1));
-    o_B[m] = take(2 * sizeof(int64_t) * hms[m].B.size());
-    o_S[m] = 0;
+    o_SD[m] = take(sizeof(FftRow) * hms[m].S.size());
+    o_B[m] = grids[m].k_min != 0.0 ? take(sizeof(int64_t) * hms[m].B.size()) : 0;
     o_band[m] = take(sizeof(int32_t) * hms[m].band.size());
     o_f0[m] = take(sizeof(double) * hms[m].f0.size());
     o_f0n[m] = take(sizeof(double) * hms[m].f0n.size());
-    o_csr[m] = take(sizeof(int64_t) * (size_t)(grids[m].bin_hi - grids[m].bin_lo + 2));
   }
   const size_t o_single = take(sizeof(int64_t) * 2);
-  const size_t o_next = take(sizeof(int) * 2);
   const size_t total = off;
 
   gfh_plan* p = new (std::nothrow) gfh_plan();
@@ -602,14 +756,23 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   p->n_maps = n_maps;
   p->grids.assign(grids, grids + n_maps);
   p->cfg = tc;
+  p->planned = planned;
+  p->shape = shape;
+  p->cells = cells;
+  p->cells_x = cells_x;
   if (cudaSetDevice(ctx->device) != cudaSuccess) { delete p; return GFH_ERR_CUDA; }
   if (cudaMalloc(&p->d_buf, total) != cudaSuccess) { delete p; return GFH_ERR_NOMEM; }
   p->buf_bytes = total;
   char* base = (char*)p->d_buf;
   std::vector<char> h(total, 0);
   std::vector<MapDev> mds(n_maps);
-  std::vector<int32_t> csr_map;
-  csr_map.reserve(csr_entries);
+  std::vector<int32_t> csr_list;
+  csr_list.reserve(csr_entries);
+  for (size_t l = 0; l < lists.size(); ++l) {
+    lists[l].csr = (int64_t*)(base + o_csr[l]);
+    lists[l].blk = (int32_t*)(base + o_blk[l]);
+    csr_list.insert(csr_list.end(), lists[l].n_bins, (int32_t)l);
+  }
   size_t key_off = 0;
   for (int m = 0; m < n_maps; ++m) {
     const gfh_grid& g = grids[m];
@@ -617,11 +780,20 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
     MapDev& md = mds[m];
     md.out = h_maps[m];
     md.UP = (const longlong2*)(base + o_U[m]);
-    md.BS = (const longlong2*)(base + o_B[m]);
+    md.SD = (const FftRow*)(base + o_SD[m]);
+    md.B = g.k_min != 0.0 ? (const int64_t*)(base + o_B[m]) : nullptr;
+    md.b0 = hm.B[0];
+    md.s0 = hm.S[0];
+    md.db = g.n_fft > 1 ? (float)((double)(hm.B[g.n_fft - 1] - hm.B[0]) / (g.n_fft - 1)) : 0.f;
+    md.ds = g.n_fft > 1 ? (float)((double)(hm.S[g.n_fft - 1] - hm.S[0]) / (g.n_fft - 1)) : 0.f;
     md.col_band = (const int32_t*)(base + o_band[m]);
     md.f0c = (const double*)(base + o_f0[m]);
     md.f0n = (const double*)(base + o_f0n[m]);
-    md.csr = (int64_t*)(base + o_csr[m]);
+    const ListDev& ld = lists[list_at[g.list]];
+    md.csr = ld.csr + (g.bin_lo - ld.bin_lo);
+    md.blk = ld.blk + (size_t)(g.bin_lo - ld.bin_lo) * ld.nb1;
+    md.nb1 = ld.nb1;
+    md.shift = ld.shift;
     md.keys = (unsigned long long*)(base + o_keys) + key_off;
     md.sums = md.keys + g.n_bands;
     key_off += g.n_bands + 2;
@@ -640,20 +812,20 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
     md.n_fft = g.n_fft;
     md.list = g.list;
     md.n_bands = g.n_bands;
-    md.csr_base = (int32_t)csr_map.size();
     // paired tables: one 16-byte load per bin and one per FFT in the kernel
     int64_t* up = (int64_t*)(h.data() + o_U[m]);
-    for (size_t j = 0; j + 1 < hm.U.size(); ++j) { up[2 * j] = hm.U[j + 1]; up[2 * j + 1] = hm.U[j]; }
-    int64_t* bs = (int64_t*)(h.data() + o_B[m]);
-    for (size_t i = 0; i < hm.B.size(); ++i) { bs[2 * i] = hm.B[i]; bs[2 * i + 1] = hm.S[i]; }
+    for (size_t j = 0; j + 1 < hm.U.size(); ++j) { up[2 * j] = hm.U[j + 1]; up[2 * j + 1] = hm.U[j] - 1; }
+    FftRow* sd = (FftRow*)(h.data() + o_SD[m]);
+    for (size_t i = 0; i < hm.S.size(); ++i) sd[i] = FftRow{hm.S[i], rows_per_column(hm.S[i])};
+    if (md.B) std::memcpy(h.data() + o_B[m], hm.B.data(), sizeof(int64_t) * hm.B.size());
     std::memcpy(h.data() + o_band[m], hm.band.data(), sizeof(int32_t) * hm.band.size());
     std::memcpy(h.data() + o_f0[m], hm.f0.data(), sizeof(double) * hm.f0.size());
     std::memcpy(h.data() + o_f0n[m], hm.f0n.data(), sizeof(double) * hm.f0n.size());
-    for (int e = 0; e < g.bin_hi - g.bin_lo + 2; ++e) csr_map.push_back(m);
   }
   std::memcpy(h.data() + o_maps, mds.data(), sizeof(MapDev) * n_maps);
   if (!tiles.empty()) std::memcpy(h.data() + o_tiles, tiles.data(), sizeof(TileDev) * tiles.size());
-  std::memcpy(h.data() + o_csrmap, csr_map.data(), sizeof(int32_t) * csr_map.size());
+  std::memcpy(h.data() + o_lists, lists.data(), sizeof(ListDev) * lists.size());
+  std::memcpy(h.data() + o_csrmap, csr_list.data(), sizeof(int32_t) * csr_list.size());
   if (cudaMemcpy(p->d_buf, h.data(), total, cudaMemcpyHostToDevice) != cudaSuccess) {
     gfh_plan_destroy(p);
     return GFH_ERR_CUDA;
@@ -664,13 +836,18 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   p->n_tiles_x = (int)tiles.size() - n_tiles_k;
   p->map_xd = map_xd;
   p->max_tile_bands = max_tile_bands;
+  p->d_zeroed = base + o_keys;
+  p->zeroed_bytes = zeroed;
   p->d_keys = (unsigned long long*)(base + o_keys);
-  p->key_words = key_words;
+  p->d_list_state = (int*)(p->d_keys + key_words);
+  p->n_list_states = n_lists;
+  p->d_next = p->d_list_state + n_lists;
+  p->d_sel_count = p->d_next + 2;
   p->csr_entries = (int32_t)csr_entries;
-  p->d_csr_map = (int32_t*)(base + o_csrmap);
+  p->d_lists = (ListDev*)(base + o_lists);
+  p->d_csr_list = (int32_t*)(base + o_csrmap);
   p->select = h_cands != nullptr || d_stats != nullptr;
   p->d_offsets_single = (int64_t*)(base + o_single);
-  p->d_next = (int*)(base + o_next);
   p->h_maps.assign(h_maps, h_maps + n_maps);
   if (h_cands) p->h_cands.assign(h_cands, h_cands + n_maps);
   p->d_stats = d_stats;
@@ -702,16 +879,8 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
   const int nct = coarse_k * coarse_x;
   std::vector<TileDev> fine;
   std::vector<int32_t> first;
-  // the search's tile, chunk sums and band keys; the FFT sub-ranges fit in what the list kernel's
-  // occupancy leaves
-  const int sub_cap = sub_capacity((size_t)p->cfg.rows * (p->cfg.cols + 2) * 4 + 32 * 4 +
-                                       (p->select ? (size_t)p->max_tile_bands * 8 + 64 : 0),
-                                   p->cfg.threads);
-  std::vector<CoarseMapDev> cms(p->n_maps);
-  std::vector<size_t> fblk_off(p->n_maps);
-  size_t fblk_total = 0;
-  int n_lists = 0, fblk_entries = 0;
   first.reserve((size_t)p->n_maps * (nct + 1) + 1);
+  const TilePlan tp = p->planned ? TilePlan{0, 0, kPlannedListWords} : p->shape;
   int max_fine = 0, max_bands = p->max_tile_bands;
   size_t worst = 0;                        // longest gathered list: every map at its largest
   for (int m = 0; m < p->n_maps; ++m) {
@@ -721,22 +890,7 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
     if (rc) return rc;
     rc = gfh_host_columns(&g, hm.band, hm.f0, hm.f0n);
     if (rc) return rc;
-    const size_t map_begin = fine.size();
-    {
-      CoarseMapDev& cm = cms[m];
-      const int J = g.bin_hi - g.bin_lo + 1;
-      cm.nb1 = (g.n_fft + kFftBlock - 1) / kFftBlock + 1;
-      cm.list = g.list;
-      cm.b0 = hm.B[0];
-      cm.s0 = hm.S[0];
-      cm.db = g.n_fft > 1 ? (double)(hm.B[g.n_fft - 1] - hm.B[0]) / (g.n_fft - 1) : 0.0;
-      cm.ds = g.n_fft > 1 ? (double)(hm.S[g.n_fft - 1] - hm.S[0]) / (g.n_fft - 1) : 0.0;
-      if ((int64_t)J * cm.nb1 > INT32_MAX) return GFH_ERR_SIZE;
-      fblk_off[m] = fblk_total;
-      fblk_total += (size_t)J * cm.nb1;
-      fblk_entries = std::max(fblk_entries, J * cm.nb1);
-      n_lists = std::max(n_lists, g.list + 1);
-    }
+    find_analysis_columns(hm);
     // columns of each f0 tile: analysis columns only; f0 falls with the column, so each range is
     // contiguous
     std::vector<int64_t> cmin(coarse_x, INT64_MAX), cmax(coarse_x, -1);
@@ -760,7 +914,7 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
           // 16-byte aligned column range (vector stores): neighbouring tiles may share <= 3 columns
           const int64_t c_lo = cmin[xt] & ~int64_t(3);
           const int64_t c_hi = std::min<int64_t>(g.ld_x0, (cmax[xt] + 4) & ~int64_t(3));
-          map_tiles(g, hm, m, p->cfg, r0, r1, c_lo, c_hi, fine, max_bands);
+          map_tiles(g, hm, m, tp, r0, r1, c_lo, c_hi, fine);
         }
         const int cnt = (int)(fine.size() - before);
         max_fine = std::max(max_fine, cnt);
@@ -770,10 +924,8 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
     // group nct: the whole map, as gfh_plan_execute tiles it
     first.push_back((int32_t)fine.size());
     const size_t before = fine.size();
-    map_tiles(g, hm, m, p->cfg, 0, g.n_k, 0, g.ld_x0, fine, max_bands);
+    map_tiles(g, hm, m, tp, 0, g.n_k, 0, g.ld_x0, fine);
     const size_t whole = fine.size() - before;
-    for (size_t q = map_begin; q < fine.size(); ++q)
-      fine[q].sub = tile_walks_sub_ranges(g, hm, fine[q], p->cfg.rows, sub_cap) ? 1 : 0;
     std::sort(sizes.begin(), sizes.end(), std::greater<int>());
     size_t top = 0;
     for (int i = 0; i < max_sel && i < (int)sizes.size(); ++i) top += sizes[i];
@@ -781,55 +933,35 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
   }
   first.push_back((int32_t)fine.size());
   if (fine.size() > (size_t)INT32_MAX || worst > (size_t)INT32_MAX) return GFH_ERR_SIZE;
-  if (max_bands > p->max_tile_bands + 8) {   // the sub-range room assumed the plan's band keys
-    for (TileDev& t : fine) t.sub = 0;
-  }
-  const size_t smem = (size_t)p->cfg.rows * (p->cfg.cols + 2) * 4 + 32 * 4 +
-                      (p->select ? (size_t)max_bands * 8 : 0) + (size_t)sub_cap * 8 + 16;
-  if (smem > kHoughSmemLimit) return GFH_ERR_SIZE;
-
+  const size_t cells_list = tile_bytes(fine, 0, &max_bands);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   const size_t o_fine = take(sizeof(TileDev) * std::max<size_t>(fine.size(), 1));
   const size_t o_first = take(sizeof(int32_t) * first.size());
   const size_t o_sel = take(sizeof(TileDev) * std::max<size_t>(worst, 1));
-  const size_t o_cnt = take(2 * sizeof(int));
-  const size_t o_cms = take(sizeof(CoarseMapDev) * p->n_maps);
-  const size_t o_uns = take(sizeof(int) * std::max(n_lists, 1));
-  const size_t o_fblk = take(sizeof(int32_t) * std::max<size_t>(fblk_total, 1));
   GFH_CUDA_TRY(cudaSetDevice(p->ctx->device));
   if (p->ctx->stream) GFH_CUDA_TRY(cudaStreamSynchronize(p->ctx->stream));
   void* buf = nullptr;
   if (cudaMalloc(&buf, off) != cudaSuccess) return GFH_ERR_NOMEM;
   char* base = (char*)buf;
-  for (int m = 0; m < p->n_maps; ++m) cms[m].fblk = (int32_t*)(base + o_fblk) + fblk_off[m];
   cudaError_t e = cudaSuccess;
   if (!fine.empty())
     e = cudaMemcpy(base + o_fine, fine.data(), sizeof(TileDev) * fine.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(base + o_first, first.data(), sizeof(int32_t) * first.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(base + o_cms, cms.data(), sizeof(CoarseMapDev) * cms.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) { cudaFree(buf); return GFH_ERR_CUDA; }
   if (p->d_coarse_buf) cudaFree(p->d_coarse_buf);
   p->d_coarse_buf = buf;
   p->d_fine = (TileDev*)(base + o_fine);
   p->d_coarse_first = (int32_t*)(base + o_first);
   p->d_sel_tiles = (TileDev*)(base + o_sel);
-  p->d_sel_count = (int*)(base + o_cnt);
   p->sel_cap = (int)std::max<size_t>(worst, 1);
   p->coarse_k = coarse_k;
   p->coarse_x = coarse_x;
   p->max_sel = max_sel;
   p->max_fine = max_fine;
   p->max_tile_bands = max_bands;
-  p->d_cmaps = (CoarseMapDev*)(base + o_cms);
-  p->d_fft_unsorted = (int*)(base + o_uns);
-  p->n_list_flags = std::max(n_lists, 1);
-  p->sub_cap = sub_cap;
-  p->fblk_entries = fblk_entries;
-  p->n_sub_tiles = 0;
-  for (const TileDev& t : fine) p->n_sub_tiles += t.sub;
+  p->cells_list = cells_list;
   return GFH_OK;
 }
 
@@ -970,11 +1102,6 @@ extern "C" int gfh_plan_autotune(gfh_plan* p, const gfh_peaks* peaks, int32_t re
         rc = try_shape(gfh_tile_config{r, c, t, 0});
         if (rc) return rc;
       }
-  // the fastest shape with the other drawing form
-  gfh_tile_config other = best;
-  other.form = 1 - best.form;
-  rc = try_shape(other);
-  if (rc) return rc;
   rc = reshape_plan(p, best);
   if (rc) return rc;
   {

@@ -3,18 +3,25 @@
 // Each peak (FFT i, bin j) is the set of lines x0 = x - (n-1) k t_i for x across its bin
 // (Eq. transform, Sec. IV).  On k row r it covers the x0 columns that the half-open fixed-point
 // interval [U[j+1] - B_i - r S_i, U[j] - B_i - r S_i) overlaps.  The map is built per tile of
-// R rows x C columns in shared memory by differential counting: +1 at the first covered column,
-// -1 after the last (warp-level shared-memory atomics; intervals that start left of the tile go to
-// a per-thread register carry instead of contending on column 0), then a running sum along x0 and
-// one vectorised streaming store of every map cell.  Candidate selection (Sec. IV: highest count
+// k rows x x0 columns in shared memory by differential counting: +1 at the first covered column,
+// -1 after the last on the tile's first row, then one event for every column an edge moves
+// (shared-memory increments; intervals that start left of the tile go to a per-thread register carry
+// instead of contending on column 0), then running sums and one vectorised streaming store of every
+// map cell.  Candidate selection (Sec. IV: highest count
 // per f0 band, critical ratio from the map's mean and deviation) is fused into the store pass.
-#include <cstdio>
+#include <algorithm>
+#include <type_traits>
 
 #include "gfh_internal.h"
 
 namespace {
 
 constexpr int kLane = 32;
+constexpr int kListUnsorted = 1, kListFftUnsorted = 2;   // bits of a peak list's order state
+constexpr int kFewBands = 4;     // a tile of at most this many bands looks for its best cells only if they can win
+template <int NT> constexpr int kSumBytes = NT / kLane * 16;   // two sums per warp
+constexpr int kRowBits = 57;     // fraction bits of an event's row
+constexpr int kEventUnroll = kHoughSpare;   // events of each edge per turn of the drawing loop
 
 __device__ __forceinline__ int warp_sum(int v) {
 #pragma unroll
@@ -45,231 +52,212 @@ __device__ __forceinline__ unsigned long long cand_key(int count, uint32_t lin) 
 
 // ---- per-execute preparation --------------------------------------------------------------------
 
-// Flags peak lists whose bins are not sorted ascending.  fft_unsorted (may be null; n_flags
-// entries, zeroed before): 1 for a list in which some bin's peaks are not in FFT order (the
-// coarse-tile search then walks that list's peaks in full).
+// Order of each peak list (state[l], l < n_states, zeroed before): kListUnsorted when its bins are not ascending
+// (also flagged; such a list is not drawn), kListFftUnsorted when some bin's peaks are not in FFT
+// order (the tiles then read all peaks of their bins).
 __global__ void k_check_sorted(const uint32_t* __restrict__ bins, const uint32_t* __restrict__ fft,
                                const int64_t* __restrict__ off, unsigned int* flag,
-                               int* __restrict__ fft_unsorted, int n_flags) {
+                               int* __restrict__ state, int n_states) {
   const int l = blockIdx.y;
   const int64_t b = off[l], e = off[l + 1];
-  const bool check_fft = fft_unsorted && l < n_flags;
-  for (int64_t p = b + 1 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < e;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t j1 = bins[p], j0 = bins[p - 1];
-    if (j1 < j0) atomicOr(flag, GFH_FLAG_UNSORTED);
-    else if (check_fft && j1 == j0 && fft[p] < fft[p - 1]) fft_unsorted[l] = 1;
+  int bad = 0;
+  // four independent pairs per turn
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t p0 = b + 1 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p0 < e; p0 += 4 * step) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t p = p0 + q * step;
+      if (p >= e) continue;
+      const uint32_t j1 = bins[p], j0 = bins[p - 1], f1 = fft[p], f0 = fft[p - 1];
+      if (j1 < j0) bad |= kListUnsorted;
+      else if (j1 == j0 && f1 < f0) bad |= kListFftUnsorted;
+    }
   }
+  if (bad & kListUnsorted) atomicOr(flag, GFH_FLAG_UNSORTED);
+  if (bad && l < n_states) atomicOr(&state[l], bad);
 }
 
-// Per map (blockIdx.y), bin jl and FFT block b: the offset in the bin's peaks of its first peak
-// with FFT index >= kFftBlock b (the bin's count when none), by bisection over the bin's FFT
-// indices.  Meaningful for lists whose bins hold their peaks in FFT order.
-__global__ void k_fft_blocks(const MapDev* __restrict__ maps, const CoarseMapDev* __restrict__ cmaps,
-                             const uint32_t* __restrict__ fft) {
-  const MapDev& md = maps[blockIdx.y];
-  const CoarseMapDev& cm = cmaps[blockIdx.y];
-  const int J = md.bin_hi - md.bin_lo + 1;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= J * cm.nb1) return;
-  const int jl = e / cm.nb1, b = e - jl * cm.nb1;
-  const int64_t s = md.csr[jl], t = md.csr[jl + 1];
-  const uint32_t key = (uint32_t)b * (uint32_t)kFftBlock;
-  int64_t lo = s, hi = t;
-  while (lo < hi) {
-    const int64_t mid = lo + ((hi - lo) >> 1);
-    if (__ldg(fft + mid) < key) lo = mid + 1; else hi = mid;
+// Index of the peak lists, one warp per (list, bin): csr = the bin's first peak (by a 32-way search
+// of the list, five bits a step), and per block of 2^shift FFTs the offset inside the bin of its
+// first peak with FFT index in that block or later (meaningful where the bin is in FFT order).
+__global__ void k_index(const ListDev* __restrict__ lists, const int32_t* __restrict__ entry_list,
+                        int n_entries, const uint32_t* __restrict__ bins,
+                        const uint32_t* __restrict__ fft, const int64_t* __restrict__ off) {
+  const int e = blockIdx.x * (blockDim.x / kLane) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (e >= n_entries) return;
+  const ListDev& ld = lists[entry_list[e]];
+  const int jl = e - ld.entry0;
+  // first peaks with bin >= key and >= key + 1
+  int64_t lo[2], hi[2];
+#pragma unroll
+  for (int w = 0; w < 2; ++w) { lo[w] = off[ld.list]; hi[w] = off[ld.list + 1]; }
+  while (lo[0] < hi[0] || lo[1] < hi[1]) {
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      const int64_t n = hi[w] - lo[w];
+      if (n <= 0) continue;
+      const uint32_t key = (uint32_t)(ld.bin_lo + jl + w);
+      const int64_t step = n / kLane + 1;          // probes lo + step (lane + 1) - 1
+      const int64_t at = lo[w] + step * (lane + 1) - 1;
+      const bool less = at < hi[w] && bins[at] < key;
+      const int c = __popc(__ballot_sync(0xffffffffu, less));
+      const int64_t l = lo[w] + step * c;
+      hi[w] = min(hi[w], l + step - 1);
+      lo[w] = l;
+    }
   }
-  cm.fblk[e] = (int32_t)(lo - s);
-}
-
-// csr[e] = index of the first peak of the map's list whose bin is >= bin_lo + e.
-__global__ void k_csr(const MapDev* __restrict__ maps, const int32_t* __restrict__ entry_map,
-                      int n_entries, const uint32_t* __restrict__ bins,
-                      const int64_t* __restrict__ off) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n_entries) return;
-  const MapDev& md = maps[entry_map[q]];
-  const int e = q - md.csr_base;
-  const uint32_t key = (uint32_t)(md.bin_lo + e);
-  int64_t lo = off[md.list], hi = off[md.list + 1];
-  while (lo < hi) {
-    const int64_t mid = lo + ((hi - lo) >> 1);
-    if (bins[mid] < key) lo = mid + 1; else hi = mid;
+  if (lane == 0) {
+    ld.csr[jl] = lo[0];
+    if (jl == ld.n_bins - 1) ld.csr[jl + 1] = lo[1];
   }
-  md.csr[e] = lo;
+  const int n = (int)(lo[1] - lo[0]);
+  for (int b = lane; b < ld.nb1; b += kLane) {
+    const uint32_t key = (uint32_t)b << ld.shift;
+    int l = 0, h = b + 1 < ld.nb1 ? n : 0;
+    while (l < h) {
+      const int mid = (l + h) >> 1;
+      if (__ldg(fft + lo[0] + mid) < key) l = mid + 1; else h = mid;
+    }
+    ld.blk[(int64_t)jl * ld.nb1 + b] = b + 1 < ld.nb1 ? l : n;
+  }
 }
 
 __global__ void k_set_offsets(int64_t* off, int64_t n) {
   if (threadIdx.x == 0) { off[0] = 0; off[1] = n; }
 }
 
-// Table rows of peak (f, bin): the FFT's base and shift per row, the bin's fixed-point edges.
-// Returns false (and flags the input) for an out-of-range FFT index or a bin outside the map band,
-// which only an unsorted peak list can put in a tile's range; the rows are then not read.
-__device__ __forceinline__ bool peak_rows(const longlong2* __restrict__ BS,
-                                          const longlong2* __restrict__ UP, int bin_lo, uint32_t f,
-                                          int bin, uint32_t nfft, unsigned jmax,
-                                          unsigned int* flag, longlong2& bs, longlong2& up) {
-  const unsigned jl = (unsigned)(bin - bin_lo);
-  if (f >= nfft) { atomicOr(flag, GFH_FLAG_FFT_RANGE); return false; }
-  if (jl > jmax) { atomicOr(flag, GFH_FLAG_UNSORTED); return false; }
-  bs = __ldg(BS + f);
-  up = __ldg(UP + jl);
-  return true;
+// (f D) / 2^32 rounded up: the time, in rows of 2^-kRowBits, at which an edge whose position has the
+// fraction f (2^-32 columns) above a column boundary reaches that boundary.
+__device__ __forceinline__ uint64_t first_crossing(uint32_t f, uint64_t D) {
+  const uint64_t lo = (uint64_t)f * (uint32_t)D + 0xffffffffull;
+  return (uint64_t)f * (uint32_t)(D >> 32) + (lo >> 32);
 }
 
-// Interval of a peak on the tile's first row from its table rows: [A, B1 + 1) in 2^-32 columns,
-// and its per-row shift S.
-__device__ __forceinline__ void peak_interval(int row0, const longlong2 bs, const longlong2 up,
-                                              int64_t& A, int64_t& B1, int64_t& S) {
-  S = bs.y;
-  const int64_t base = bs.x + (int64_t)row0 * S;
-  A = up.x - base;        // interval start (upper-f edge)
-  B1 = up.y - base - 1;   // interval end - 1 (lower-f edge)
+// Adds 1 to the shared word at byte address p.  A conditional increment with no upper bound: the
+// hardware counts the lanes of a warp that hit one word at the full rate, as for atomicAdd(p, 1),
+// while an atomicAdd(p, -1) serialises them (33 cycles a warp instruction with all lanes on one
+// word, against 1.1).
+__device__ __forceinline__ void inc_shared(uint32_t p) {
+  asm volatile("red.shared.inc.u32 [%0], 0xffffffff;" ::"r"(p) : "memory");
 }
 
-
-// Whether the interval of a peak ([a, b1 + 1) on the tile's first row, shifted left by s >= 0 per
-// row: t_first >= 0 and dk > 0 make every S_i non-negative) meets columns c0 .. ub on any of the
-// R rows: its right edge is highest on the first row and its left edge lowest on the last.  A
-// tile's bin range holds every bin that some FFT can bring into the tile at some row, so on a tall
-// map many of the peaks read lie outside it on all R rows; they draw nothing and are skipped whole.
-template <int R>
-__device__ __forceinline__ bool meets_tile(int64_t a, int64_t b1, int64_t s, int c0, int ub) {
-  return (b1 >> GFH_FRAC_BITS) >= (int64_t)c0 &&
-         ((a - (int64_t)(R - 1) * s) >> GFH_FRAC_BITS) <= (int64_t)ub;
+// One event: adds 1 at row v / 2^kRowBits of the column Q before the one p points at; with LIMIT only
+// if n > Q, else to one of the warp's spare words.  (A predicated increment compiles to a branch
+// around it, with its reconvergence three instructions more per event; lanes that share the spare
+// word cost nothing.)
+template <int Q, bool LIMIT>
+__device__ __forceinline__ void event(uint64_t v, uint32_t p, int n, uint32_t row_bytes,
+                                      uint32_t spare) {
+  uint32_t at = (uint32_t)(v >> kRowBits) * row_bytes + p;
+  if (LIMIT) at = n > Q ? at : spare;
+  asm volatile("red.shared.inc.u32 [%0 + %1], 0xffffffff;" ::"r"(at),
+               "n"(-4 * Q)
+               : "memory");
 }
 
-// Largest i in [-1, n) with shift B_i + r S_i <= x on row r; with k_min >= 0 the shift does not
-// fall as i grows (t_i grows, dk > 0).  The guess comes from the straight line through the
-// table's first and last rows (B_i and S_i are floors of linear functions of t_i, so it is off by
-// far less than one FFT); the table confirms it with two loads issued together, and a bisection
-// over the table settles a guess it does not confirm.
-__device__ __forceinline__ int last_shift_at_most(const longlong2* __restrict__ BS, int n,
-                                                  int64_t r, int64_t x, int64_t base0,
-                                                  double inv_slope) {
-  int i;
-  if (inv_slope > 0.0) {
-    const double e = floor((double)(x - base0) * inv_slope);
-    i = e < -1.0 ? -1 : (e > (double)(n - 1) ? n - 1 : (int)e);
-  } else {
-    i = x >= base0 ? n - 1 : -1;        // every row of the table holds the same shift
+// kEventUnroll events of the left and of the right edge.
+template <int Q, bool LIMIT>
+__device__ __forceinline__ void events(uint64_t& v1, uint64_t& v2, uint64_t D, uint32_t p1,
+                                       uint32_t p2, int n1, int n2, uint32_t row_bytes,
+                                       uint32_t spare) {
+  if constexpr (Q < kEventUnroll) {
+    event<Q, LIMIT>(v1, p1, n1, row_bytes, spare);
+    event<Q, LIMIT>(v2, p2, n2, row_bytes, spare);
+    v1 += D;
+    v2 += D;
+    events<Q + 1, LIMIT>(v1, v2, D, p1, p2, n1, n2, row_bytes, spare);
   }
-  const longlong2 a = __ldg(BS + max(i, 0));
-  const longlong2 b = __ldg(BS + min(i + 1, n - 1));
-  if ((i < 0 || a.x + r * a.y <= x) && (i + 1 >= n || b.x + r * b.y > x)) return i;
-  int lo = 0, hi = n;                   // count of the FFTs with shift <= x
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    const longlong2 bs = __ldg(BS + mid);
-    if (bs.x + r * bs.y <= x) lo = mid + 1; else hi = mid;
-  }
-  return lo - 1;
 }
 
-// Events of one peak on the R rows of a tile (layout described at k_hough below).  The interval
-// on row 0 is [a, b1 + 1) in 2^-32 columns and moves left by s per row.  G0 + m is column m of row
-// 0 in absolute column numbering (the tile's first column is c0); ub = min(last column of the
-// tile, last column of the map).
-// A peak that moves less than a column per row, starts at least R - 1 columns right of the tile's
-// first column and ends before the tile's last column and inside the map stays clear of every
-// edge on all R rows (its left edge is lowest on the last row, its right edge highest on row 0):
-// no clamp, no carry, and on rows r > 0 a column is entered where the left edge moved and left
-// where the right edge moved.
-template <int R>
-__device__ __forceinline__ bool peak_interior(int64_t a, int64_t b1, int64_t s, int c0, int c1m1,
-                                              int ub) {
-  constexpr int64_t kOne = int64_t(1) << GFH_FRAC_BITS;
-  const int lo = (int)(a >> GFH_FRAC_BITS), hr = (int)(b1 >> GFH_FRAC_BITS);
-  return (s < kOne) & (lo >= c0 + (R - 1)) & (hr <= ub) & (hr < c1m1) & (a <= b1);
-}
-
-// interior: draw in the interior form (the caller has checked peak_interior for this peak); the
-// edge-following form below draws every peak, interior ones with the same events.
-template <int R>
-__device__ __forceinline__ void draw_peak(int* G0, int lds, int64_t a, int64_t b1, int64_t s,
-                                          int c0, int c1m1, int ub, int& carry, bool interior) {
-  constexpr int64_t kOne = int64_t(1) << GFH_FRAC_BITS;
-  int lo = (int)(a >> GFH_FRAC_BITS);
-  const int hr = (int)(b1 >> GFH_FRAC_BITS);    // row-0 last column before any clamp
-  if (interior) {
-    atomicAdd(G0 + lo, 1);
-    atomicAdd(G0 + hr + 1, -1);
-    int o1 = lo, o2 = hr;
-#pragma unroll
-    for (int rr = 1; rr < R; ++rr) {
-      a -= s;
-      b1 -= s;
-      const int n1 = (int)(a >> GFH_FRAC_BITS), n2 = (int)(b1 >> GFH_FRAC_BITS);
-      int* const Gr = G0 + rr * lds;
-      if (n1 < o1) atomicAdd(Gr + n1, 1);
-      if (n2 < o2) atomicAdd(Gr + o2, -1);
-      o1 = n1;
-      o2 = n2;
-    }
-    return;
+// Draws one peak of each lane on the nr rows of a tile (layout described at hough_tile below); all
+// 32 lanes call it together, `ok` where the lane has a peak.  On row 0 the peak's interval is
+// [a, b1 + 1) in 2^-32 columns from the tile's first column, and it moves left by s >= 0 per row
+// (t_first >= 0 and dk > 0 make every S_i non-negative).  ge, gl: shared addresses of the entered
+// and the left columns' counts.
+//
+// The rows after the first are drawn edge event by edge event and not row by row.  An edge at
+// position p on row 0, f = frac(p), crosses its (e+1)-th column boundary (e = 0, 1, ...) at the
+// first row r with r s > f + e 2^32, so r = floor(x_e) + 1 with x_e = (f + e 2^32) / s.  x_e is kept
+// in rows of 2^-57 and stepped by D = ceil(2^89 / s), the rows per column (a table entry per FFT):
+// every rounding is upwards and below 130 units of 2^-57 in all, while an x_e that is no integer
+// lies at least 1/s >= 2^-33 below the next one, so floor() is exact.  The left edge enters a
+// column at its event (one lower each event), the right edge leaves one.
+// Lanes of a warp hold neighbouring FFTs of one bin, whose s, and so whose event counts, are nearly
+// alike: the loop runs to the warp's largest count.
+// D = 0 marks s <= 2^25 (D would not fit): at most one crossing in the tile's rows (at most 128),
+// placed by an integer division.
+__device__ __forceinline__ void draw_peaks(uint32_t ge, uint32_t gl, uint32_t row_bytes,
+                                           uint32_t spare, int nr, int C, int ub, bool ok, int64_t a, int64_t b1, int64_t s,
+                                           uint64_t D, int& carry) {
+  const int64_t sr = (int64_t)((uint64_t)(uint32_t)(nr - 1) * (uint64_t)s);
+  int lo = (int)(a >> GFH_FRAC_BITS), hr = (int)(b1 >> GFH_FRAC_BITS);
+  const int lo_n = (int)((a - sr) >> GFH_FRAC_BITS), hr_n = (int)((b1 - sr) >> GFH_FRAC_BITS);
+  // The interval meets the tile on some row: its right edge is highest on the first row, its left
+  // edge lowest on the last.
+  ok = ok && hr >= 0 && lo_n <= ub;
+  if (!__any_sync(0xffffffffu, ok)) return;
+  // row 0 along x0: clamped to the map's last column and to the tile; an interval that starts left
+  // of the tile is a carry into its first column
+  const int o1 = max(lo, 0), o2 = min(hr, ub);
+  const bool on = ok && o1 <= o2;
+  carry += on && lo < 0;
+  inc_shared(on && lo >= 0 ? ge + 4u * (uint32_t)lo : spare);
+  inc_shared(on && o2 < C - 1 ? gl + 4u * (uint32_t)(o2 + 1) : spare);
+  // events of the left and the right edge: columns entered, lo - 1 down to lo_n, and left, hr down to
+  // hr_n + 1; those below 0 are not drawn
+  int n1 = ok ? lo - max(lo_n, 0) : 0;
+  int n2 = ok ? hr - max(hr_n, -1) : 0;
+  if (__any_sync(0xffffffffu, max(n1, n2) > 0) == 0) return;
+  uint64_t v1 = first_crossing((uint32_t)a, D), v2 = first_crossing((uint32_t)b1, D);
+  if (D == 0 && ok) {
+    const uint32_t d = max((uint32_t)s, 1u);
+    v1 = (uint64_t)((uint32_t)a / d) << kRowBits;
+    v2 = (uint64_t)((uint32_t)b1 / d) << kRowBits;
   }
-  // row 0: first / last covered column, clamped to the map's last column and to the tile
-  int hi = min(hr, ub);
-  int o1 = max(lo, c0), o2 = hi;
-  if (o1 <= o2) {
-    if (lo < c0) carry += 1;
-    else atomicAdd(G0 + o1, 1);
-    if (hi < c1m1) atomicAdd(G0 + hi + 1, -1);
+  // columns right of the tile come first: skip their events
+  if (__any_sync(0xffffffffu, ok && hr >= C)) {
+    const int e1 = max(lo - C, 0), e2 = max(hr - (C - 1), 0);
+    v1 += (uint64_t)(uint32_t)e1 * D;
+    v2 += (uint64_t)(uint32_t)e2 * D;
+    lo -= e1;
+    n1 -= e1;
+    hr -= e2;
+    n2 -= e2;
   }
-  // rows 1 .. R-1 (rows past the map's last k row are drawn too: they exist in shared memory
-  // and are never stored).  A shift below one column per row moves each edge by at most one
-  // column per row: the left edge enters column n1 when it moves, the right edge leaves column
-  // o2 when it moves.  Edges are followed unclamped and an event is drawn only inside the tile's
-  // columns: an event right of the map's last column (inside the last tile of a map) lands in a
-  // cell that is never stored and changes no stored cell, because sums run rightwards and down.
-  if (s < kOne) {
-    o1 = lo;
-    o2 = hr;
-#pragma unroll
-    for (int rr = 1; rr < R; ++rr) {
-      a -= s;
-      b1 -= s;
-      const int n1 = (int)(a >> GFH_FRAC_BITS), n2 = (int)(b1 >> GFH_FRAC_BITS);
-      int* const Gr = G0 + rr * lds;
-      if ((n1 < o1) & ((unsigned)(n1 - c0) <= (unsigned)(c1m1 - c0))) atomicAdd(Gr + n1, 1);
-      if ((n2 < o2) & ((unsigned)(o2 - c0) <= (unsigned)(c1m1 - c0))) atomicAdd(Gr + o2, -1);
-      o1 = n1;
-      o2 = n2;
-    }
-  } else {
-    for (int rr = 1; rr < R; ++rr) {
-      a -= s;
-      b1 -= s;
-      lo = (int)(a >> GFH_FRAC_BITS);
-      const int n1 = max(lo, c0), n2 = min((int)(b1 >> GFH_FRAC_BITS), ub);
-      int* const Gr = G0 + rr * lds;
-      const int e2 = min(n2, o1 - 1);
-      for (int m = n1; m <= e2; ++m) atomicAdd(Gr + m, 1);
-      for (int m = max(o1, n2 + 1); m <= o2; ++m) atomicAdd(Gr + m, -1);
-      o1 = n1;
-      o2 = n2;
-    }
+  uint32_t p1 = ge + row_bytes + 4u * (uint32_t)(lo - 1);
+  uint32_t p2 = gl + row_bytes + 4u * (uint32_t)hr;
+  // first the turns in which every lane has all its events, then the rest
+  const int most = __reduce_max_sync(0xffffffffu, max(n1, n2));
+  const int least = __reduce_min_sync(0xffffffffu, min(n1, n2));
+  int e = 0;
+  for (; e + kEventUnroll <= least; e += kEventUnroll) {
+    events<0, false>(v1, v2, D, p1, p2, n1, n2, row_bytes, spare);
+    p1 -= 4 * kEventUnroll;
+    p2 -= 4 * kEventUnroll;
+  }
+  for (; e < most; e += kEventUnroll) {
+    events<0, true>(v1, v2, D, p1, p2, n1 - e, n2 - e, row_bytes, spare);
+    p1 -= 4 * kEventUnroll;
+    p2 -= 4 * kEventUnroll;
   }
 }
 
 // Events of one peak on the R rows of a tile in the x-direction form: every row differenced along
-// x0 (+1 at its first column, -1 after its last), so a row costs two events whatever the shift per
-// row; an interval entering from the left of the tile counts in that row's carry.
+// x0 (entered at its first column, left after its last), so a row costs two events whatever the
+// shift per row; an interval entering from the left of the tile counts in that row's carry.
 template <int R>
-__device__ __forceinline__ void draw_peak_x(int* G0, int lds, int64_t a, int64_t b1, int64_t s,
-                                            int c0, int c1m1, int ub, int (&carry)[R]) {
+__device__ __forceinline__ void draw_peak_x(uint32_t ge, uint32_t gl, uint32_t row_bytes, int64_t a,
+                                            int64_t b1, int64_t s, int C, int ub, int (&carry)[R]) {
 #pragma unroll
   for (int rr = 0; rr < R; ++rr) {
     const int lo = (int)(a >> GFH_FRAC_BITS);
     const int hi = min((int)(b1 >> GFH_FRAC_BITS), ub);
-    const int o1 = max(lo, c0);
-    int* const Gr = G0 + rr * lds;
+    const int o1 = max(lo, 0);
     if (o1 <= hi) {
-      if (lo < c0) carry[rr] += 1;
-      else atomicAdd(Gr + o1, 1);
-      if (hi < c1m1) atomicAdd(Gr + hi + 1, -1);
+      if (lo < 0) carry[rr] += 1;
+      else inc_shared(ge + rr * row_bytes + 4u * (uint32_t)o1);
+      if (hi < C - 1) inc_shared(gl + rr * row_bytes + 4u * (uint32_t)(hi + 1));
     }
     a -= s;
     b1 -= s;
@@ -278,373 +266,549 @@ __device__ __forceinline__ void draw_peak_x(int* G0, int lds, int64_t a, int64_t
 
 // ---- the accumulation + running sums + select kernel --------------------------------------------
 
-// A tile is R k rows x C columns.  Lane l draws its own peaks on all R rows.
+// A tile that no edge meets: every cell holds the number of intervals that cover the tile.  mine: a
+// warp's share of it (the same in all its lanes).
+template <int NT, bool SELECT>
+__device__ __forceinline__ void fill_tile(const MapDev& md, const TileDev& t, int mine, int* wsum,
+                                          int nb_tile, uint64_t* s_sums) {
+  constexpr int NW = NT / kLane;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __syncthreads();                               // wsum is free
+  if (lane == 0) wsum[warp] = mine;
+  __syncthreads();
+  const int c = warp_sum(lane < NW ? wsum[lane] : 0);
+  const int C = t.ncols, quads = C / 4;
+  int32_t* const out = md.out + (int64_t)t.row0 * md.ld + t.col0;
+  const int real = (int)min((int64_t)C, md.W - t.col0);          // the padding stays 0
+  for (int rr = warp; rr < t.nrows; rr += NW)
+    for (int q = lane; q < quads; q += kLane) {
+      const int m = 4 * q;
+      __stcs(reinterpret_cast<int4*>(out + rr * md.ld + m),
+             make_int4(m < real ? c : 0, m + 1 < real ? c : 0, m + 2 < real ? c : 0, m + 3 < real ? c : 0));
+    }
+  if (!SELECT || nb_tile == 0) return;
+  // each band's lowest cell is its first column on the tile's first row
+  int n = 0;
+  for (int m = tid; m < real; m += NT) {
+    const int b = __ldg(md.col_band + t.col0 + m);
+    if (b < 0) continue;
+    ++n;
+    if (m > 0 && __ldg(md.col_band + t.col0 + m - 1) == b) continue;
+    const unsigned long long now = *reinterpret_cast<volatile unsigned long long*>(&md.keys[b]);
+    if (now == 0 || c >= (int)(now >> 32))
+      atomicMax(&md.keys[b], cand_key(c, (uint32_t)t.row0 * (uint32_t)md.W + (uint32_t)(t.col0 + m)));
+  }
+  n = warp_sum(n);
+  if (lane == 0) {
+    const uint64_t cells = (uint64_t)n * (uint32_t)t.nrows;
+    s_sums[2 * warp] += cells * (uint32_t)c;
+    s_sums[2 * warp + 1] += cells * (uint32_t)c * (uint32_t)c;
+  }
+}
+
+// A tile is some k rows x C columns; each lane draws peaks of its own on all its rows.
 //
-// Shared memory holds G[R][C+2] int32, a mixed differential of the tile:
+// Shared memory holds two counts per cell, G[rows][C + pad] of the columns entered and, after it, of
+// the columns left; their difference is a mixed differential of the tile:
 //   row 0:     along x0 - +1 at the first column an interval covers, -1 after its last, so that
 //              M[0][m] = sum_{m' <= m} G[0][m'];
 //   row r > 0: along k - +1 at each column the interval newly covers on row r, -1 at each column it
 //              covered on row r-1 but no longer does, so that M[r][m] = M[r-1][m] + G[r][m].
+// (Two counts and not one signed one: see inc_shared.)
 // Along k a peak's interval shifts left by S_i < 1 column per row with the default k step, so on
 // most rows it enters no column and leaves none: rows after the first cost about one event per
-// (peak, row) instead of two.  Intervals are clamped to the tile and to the map's last column;
-// an interval entering from the left of the tile on row 0 is a per-thread carry into column c0.
+// (peak, row) instead of two.  An interval entering from the left of the tile on row 0 is a
+// per-thread carry into the first column.
 //
-// Shared memory: G[R][C+2] | tot[32] row-0 chunk sums | skey[bands] candidate keys.
+// Peaks.  The tile reads the bins that some FFT can bring into it on some row.  Over tall maps the
+// FFTs' shifts spread far wider than a bin, so of each bin only the FFTs of one window have an edge
+// in the tile: the window comes from the line that the shifts follow, its peaks from the list's
+// index (k_index), and only those are walked (whole blocks of FFTs, so a few beside them too).
+// Peak lists that are not in FFT order inside a bin read whole bins.  The windows of up to `batch`
+// bins at a time are laid end to end, two pieces per bin: ent[] = {end of the piece in that order,
+// where its peaks lie in the list less its begin}.  Each warp walks one contiguous part, 32 peaks at
+// a time whatever bins they are of.  A tile that no edge meets holds one number and needs no sums.
+//
+// What bounds it: on dense maps (20 sub-band maps of 2000 rows, 226M cells, 8.8e9 peak rows) the
+// events' integer instructions, about 7 per event, and the increments' bank conflicts (2.4 wavefronts
+// each): 4.68 ms against 7.56 ms for the row-by-row form on flat 16 x 3072 tiles.  On sparse maps
+// (11 braking indices, 1.76e9 cells, 1.3 peak rows per cell) the tiles' chain of dependent loads and
+// barriers: 5.63 against 5.67 ms.  Small maps gain from the split tiles: 500 rows x 51,695 columns
+// 129 against 215 us, the 32 rows of a followed-up candidate 26 against 70 us, 12 uneven peakmaps
+// 0.50 against 1.36 ms.
+//
+// Shared memory: tot[32] row-0 chunk sums | spare words | skey[bands] candidate keys | sums per warp
+// | ent[2 batch] | G.
 // XD (maps whose line moves more than two x0 columns per k row): every row differenced along x0
 // and scanned on its own; chunk sums tot[R][32].
-//
-// SUB (the coarse-tile search): a tile flagged `sub` whose list holds each bin's peaks in FFT
-// order walks only, per read bin, the peaks of the FFTs whose interval can meet it.  On a narrow
-// tile over k rows where the FFTs' shifts spread far wider than the tile, most peaks of its bins
-// miss it.  Each bin's window of FFTs comes from the shift table (last_shift_at_most), its peaks
-// from the FFT-block index (whole 64-FFT blocks, so a few peaks outside the window are read and
-// dropped by the meets test).  The bins' start offsets and a prefix sum of their counts take the
-// last 8 sub_cap + 16 bytes of the dynamic shared memory.
-template <int R, int NT, bool SELECT, bool XD = false, int LDS = 0, bool UNIF = false,
-          bool SUB = false>
+template <int R, int NT, bool SELECT, bool XD>
 __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, const TileDev t,
                                            const uint32_t* __restrict__ fft_idx,
-                                           const uint32_t* __restrict__ bins,
-                                           unsigned int* __restrict__ flag, int c_max,
-                                           unsigned char* smem,
-                                           const CoarseMapDev* __restrict__ cmaps = nullptr,
-                                           const int* __restrict__ fft_unsorted = nullptr,
-                                           int sub_cap = 0) {
+                                           const int* __restrict__ list_state,
+                                           unsigned int* __restrict__ flag, unsigned char* smem,
+                                           uint64_t* s_sums, int2* ent, int batch, int* G) {
+  __shared__ int s_best[kFewBands], s_seek[kFewBands];
   constexpr int NW = NT / kLane;
   const MapDev& md = maps[t.map];
   const int C = t.ncols;
-  // row stride: the plan's tile width + 2 when fixed at compile time (row offsets become
-  // immediates), else this tile's
-  const int lds = LDS ? LDS : C + 2;
-  int* G = reinterpret_cast<int*>(smem);
-  int* tot = G + R * (c_max + 2);
-  unsigned long long* skey = reinterpret_cast<unsigned long long*>(tot + (XD ? R : 1) * kLane);
+  const int lds = C + kHoughPad;                 // row stride
+  const int gap = (XD ? R : t.nrows) * lds;      // from the columns entered to the columns left
+  int* tot = reinterpret_cast<int*>(smem);
+  int* wsum = tot;                               // the warps' sums while windows are laid out
+  unsigned long long* skey = reinterpret_cast<unsigned long long*>(tot + ((XD ? R : 1) + kEventUnroll) * kLane);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nb_tile = t.band_hi >= t.band_lo ? t.band_hi - t.band_lo + 1 : 0;
   const int c0 = (int)t.col0;
-  const int c1m1 = c0 + C - 1;                   // last column of the tile
-  const int ub = min(c1m1, (int)md.W - 1);       // ... and of the map
-  const int nbw = t.bin_b - t.bin_a + 1;         // bins read
-  bool use_sub = false;
-  int* sub_pre = nullptr;                        // per read bin: first walk index (then the total)
-  int* sub_st = nullptr;                         // per read bin: its first peak, from the tile's
-  if constexpr (SUB) {
-    use_sub = t.sub != 0 && nbw > 0 && nbw <= sub_cap && fft_unsorted[cmaps[t.map].list] == 0;
-    uint32_t dyn_bytes;
-    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
-    sub_pre = reinterpret_cast<int*>(smem + dyn_bytes - (8u * (uint32_t)sub_cap + 16u));
-    sub_st = sub_pre + sub_cap + 2;
-  }
-
-  for (int i = tid; i < R * lds / 2; i += NT) reinterpret_cast<int2*>(G)[i] = make_int2(0, 0);
-  if (SELECT)
+  const int ub = min(C - 1, (int)(md.W - 1 - t.col0));   // last column inside the map
+  const uint32_t ge = (uint32_t)__cvta_generic_to_shared(G), gl = ge + 4u * (uint32_t)gap;
+  const uint32_t row_bytes = 4u * (uint32_t)lds;
+  const uint32_t spare = (uint32_t)__cvta_generic_to_shared(tot + (XD ? R : 1) * kLane + kEventUnroll * (warp + 1) - 1);
+  if (SELECT) {
     for (int i = tid; i < nb_tile; i += NT) skey[i] = 0ull;
-  if constexpr (SUB) {
-    if (use_sub) {
-      // per read bin: its window of FFTs, then its peaks in those FFTs' blocks
-      const CoarseMapDev& cm = cmaps[t.map];
-      const int64_t pb0 = md.csr[t.bin_a - md.bin_lo];
-      const int64_t r0 = t.row0, r1 = (int64_t)t.row0 + (R - 1);
-      const double sl0 = cm.db + (double)r0 * cm.ds, sl1 = cm.db + (double)r1 * cm.ds;
-      const double inv0 = sl0 > 0.0 ? 1.0 / sl0 : 0.0, inv1 = sl1 > 0.0 ? 1.0 / sl1 : 0.0;
-      for (int q = tid; q < nbw; q += NT) {
-        const int jl = t.bin_a - md.bin_lo + q;
-        const longlong2 up = __ldg(md.UP + jl);
-        // right edge on the first row reaches c0; left edge on the last row stays left of ub + 1
-        const int last = last_shift_at_most(md.BS, md.n_fft, r0,
-                                            up.y - 1 - ((int64_t)c0 << GFH_FRAC_BITS),
-                                            cm.b0 + r0 * cm.s0, inv0);
-        const int first = last_shift_at_most(md.BS, md.n_fft, r1,
-                                             up.x - ((int64_t)(ub + 1) << GFH_FRAC_BITS),
-                                             cm.b0 + r1 * cm.s0, inv1) + 1;
-        int st = 0, cnt = 0;
-        if (first <= last) {
-          const int32_t* fb = cm.fblk + (int64_t)jl * cm.nb1;
-          const int o0 = fb[first / kFftBlock], o1 = fb[last / kFftBlock + 1];
-          st = (int)(md.csr[jl] - pb0) + o0;
-          cnt = o1 - o0;
-        }
-        sub_st[q] = st;
-        sub_pre[q] = cnt;
-      }
-    }
+    if (tid < kFewBands) s_best[tid] = 0;
   }
-  __syncthreads();
-  if constexpr (SUB) {
-    if (use_sub) {
-      // exclusive prefix of the counts (warp 0, 32 consecutive runs), the total after them
-      if (warp == 0) {
-        const int per = (nbw + kLane - 1) / kLane;
-        const int q0 = min(lane * per, nbw), q1 = min(q0 + per, nbw);
-        int sum = 0;
-        for (int q = q0; q < q1; ++q) sum += sub_pre[q];
-        const int incl = warp_incl_scan(sum, lane);
-        int run = incl - sum;
-        for (int q = q0; q < q1; ++q) {
-          const int c = sub_pre[q];
-          sub_pre[q] = run;
-          run += c;
-        }
-        if (lane == kLane - 1) sub_pre[nbw] = incl;
-      }
-      __syncthreads();
-    }
-  }
+  int carry = 0;
+  int carry_x[XD ? R : 1] = {};
+  bool drawn = false;                            // some peak has an edge in the tile
 
   // ---- accumulate
-  if (t.bin_a <= t.bin_b) {
-    const int64_t pb = md.csr[t.bin_a - md.bin_lo];
-    const int64_t pe = md.csr[t.bin_b - md.bin_lo + 1];
-    const uint32_t nfft = (uint32_t)md.n_fft;
-    const unsigned jmax = (unsigned)(md.bin_hi - md.bin_lo);
-    const int bin_lo = md.bin_lo;                // map fields read once, kept in registers
-    const longlong2* const BS = md.BS;
-    const longlong2* const UP = md.UP;
-    int* const G0 = G - c0;                      // rows indexed by absolute column
-    int carry = 0;
-    int carry_x[XD ? R : 1] = {};
-    // Software pipeline over this thread's peaks p, p + NT, ...: the indices are loaded two
-    // peaks ahead and the table rows one peak ahead of the peak being drawn; the next peak's
-    // interval is formed from its rows after the current peak is drawn, so the loads have the
-    // whole drawing to arrive.
+  const int state = list_state[md.list];
+  if (t.bin_a <= t.bin_b && !(state & kListUnsorted)) {
+    const int bin0 = t.bin_a - md.bin_lo, nbw = t.bin_b - t.bin_a + 1;
+    const int64_t pb = md.csr[bin0];
     // this tile's peaks with 32-bit offsets (a range beyond 2^31 - 2^20 peaks raises the capacity
     // flag and is not drawn)
-    const bool fits = pe - pb <= (int64_t)0x7fffffff - (1 << 20);
+    const bool fits = md.csr[bin0 + nbw] - pb <= (int64_t)0x7fffffff - (1 << 20);
     if (!fits && tid == 0) atomicOr(flag, GFH_FLAG_CAPACITY);
     const uint32_t* const fl = fft_idx + pb;
-    const uint32_t* const bl = bins + pb;
-    const int np = fits ? (int)(pe - pb) : 0;
-    // walk n peaks; fetch(i, f, j) gives the FFT and bin of the i-th (i < n)
-    auto walk = [&](int n, auto fetch) {
-      int p = tid;
-      uint32_t f_nx = 0xffffffffu;               // indices of peak p + NT
+    const uint32_t nfft = (uint32_t)md.n_fft;
+    const FftRow* const SD = md.SD;
+    const int64_t* const Bt = md.B;
+    const longlong2* const UP = md.UP + bin0;
+    const bool window = !XD && !(state & kListFftUnsorted);
+    const int64_t r0 = t.row0, r1 = r0 + t.nrows - 1;
+    // The shift of FFT i on row r is the line base + i slope within 2 r + 4 lattice units and the
+    // rounding of float32, so the FFTs whose shift is at most (at least) x are those up to (from)
+    // (x - base) / slope within `slack`, the other way round where k < 0 (n = 0) makes the shift
+    // fall with the FFT; with slope 0 every FFT may meet the tile and none is known to cover it.
+    const int64_t base0 = md.b0 + r0 * md.s0, base1 = md.b0 + r1 * md.s0;
+    const float sl0 = md.db + (float)r0 * md.ds, sl1 = md.db + (float)r1 * md.ds;
+    const float inv0 = sl0 != 0.f ? 1.f / sl0 : 0.f, inv1 = sl1 != 0.f ? 1.f / sl1 : 0.f;
+    const float ffts = (float)md.n_fft;
+    const float slack0 = 2.f + (float)(2 * r0 + 4) * fabsf(inv0) + ffts * 0x1p-20f;
+    const float slack1 = 2.f + (float)(2 * r1 + 4) * fabsf(inv1) + ffts * 0x1p-20f;
+    auto clampf = [&](float x) { return (int)fminf(fmaxf(x, -1.f), ffts); };
+    for (int q0 = 0; q0 < (fits ? nbw : 0); q0 += batch) {
+      const int nq = min(batch, nbw - q0);
+      // per bin (one thread each): its peaks that have an edge in the tile, in one or two pieces
+      int st1 = 0, cnt1 = 0, st2 = 0, cnt2 = 0;
+      if (tid < nq) {
+        const int q = q0 + tid;
+        const int64_t s = md.csr[bin0 + q];
+        st1 = (int)(s - pb);
+        cnt1 = (int)(md.csr[bin0 + q + 1] - s);
+        if (window && cnt1 > 0) {
+          const longlong2 up = __ldg(UP + q);
+          const int n = cnt1;
+          const int32_t* const blk = md.blk + (int64_t)(bin0 + q) * md.nb1;
+          // first peaks of the FFT block that holds FFT i, and of the first block that starts there
+          // or later (i <= 0: 0; i >= n_fft: all)
+          auto from = [&](int i) { return i <= 0 ? 0 : (i >= md.n_fft ? n : __ldg(blk + (i >> md.shift))); };
+          auto to = [&](int i) {
+            return i <= 0 ? 0 : (i >= md.n_fft ? n : __ldg(blk + ((i - 1) >> md.shift) + 1));
+          };
+          auto col = [](int c) { return (int64_t)c << GFH_FRAC_BITS; };
+          if (__ldg(fl + st1 + n - 1) >= nfft) atomicOr(flag, GFH_FLAG_FFT_RANGE);
+          // right edge on the first row reaches the tile (shift0 <= x); left edge on the last row is
+          // not past it (shift1 >= y)
+          const float x = (float)(up.y - col(c0) - base0) * inv0;
+          const float y = (float)(up.x - col(c0 + ub + 1) - base1) * inv1;
+          float lo = -1.f, hi = ffts;
+          if (inv0 > 0.f) hi = x + slack0;
+          if (inv0 < 0.f) lo = x - slack0;
+          if (inv1 > 0.f) lo = fmaxf(lo, y - slack1);
+          if (inv1 < 0.f) hi = fminf(hi, y + slack1);
+          const int o0 = from(clampf(lo)), o1 = max(to(clampf(hi) + 1), o0);
+          st1 += o0;
+          cnt1 = o1 - o0;
+          // a bin wider than the tile: the FFTs c_lo .. c_hi cover the tile on every row (left edge
+          // at or before its first column on the first row, right edge at or past its last on the
+          // last) and are counted without a walk
+          if (((up.y - up.x) >> GFH_FRAC_BITS) >= ub && ub == C - 1 && cnt1 > 0 && inv0 != 0.f && inv1 != 0.f) {
+            const float cx = (float)(up.x - col(c0 + 1) - base0) * inv0;
+            const float cy = (float)(up.y - col(c0 + ub) - base1) * inv1;
+            const float c_lo = fmaxf(inv0 > 0.f ? cx + slack0 : -1.f, inv1 < 0.f ? cy + slack1 : -1.f);
+            const float c_hi = fminf(inv1 > 0.f ? cy - slack1 : ffts, inv0 < 0.f ? cx - slack0 : ffts);
+            const int m1 = max(to(clampf(c_lo) + 1), o0), m2 = min(from(clampf(c_hi)), o1);
+            if (m1 < m2) {
+              carry += m2 - m1;
+              cnt1 = m1 - o0;
+              st2 = st1 - o0 + m2;
+              cnt2 = o1 - m2;
+            }
+          }
+        }
+      }
+      const int cnt = cnt1 + cnt2;
+      const int incl = warp_incl_scan(cnt, lane);
+      __syncthreads();                           // the previous batch is drawn
+      if (lane == kLane - 1) wsum[warp] = incl;
+      __syncthreads();
+      const int ws = lane < NW ? wsum[lane] : 0;
+      const int before = warp_sum(lane < warp ? ws : 0), total = warp_sum(ws);
+      if (total == 0) continue;
+      if (!drawn)
+        for (int i = tid; i < gap / 2; i += NT) reinterpret_cast<int4*>(G)[i] = make_int4(0, 0, 0, 0);
+      drawn = true;
+      if (tid < nq) {
+        const int e0 = before + incl - cnt;
+        ent[2 * tid] = make_int2(e0 + cnt1, st1 - e0);
+        ent[2 * tid + 1] = make_int2(e0 + cnt, st2 - (e0 + cnt1));
+      }
+      __syncthreads();
+      // this warp's part: `units` runs of 32 peaks, split as evenly as they go
+      const int units = (total + kLane - 1) / kLane;
+      const int per = units / NW, rem = units % NW;
+      const int u0 = warp * per + min(warp, rem);
+      int v = u0 * kLane + lane;
+      const int vend = min((u0 + per + (warp < rem ? 1 : 0)) * kLane, total);
+      // the lane's place: piece q ends at q_end, peak v is fl[v + q_off]
+      int q = 0, q_end = 0, q_off = 0;
+      if (v < vend) {
+        int hi = 2 * nq - 1;
+        while (q < hi) {
+          const int mid = (q + hi) >> 1;
+          if (ent[mid].x > v) hi = mid; else q = mid + 1;
+        }
+        q_end = ent[q].x;
+        q_off = ent[q].y;
+      }
+      auto fetch = [&](int x, uint32_t& f, int& j) {
+        while (x >= q_end) {
+          const int2 e = ent[++q];
+          q_end = e.x;
+          q_off = e.y;
+        }
+        f = __ldg(fl + x + q_off);
+        j = q0 + (q >> 1);
+      };
+      // table rows of a peak; false (and the input flagged) for an out-of-range FFT index
+      auto rows = [&](uint32_t f, int j, FftRow& sd, int64_t& B, longlong2& up) -> bool {
+        if (f >= nfft) { atomicOr(flag, GFH_FLAG_FFT_RANGE); return false; }
+        const longlong2 w = __ldg(reinterpret_cast<const longlong2*>(SD + f));
+        sd.S = w.x;
+        sd.D = (uint64_t)w.y;
+        B = Bt ? __ldg(Bt + f) : 0;
+        up = __ldg(UP + j);
+        return true;
+      };
+      // Software pipeline: the FFT indices are loaded two runs of peaks ahead and the table rows one
+      // run ahead of the peaks being drawn; the next peak's interval is formed from its rows after
+      // the current one is drawn, so those loads have the whole drawing to arrive.  The lanes of a
+      // warp stay together, also past the last peak.
+      bool has_nx = false;                       // indices of peak v + 32
+      uint32_t f_nx = 0;
       int j_nx = 0;
-      int64_t a_cu = 0, b_cu = 0, s_cu = 0;      // interval of peak p
-      bool ok_cu = false;
-      if (p < n) {
+      int64_t a = 0, b1 = 0, s = 0;              // interval and shift of peak v
+      uint64_t d = 0;
+      bool ok = false;
+      auto interval = [&](const FftRow& sd, int64_t B, const longlong2& up) {
+        const int64_t base = B + (int64_t)((uint64_t)(uint32_t)t.row0 * (uint64_t)sd.S) +
+                             ((int64_t)c0 << GFH_FRAC_BITS);
+        a = up.x - base;                         // columns from the tile's first: [a, b1 + 1)
+        b1 = up.y - base;
+        s = sd.S;
+        d = sd.D;
+      };
+      if (v < vend) {
         uint32_t f;
         int j;
-        fetch(p, f, j);
-        longlong2 bs, up;
-        ok_cu = peak_rows(BS, UP, bin_lo, f, j, nfft, jmax, flag, bs, up);
-        if (ok_cu) peak_interval(t.row0, bs, up, a_cu, b_cu, s_cu);
+        fetch(v, f, j);
+        FftRow sd{};
+        int64_t B = 0;
+        longlong2 up = make_longlong2(0, 0);
+        ok = rows(f, j, sd, B, up);
+        interval(sd, B, up);
       }
-      if (p + NT < n) fetch(p + NT, f_nx, j_nx);
-      for (; p < n; p += NT) {
-        uint32_t f_nn = 0xffffffffu;             // indices of peak p + 2 NT
-        int j_nn = 0;
-        if (p + 2 * NT < n) fetch(p + 2 * NT, f_nn, j_nn);
-        longlong2 bs_nx = make_longlong2(0, 0), up_nx = make_longlong2(0, 0);
-        const bool ok_nx = f_nx != 0xffffffffu &&
-                           peak_rows(BS, UP, bin_lo, f_nx, j_nx, nfft, jmax, flag, bs_nx, up_nx);
-        const bool draw = ok_cu && meets_tile<R>(a_cu, b_cu, s_cu, c0, ub);
+      if (v + kLane < vend) { fetch(v + kLane, f_nx, j_nx); has_nx = true; }
+      for (; v - lane < vend; v += kLane) {
+        FftRow sd{};
+        int64_t B = 0;
+        longlong2 up = make_longlong2(0, 0);
+        const bool ok_nx = has_nx && rows(f_nx, j_nx, sd, B, up);
+        has_nx = v + 2 * kLane < vend;
+        if (has_nx) fetch(v + 2 * kLane, f_nx, j_nx);
         if constexpr (XD) {
-          if (draw) draw_peak_x<R>(G0, lds, a_cu, b_cu, s_cu, c0, c1m1, ub, carry_x);
-        } else if constexpr (UNIF) {
-          // one drawing form per warp: the interior form when every drawing lane's peak is
-          // interior, else the edge-following form for all, so that a warp never runs both
-          const bool interior = __all_sync(__activemask(),
-                                           !draw || peak_interior<R>(a_cu, b_cu, s_cu, c0, c1m1, ub));
-          if (draw) draw_peak<R>(G0, lds, a_cu, b_cu, s_cu, c0, c1m1, ub, carry, interior);
+          if (ok) draw_peak_x<R>(ge, gl, row_bytes, a, b1, s, C, ub, carry_x);
         } else {
-          if (draw)
-            draw_peak<R>(G0, lds, a_cu, b_cu, s_cu, c0, c1m1, ub, carry,
-                         peak_interior<R>(a_cu, b_cu, s_cu, c0, c1m1, ub));
+          draw_peaks(ge, gl, row_bytes, spare, t.nrows, C, ub, ok, a, b1, s, d, carry);
         }
-        peak_interval(t.row0, bs_nx, up_nx, a_cu, b_cu, s_cu);
-        ok_cu = ok_nx;
-        f_nx = f_nn; j_nx = j_nn;
+        interval(sd, B, up);
+        ok = ok_nx;
       }
-    };
-    if (SUB && use_sub) {
-      // walk index v: its bin q is the last with sub_pre[q] <= v (empty bins share the prefix of
-      // the next), its peak the bin's first peak + v - sub_pre[q]
-      const int n_sub = fits ? sub_pre[nbw] : 0;
-      walk(n_sub, [&](int v, uint32_t& f, int& j) {
-        int lo = 0, hi = nbw - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (sub_pre[mid] <= v) lo = mid; else hi = mid - 1;
-        }
-        f = __ldg(fl + sub_st[lo] + (v - sub_pre[lo]));
-        j = t.bin_a + lo;
-      });
-    } else {
-      walk(np, [&](int p, uint32_t& f, int& j) {
-        f = __ldg(fl + p);
-        j = (int)__ldg(bl + p);
-      });
     }
-    if constexpr (XD) {
+  }
+  if (!drawn) {
+    fill_tile<NT, SELECT>(md, t, warp_sum(carry), wsum, nb_tile, s_sums);
+    return;
+  }
+  if constexpr (XD) {
 #pragma unroll
-      for (int rr = 0; rr < (XD ? R : 1); ++rr) {
-        const int v = warp_sum(carry_x[rr]);
-        if (lane == 0 && v) atomicAdd(G + rr * lds, v);
-      }
-    } else {
-      const int v = warp_sum(carry);
-      if (lane == 0 && v) atomicAdd(G, v);
+    for (int rr = 0; rr < R; ++rr) {
+      const int v = warp_sum(carry_x[rr]);
+      if (lane == 0 && v) atomicAdd(G + rr * lds, v);
     }
+  } else {
+    const int v = warp_sum(carry);
+    if (lane == 0 && v) atomicAdd(G, v);
   }
   __syncthreads();
 
-  // ---- row-0 chunk sums: chunk = 128 columns (32 lanes x 4); warp w owns chunks w, w+NW, ...
+  // ---- running sums along x0, in place: row 0 only, or every row (XD).  A chunk is 128 columns
+  // (32 lanes x 4).
   const int nch = (C + 127) / 128;
-  const int nsum = XD ? t.nrows * nch : nch;     // (row, chunk) sums: row 0 only, or every row
+  const int nsum = XD ? t.nrows * nch : nch;
+  auto load4 = [&](const int* g) {               // entered - left
+    const int4 e = *reinterpret_cast<const int4*>(g), l = *reinterpret_cast<const int4*>(g + gap);
+    return make_int4(e.x - l.x, e.y - l.y, e.z - l.z, e.w - l.w);
+  };
   for (int idx = warp; idx < nsum; idx += NW) {
     const int rr = idx / nch, ch = idx - rr * nch;
     const int col = ch * 128 + lane * 4;
     int s = 0;
     if (col < C) {
-      const int2 u = *reinterpret_cast<const int2*>(&G[rr * lds + col]);
-      const int2 w = *reinterpret_cast<const int2*>(&G[rr * lds + col + 2]);
-      s = u.x + u.y + w.x + w.y;
+      const int4 g = load4(&G[rr * lds + col]);
+      s = g.x + g.y + g.z + g.w;
     }
     s = warp_sum(s);
     if (lane == 0) tot[rr * kLane + ch] = s;
   }
   __syncthreads();
+  for (int idx = warp; idx < nsum; idx += NW) {
+    const int rr = idx / nch, ch = idx - rr * nch;
+    const int col = ch * 128 + lane * 4;
+    const int before = warp_sum((lane < ch) ? tot[rr * kLane + lane] : 0);
+    int4 g = make_int4(0, 0, 0, 0);
+    if (col < C) g = load4(&G[rr * lds + col]);
+    g.y += g.x; g.z += g.y; g.w += g.z;
+    const int add = before + warp_incl_scan(g.w, lane) - g.w;
+    if (col < C) {
+      *reinterpret_cast<int4*>(&G[rr * lds + col]) = make_int4(g.x + add, g.y + add, g.z + add, g.w + add);
+      *reinterpret_cast<int4*>(&G[rr * lds + col + gap]) = make_int4(0, 0, 0, 0);
+    }
+  }
+  __syncthreads();
 
-  // ---- row 0: running sum along x0; rows r > 0: running sum along k; store; candidates
-  long long s1 = 0, s2 = 0;
+  // ---- running sums along k; store; candidates.  A tile of few chunks is split into segments of
+  // rows so that every warp has a share: first the column sums of all segments but the last (kept
+  // where the windows were), then each (chunk, segment) from the sums before it.
+  const int nseg = XD ? min(max(NW / nch, 1), t.nrows)
+                      : max(1, min(min(NW / nch, t.nrows / 4), 1 + (int)(batch * 16) / (4 * C)));
+  const int seg_rows = (t.nrows + nseg - 1) / nseg;
+  int* const seg_sum = reinterpret_cast<int*>(ent);
+  if (!XD && nseg > 1) {
+    for (int u = warp; u < nch * (nseg - 1); u += NW) {
+      const int sg = u / nch, col = (u - sg * nch) * 128 + lane * 4;
+      if (col < C) {
+        int4 v = make_int4(0, 0, 0, 0);
+        for (int rr = sg * seg_rows; rr < min((sg + 1) * seg_rows, t.nrows); ++rr) {
+          const int4 g = load4(&G[rr * lds + col]);
+          v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w;
+        }
+        *reinterpret_cast<int4*>(seg_sum + sg * C + col) = v;
+      }
+    }
+    __syncthreads();
+  }
+  // Candidates.  A tile with columns of at most kFewBands bands (wide bins) first takes each band's
+  // largest count only, and looks for its cell in a second walk over the sums if it can win over the
+  // map's best so far; with many bands every column tracks its best cell in the one walk.
+  const bool few = nb_tile <= kFewBands;
+  uint64_t s1 = 0, s2 = 0;
   const uint32_t W32 = (uint32_t)md.W;
   // map fields of the store pass read once (a global store could otherwise force a reload)
   int32_t* const out = md.out + t.col0;
   const int64_t ld_out = md.ld;
   const int32_t* const col_band = md.col_band + t.col0;
-  for (int ch = warp; ch < nch; ch += NW) {
-    const int col = ch * 128 + lane * 4;
-    const bool in = col < C;
-    int band[4] = {-1, -1, -1, -1};
-    // per column: best count over the rows so far and its row (strictly greater, so the first
-    // row reaching the best count wins: the lowest cell index)
-    int bc[4] = {-1, -1, -1, -1}, br[4] = {0, 0, 0, 0};
-    if (SELECT && in) {
-      const int4 bv = __ldg(reinterpret_cast<const int4*>(col_band + col));
-      band[0] = bv.x; band[1] = bv.y; band[2] = bv.z; band[3] = bv.w;
-    }
-    const int cin = XD ? 0 : warp_sum((lane < ch) ? tot[lane] : 0);
-    int4 v = make_int4(0, 0, 0, 0);
-    for (int rr = 0; rr < t.nrows; ++rr) {
-      int4 g = make_int4(0, 0, 0, 0);
-      if (in) {
-        const int2 u = *reinterpret_cast<const int2*>(&G[rr * lds + col]);
-        const int2 w = *reinterpret_cast<const int2*>(&G[rr * lds + col + 2]);
-        g = make_int4(u.x, u.y, w.x, w.y);
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int u = warp; u < nch * nseg; u += NW) {
+      const int sg = u / nch, col = (u - sg * nch) * 128 + lane * 4;
+      const bool in = col < C;
+      int band[4] = {-1, -1, -1, -1};
+      if (SELECT && nb_tile > 0 && in) {
+        const int4 bv = __ldg(reinterpret_cast<const int4*>(col_band + col));
+        band[0] = bv.x; band[1] = bv.y; band[2] = bv.z; band[3] = bv.w;
       }
-      if (XD || rr == 0) {
-        const int cr = XD ? warp_sum((lane < ch) ? tot[rr * kLane + lane] : 0) : cin;
-        g.y += g.x; g.z += g.y; g.w += g.z;
-        const int incl = warp_incl_scan(g.w, lane);
-        const int add = cr + incl - g.w;
-        v = make_int4(g.x + add, g.y + add, g.z + add, g.w + add);
-      } else {
-        v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w;
-      }
-      if (in) {
-        const int64_t row = t.row0 + rr;
-        __stcs(reinterpret_cast<int4*>(out + row * ld_out + col), v);
-        if (SELECT) {
+      const bool any = SELECT && (band[0] & band[1] & band[2] & band[3]) != -1;
+      const bool all = SELECT && (band[0] | band[1] | band[2] | band[3]) >= 0;
+      int4 v = make_int4(0, 0, 0, 0);
+      if (!XD && in)
+        for (int q = 0; q < sg; ++q) {
+          const int4 g = *reinterpret_cast<const int4*>(seg_sum + q * C + col);
+          v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w;
+        }
+      const int rb = sg * seg_rows, re = in ? min(rb + seg_rows, t.nrows) : rb;
+      const int* g0 = G + rb * lds + col;
+      auto next = [&]() {
+        const int4 g = load4(g0);
+        g0 += lds;
+        if (XD) v = g;
+        else { v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w; }
+      };
+      if (pass == 1) {                             // the cells that hold a sought band's best count
+        int want[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          want[q] = band[q] >= 0 && s_seek[band[q] - t.band_lo] ? s_best[band[q] - t.band_lo] : -1;
+        if ((want[0] & want[1] & want[2] & want[3]) == -1) continue;
+        for (int rr = rb; rr < re; ++rr) {
+          next();
           const int vals[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < 4; ++q)
+            if (vals[q] == want[q])
+              atomicMax(&skey[band[q] - t.band_lo],
+                        cand_key(vals[q], (uint32_t)(t.row0 + rr) * W32 + (uint32_t)(t.col0 + col + q)));
+        }
+        continue;
+      }
+      int32_t* o = out + (int64_t)(t.row0 + rb) * ld_out + col;
+      auto sums = [&]() {                          // of the analysis columns
+        if (all) {
+          s1 += (uint64_t)((uint32_t)v.x + (uint32_t)v.y) + (uint64_t)((uint32_t)v.z + (uint32_t)v.w);
+          s2 += (uint64_t)(uint32_t)v.x * (uint32_t)v.x;
+          s2 += (uint64_t)(uint32_t)v.y * (uint32_t)v.y;
+          s2 += (uint64_t)(uint32_t)v.z * (uint32_t)v.z;
+          s2 += (uint64_t)(uint32_t)v.w * (uint32_t)v.w;
+        } else {
+          const int vals[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
             if (band[q] >= 0) {
-              s1 += vals[q];
-              s2 += (long long)vals[q] * vals[q];
-              if (vals[q] > bc[q]) { bc[q] = vals[q]; br[q] = rr; }
+              s1 += (uint32_t)vals[q];
+              s2 += (uint64_t)(uint32_t)vals[q] * (uint32_t)vals[q];
             }
-          }
+        }
+      };
+      if (!any) {
+        for (int rr = rb; rr < re; ++rr) {
+          next();
+          __stcs(reinterpret_cast<int4*>(o), v);
+          o += ld_out;
+        }
+      } else if (few) {
+        int best[4] = {0, 0, 0, 0};
+        for (int rr = rb; rr < re; ++rr) {
+          next();
+          __stcs(reinterpret_cast<int4*>(o), v);
+          o += ld_out;
+          sums();
+          best[0] = max(best[0], v.x); best[1] = max(best[1], v.y);
+          best[2] = max(best[2], v.z); best[3] = max(best[3], v.w);
+        }
+        if (all && band[0] == band[3]) {           // bands follow the columns
+          atomicMax(&s_best[band[0] - t.band_lo], max(max(best[0], best[1]), max(best[2], best[3])));
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (band[q] >= 0) atomicMax(&s_best[band[q] - t.band_lo], best[q]);
+        }
+      } else {
+        // per column: best count over the rows so far and its row (strictly greater, so the first
+        // row reaching the best count wins: the lowest cell index)
+        int bc[4] = {-1, -1, -1, -1}, br[4] = {0, 0, 0, 0};
+        for (int rr = rb; rr < re; ++rr) {
+          next();
+          __stcs(reinterpret_cast<int4*>(o), v);
+          o += ld_out;
+          sums();
+          const int vals[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (vals[q] > bc[q]) { bc[q] = vals[q]; br[q] = rr; }
+        }
+        unsigned long long best[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          best[q] = bc[q] < 0 ? 0ull : cand_key(bc[q], (uint32_t)(t.row0 + br[q]) * W32 + (uint32_t)(t.col0 + col + q));
+        // merge equal-band neighbours among the lane's 4 columns, then one shared atomic per run
+        // (at the run's last column; every index static, so the arrays stay in registers)
+        unsigned long long run = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          run = (q > 0 && band[q] == band[q - 1]) ? (best[q] > run ? best[q] : run) : best[q];
+          const bool last = q == 3 || band[q < 3 ? q + 1 : q] != band[q];
+          if (band[q] >= 0 && last) atomicMax(&skey[band[q] - t.band_lo], run);
         }
       }
     }
-    if (SELECT) {
-      unsigned long long best[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        best[q] = cand_key(bc[q], (uint32_t)(t.row0 + br[q]) * W32 + (uint32_t)(t.col0 + col + q));
-      // merge equal-band neighbours among the lane's 4 columns, then one shared atomic per run
-      // (at the run's last column; every index static, so the arrays stay in registers)
-      unsigned long long run = 0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        run = (q > 0 && band[q] == band[q - 1]) ? (best[q] > run ? best[q] : run) : best[q];
-        const bool last = q == 3 || band[q < 3 ? q + 1 : q] != band[q];
-        if (band[q] >= 0 && last) atomicMax(&skey[band[q] - t.band_lo], run);
-      }
-    }
-  }
-  if (SELECT) {
-    s1 = warp_sum64(s1);
-    s2 = warp_sum64(s2);
-    if (lane == 0 && (s1 | s2)) {
-      atomicAdd(&md.sums[0], (unsigned long long)s1);
-      atomicAdd(&md.sums[1], (unsigned long long)s2);
+    if (!SELECT || nb_tile == 0) return;
+    if (pass == 0) {
+      // the block's sums so far, per warp (flushed to the map's when the block leaves the map)
+      s1 = (uint64_t)warp_sum64((long long)s1);
+      s2 = (uint64_t)warp_sum64((long long)s2);
+      if (lane == 0) { s_sums[2 * warp] += s1; s_sums[2 * warp + 1] += s2; }
     }
     __syncthreads();
-    for (int i = tid; i < nb_tile; i += NT)
-      if (skey[i]) atomicMax(&md.keys[t.band_lo + i], skey[i]);
+    if (!few || pass == 1) break;
+    if (tid < nb_tile) {
+      const unsigned long long now = *reinterpret_cast<volatile unsigned long long*>(&md.keys[t.band_lo + tid]);
+      s_seek[tid] = now == 0 || s_best[tid] >= (int)(now >> 32);
+    }
+    if (!__syncthreads_or(tid < nb_tile && s_seek[tid])) return;
   }
+  for (int i = tid; i < nb_tile; i += NT)
+    if (skey[i]) atomicMax(&md.keys[t.band_lo + i], skey[i]);
 }
 
-// Persistent blocks over the plan's n_tiles tiles (every map of the plan in one launch): each block
-// takes the next tile from the counter `next` (zeroed before the launch) until none is left.  The
-// plan lists the tiles longest first, so the blocks finish together.  The index of a block's next
-// tile is claimed when it starts a tile and read when it has finished it, so the atomic's round
-// trip is hidden behind the tile.
-template <int R, int NT, bool SELECT, bool XD, int LDS = 0, bool UNIF = false>
-__global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (R <= 4 ? 3 : (R == 8 ? 2 : 1)))
+// Persistent blocks over a list of tiles (every map of the plan in one launch): each block takes the
+// next tile from the counter `next` (zeroed before the launch) until none is left.  The list holds
+// n_tiles tiles, or min(*count, n_tiles) where count is given (the coarse-tile search's list, whose
+// length is known on the device only).  A plan lists its tiles longest first, so the blocks finish
+// together.  The index of a block's next tile is claimed when it starts a tile and read when it has
+// finished it, so the atomic's round trip is hidden behind the tile.
+template <int R, int NT, bool SELECT, bool XD>
+__global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
 k_hough(const MapDev* __restrict__ maps, const TileDev* __restrict__ tiles, int n_tiles,
-        int* __restrict__ next, const uint32_t* __restrict__ fft_idx,
-        const uint32_t* __restrict__ bins, unsigned int* __restrict__ flag, int c_max) {
+        const int* __restrict__ count, int* __restrict__ next, const uint32_t* __restrict__ fft_idx,
+        const int* __restrict__ list_state, unsigned int* __restrict__ flag, int sum_off, int batch) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_next;
+  uint64_t* const s_sums = reinterpret_cast<uint64_t*>(smem + sum_off);
+  int2* const ent = reinterpret_cast<int2*>(smem + sum_off + kSumBytes<NT>);
+  int* const G = reinterpret_cast<int*>(ent + 2 * batch);
+  const int n = count ? min(*count, n_tiles) : n_tiles;
   if (threadIdx.x == 0) s_next = atomicAdd(next, 1);
+  if (threadIdx.x < 2 * NT / kLane) s_sums[threadIdx.x] = 0;
   __syncthreads();
-  int ti = s_next;
-  while (ti < n_tiles) {
+  int ti = s_next, map = -1;
+  // adds the block's sums over the tiles of one map to the map's, and clears them
+  auto flush = [&]() {
+    if (!SELECT || map < 0 || threadIdx.x >= kLane) return;
+    const int l = threadIdx.x;
+    const bool on = l < NT / kLane;
+    const long long a = warp_sum64(on ? (long long)s_sums[2 * l] : 0);
+    const long long b = warp_sum64(on ? (long long)s_sums[2 * l + 1] : 0);
+    if (on) s_sums[2 * l] = s_sums[2 * l + 1] = 0;
+    if (l == 0 && (a | b)) {
+      atomicAdd(&maps[map].sums[0], (unsigned long long)a);
+      atomicAdd(&maps[map].sums[1], (unsigned long long)b);
+    }
+    __syncwarp();
+  };
+  while (ti < n) {
     __syncthreads();                                  // every thread has read s_next
     int claimed = 0;
     if (threadIdx.x == 0) claimed = atomicAdd(next, 1);
     const TileDev t = tiles[ti];
+    if (t.map != map) { flush(); map = t.map; }
     if (t.nrows > 0)
-      hough_tile<R, NT, SELECT, XD, LDS, UNIF>(maps, t, fft_idx, bins, flag, c_max, smem);
+      hough_tile<R, NT, SELECT, XD>(maps, t, fft_idx, list_state, flag, smem, s_sums, ent, batch, G);
     if (threadIdx.x == 0) s_next = claimed;
     __syncthreads();
     ti = s_next;
   }
-}
-
-// Persistent blocks over a tile list whose length is known on the device only (the coarse-tile
-// search): each block takes the next tile from a counter until the list is exhausted.  Its tiles
-// are mostly narrow (a coarse tile's columns), where many warps mix interior peaks with peaks near
-// an edge, so it always draws one form per warp, and tiles flagged `sub` walk only their bins'
-// FFT sub-ranges (hough_tile).
-template <int R, int NT, bool SELECT>
-__global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (R <= 4 ? 3 : (R == 8 ? 2 : 1)))
-k_hough_list(const MapDev* __restrict__ maps, const TileDev* __restrict__ tiles,
-             const int* __restrict__ count, int* __restrict__ next, int cap,
-             const uint32_t* __restrict__ fft_idx, const uint32_t* __restrict__ bins,
-             unsigned int* __restrict__ flag, int c_max, const CoarseMapDev* __restrict__ cmaps,
-             const int* __restrict__ fft_unsorted, int sub_cap) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int s_next;
-  const int n = min(*count, cap);
-  if (threadIdx.x == 0) s_next = atomicAdd(next, 1);
-  __syncthreads();
-  int ti = s_next;
-  while (ti < n) {                                    // next tile claimed during this one
-    __syncthreads();
-    int claimed = 0;
-    if (threadIdx.x == 0) claimed = atomicAdd(next, 1);
-    const TileDev t = tiles[ti];
-    if (t.nrows > 0)
-      hough_tile<R, NT, SELECT, false, 0, true, true>(maps, t, fft_idx, bins, flag, c_max, smem,
-                                                      cmaps, fft_unsorted, sub_cap);
-    if (threadIdx.x == 0) s_next = claimed;
-    __syncthreads();
-    ti = s_next;
-  }
+  flush();
 }
 
 // ---- candidate records ----------------------------------------------------------------------------
@@ -720,89 +884,78 @@ __global__ void k_select_cols(const int32_t* __restrict__ map, const MapDev* __r
   }
 }
 
-// Launch (prepare = false) or set the shared-memory attribute (prepare = true).  Setting the
-// attribute at plan creation keeps gfh_plan_execute to stream operations only (capturable).  The
-// attribute belongs to the kernel, not to a plan, so it is set to the largest size any plan may
-// request: each launch still asks only for its own size (which alone decides occupancy).
-// n_tiles < 0: the persistent list form over p->d_sel_tiles with its device-side count.
-// xd: the x-direction form (tiles of maps with large shifts per k row).
-template <int R, int NT, bool SEL>
-int launch_hough_t(gfh_plan* p, const gfh_peaks* peaks, const TileDev* tiles, int n_tiles,
-                   size_t smem, bool prepare, bool xd) {
-  // the shapes the autotuner picks on the paper-shaped workloads (8-row tiles of 2048 or 3072
-  // columns at 512 threads, 16-row tiles of 3072 columns at 1024 threads) have the row stride
-  // fixed at compile time
-  // drawing form 1: one form per warp
-  const bool unif = p->cfg.form == 1;
-  auto fk = unif ? k_hough<R, NT, SEL, false, 0, true> : k_hough<R, NT, SEL, false>;
-  if constexpr (R == 8 && NT == 512) {
-    if (p->cfg.cols == 3072) fk = unif ? k_hough<R, NT, SEL, false, 3074, true> : k_hough<R, NT, SEL, false, 3074>;
-    if (p->cfg.cols == 2048) fk = unif ? k_hough<R, NT, SEL, false, 2050, true> : k_hough<R, NT, SEL, false, 2050>;
+// Sets the shared-memory attribute of the kernels that a plan launches.  Doing so at plan creation
+// keeps gfh_plan_execute to stream operations only (capturable).  The attribute belongs to the
+// kernel, not to a plan, so it is set to the largest size any plan may request: each launch still
+// asks only for its own size (which alone decides occupancy).
+template <int R, int NT, bool XD>
+int prepare_hough() {
+  for (const void* f : {(const void*)k_hough<R, NT, false, XD>, (const void*)k_hough<R, NT, true, XD>}) {
+    cudaFuncAttributes fa{};
+    GFH_CUDA_TRY(cudaFuncGetAttributes(&fa, f));
+    GFH_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(kMaxSmemBytes - fa.sharedSizeBytes)));
   }
-  if constexpr (R == 16 && NT == 1024) {
-    if (p->cfg.cols == 3072) fk = unif ? k_hough<R, NT, SEL, false, 3074, true> : k_hough<R, NT, SEL, false, 3074>;
-  }
-  auto fn = xd ? k_hough<R, NT, SEL, true> : fk;
-  auto fl = k_hough_list<R, NT, SEL>;
-  if (prepare) {
-    // the kernels this plan launches; each also holds a few bytes of static shared memory (the
-    // tile counter)
-    auto set_max = [](const void* f) -> int {
-      cudaFuncAttributes fa{};
-      GFH_CUDA_TRY(cudaFuncGetAttributes(&fa, f));
-      GFH_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)(kMaxSmemBytes - fa.sharedSizeBytes)));
-      return GFH_OK;
-    };
-    int rc = set_max((const void*)fk);
-    if (!rc) rc = set_max((const void*)k_hough<R, NT, SEL, true>);
-    if (!rc) rc = set_max((const void*)fl);
-    return rc;
-  }
-  if (smem > kHoughSmemLimit) return GFH_ERR_SIZE;
-  if (n_tiles >= 0) {
-    if (n_tiles == 0) return GFH_OK;
-    int per_sm = 0;
-    GFH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NT, smem));
-    const int grid = std::min(n_tiles, p->ctx->num_sms * (per_sm > 0 ? per_sm : 1));
-    fn<<<grid, NT, smem, p->ctx->stream>>>(p->d_maps, tiles, n_tiles, p->d_next + (xd ? 1 : 0),
-                                           peaks->fft_idx, peaks->bin, p->ctx->d_flag,
-                                           p->cfg.cols);
-  } else {
-    int per_sm = 0;
-    GFH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fl, NT, smem));
-    const int grid = p->ctx->num_sms * (per_sm > 0 ? per_sm : 1);
-    fl<<<grid, NT, smem, p->ctx->stream>>>(p->d_maps, tiles, p->d_sel_count, p->d_sel_count + 1,
-                                           p->sel_cap, peaks->fft_idx, peaks->bin, p->ctx->d_flag,
-                                           p->cfg.cols, p->d_cmaps, p->d_fft_unsorted, p->sub_cap);
-  }
+  return GFH_OK;
+}
+
+enum { kFull, kFullX, kList };   // full search's two tile lists (XD: the second), coarse tiles
+
+template <int R, int NT, bool XD>
+int launch_hough_t(gfh_plan* p, const gfh_peaks* peaks, int which) {
+  auto fn = p->select ? k_hough<R, NT, true, XD> : k_hough<R, NT, false, XD>;
+  const bool list = which == kList;
+  const int n_tiles = XD ? p->n_tiles_x : p->n_tiles;
+  if (!list && n_tiles == 0) return GFH_OK;
+  const TileDev* const tiles = list ? p->d_sel_tiles : p->d_tiles + (XD ? p->n_tiles : 0);
+  const size_t cells = list ? p->cells_list : XD ? p->cells_x : p->cells;
+  const size_t head = (size_t)kLane * 4 * (kHoughSpare + (XD ? R : 1)) +
+                      (p->select ? (size_t)p->max_tile_bands * 8 : 0);
+  // head (chunk sums, spare words, band keys), sums, the windows of as many bins as there are
+  // threads, or as fit beside the tile without lowering the blocks per SM, the tile
+  constexpr size_t kOwn = 1024 + 64;             // reserved per block, and the kernel's static bytes
+  const size_t sum_off = (head + 15) / 16 * 16;
+  const size_t fixed = sum_off + kSumBytes<NT> + cells;
+  const size_t blocks = std::max<size_t>(1, std::min<size_t>(kSmemPerSm / (fixed + 16 + kOwn), 2048 / NT));
+  const size_t room = std::min(kSmemPerSm / blocks - kOwn, kMaxSmemBytes - 64);
+  if (fixed + 16 > room) return GFH_ERR_SIZE;
+  const int batch = (int)std::min<size_t>(NT, (room - fixed) / 16);
+  const size_t bytes = fixed + (size_t)batch * 16;
+  int per_sm = 0;
+  GFH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NT, bytes));
+  int grid = p->ctx->num_sms * (per_sm > 0 ? per_sm : 1);
+  if (!list) grid = std::min(grid, n_tiles);
+  fn<<<grid, NT, bytes, p->ctx->stream>>>(
+      p->d_maps, tiles, list ? p->sel_cap : n_tiles, list ? p->d_sel_count : nullptr,
+      list ? p->d_sel_count + 1 : p->d_next + (XD ? 1 : 0), peaks->fft_idx, p->d_list_state,
+      p->ctx->d_flag, (int)sum_off, batch);
   GFH_CUDA_TRY(cudaGetLastError());
   return GFH_OK;
 }
 
-template <int R, int NT>
-int launch_hough_sel(gfh_plan* p, const gfh_peaks* peaks, const TileDev* tiles, int n_tiles,
-                     size_t smem, bool prepare, bool xd) {
-  return p->select ? launch_hough_t<R, NT, true>(p, peaks, tiles, n_tiles, smem, prepare, xd)
-                   : launch_hough_t<R, NT, false>(p, peaks, tiles, n_tiles, smem, prepare, xd);
+// The kernels of a plan: f(rows, threads, XD) as compile-time constants.  The threads are the given
+// shape's (a planned one: 512, and 256 for its coarse tiles).
+template <class F>
+int with_kernel(const gfh_plan* p, int which, F f) {
+  auto rows = [&](auto nt) -> int {
+    if (which != kFullX) return f(std::integral_constant<int, 1>{}, nt, std::false_type{});
+    switch (p->cfg.rows) {
+      case 4: return f(std::integral_constant<int, 4>{}, nt, std::true_type{});
+      case 8: return f(std::integral_constant<int, 8>{}, nt, std::true_type{});
+      case 16: return f(std::integral_constant<int, 16>{}, nt, std::true_type{});
+      default: return f(std::integral_constant<int, 32>{}, nt, std::true_type{});
+    }
+  };
+  const int threads = p->planned && which == kList ? 256 : p->cfg.threads;
+  if (threads == 256) return rows(std::integral_constant<int, 256>{});
+  if (threads == 512) return rows(std::integral_constant<int, 512>{});
+  return rows(std::integral_constant<int, 1024>{});
 }
 
-template <int R>
-int launch_hough_r(gfh_plan* p, const gfh_peaks* peaks, const TileDev* tiles, int n_tiles,
-                   size_t smem, bool prepare, bool xd) {
-  if constexpr (R >= 16)   // 1024 threads: one block of 32 warps per SM holds a 16- or 32-row tile
-    if (p->cfg.threads == 1024) return launch_hough_sel<R, 1024>(p, peaks, tiles, n_tiles, smem, prepare, xd);
-  return p->cfg.threads == 256
-             ? launch_hough_sel<R, 256>(p, peaks, tiles, n_tiles, smem, prepare, xd)
-             : launch_hough_sel<R, 512>(p, peaks, tiles, n_tiles, smem, prepare, xd);
-}
-
-int launch_hough(gfh_plan* p, const gfh_peaks* peaks, const TileDev* tiles, int n_tiles,
-                 size_t smem, bool prepare, bool xd = false) {
-  return p->cfg.rows == 4    ? launch_hough_r<4>(p, peaks, tiles, n_tiles, smem, prepare, xd)
-         : p->cfg.rows == 8  ? launch_hough_r<8>(p, peaks, tiles, n_tiles, smem, prepare, xd)
-         : p->cfg.rows == 16 ? launch_hough_r<16>(p, peaks, tiles, n_tiles, smem, prepare, xd)
-                             : launch_hough_r<32>(p, peaks, tiles, n_tiles, smem, prepare, xd);
+int launch_hough(gfh_plan* p, const gfh_peaks* peaks, int which) {
+  return with_kernel(p, which, [&](auto r, auto nt, auto xd) {
+    return launch_hough_t<decltype(r)::value, decltype(nt)::value, decltype(xd)::value>(p, peaks, which);
+  });
 }
 
 // Appends to one compact list the fine tiles of each map's selected coarse tiles, or, for a map
@@ -835,41 +988,33 @@ __global__ void k_gather_tiles(const TileDev* __restrict__ fine, const int32_t* 
 
 }  // namespace
 
-size_t gfh_hough_smem_bytes(const gfh_plan* p, bool xd) {
-  return (size_t)p->cfg.rows * (p->cfg.cols + 2) * 4 + (size_t)kLane * 4 * (xd ? p->cfg.rows : 1) +
-         (p->select ? (size_t)p->max_tile_bands * 8 : 0);
-}
-
 int gfh_prepare_plan(gfh_plan* p) {
-  const size_t smem = gfh_hough_smem_bytes(p, p->n_tiles_x > 0);
-  if (smem > kHoughSmemLimit) return GFH_ERR_SIZE;
-  return launch_hough(p, nullptr, nullptr, 0, smem, true);
+  for (int which : {kFull, kFullX, kList}) {
+    if (which == kFullX && p->n_tiles_x == 0) continue;
+    const int rc = with_kernel(p, which, [&](auto r, auto nt, auto xd) {
+      return prepare_hough<decltype(r)::value, decltype(nt)::value, decltype(xd)::value>();
+    });
+    if (rc) return rc;
+  }
+  return GFH_OK;
 }
 
 // Per-execute preparation shared by the full and the coarse-tile forms: input check, per-map CSR
 // over bins, zeroed candidate keys.
-static int launch_prologue(gfh_plan* p, const gfh_peaks* peaks, bool coarse = false) {
+static int launch_prologue(gfh_plan* p, const gfh_peaks* peaks) {
   gfh_ctx* ctx = p->ctx;
   cudaStream_t st = ctx->stream;
-  coarse = coarse && p->d_fft_unsorted;
-  if (coarse)
-    GFH_CUDA_TRY(cudaMemsetAsync(p->d_fft_unsorted, 0, sizeof(int) * p->n_list_flags, st));
+  GFH_CUDA_TRY(cudaMemsetAsync(p->d_zeroed, 0, p->zeroed_bytes, st));
   {
-    dim3 grid(64, peaks->n_lists);
+    // a few blocks per SM in all, at least 8 per list
+    dim3 grid(std::max(8, 4 * ctx->num_sms / peaks->n_lists), peaks->n_lists);
     k_check_sorted<<<grid, 256, 0, st>>>(peaks->bin, peaks->fft_idx, peaks->offsets, ctx->d_flag,
-                                         coarse ? p->d_fft_unsorted : nullptr, p->n_list_flags);
+                                         p->d_list_state, p->n_list_states);
     GFH_CUDA_TRY(cudaGetLastError());
   }
-  k_csr<<<(p->csr_entries + 255) / 256, 256, 0, st>>>(p->d_maps, p->d_csr_map, p->csr_entries,
-                                                      peaks->bin, peaks->offsets);
+  k_index<<<(p->csr_entries + 7) / 8, 256, 0, st>>>(p->d_lists, p->d_csr_list, p->csr_entries,
+                                                    peaks->bin, peaks->fft_idx, peaks->offsets);
   GFH_CUDA_TRY(cudaGetLastError());
-  if (coarse && p->fblk_entries > 0) {
-    k_fft_blocks<<<dim3((p->fblk_entries + 255) / 256, p->n_maps), 256, 0, st>>>(
-        p->d_maps, p->d_cmaps, peaks->fft_idx);
-    GFH_CUDA_TRY(cudaGetLastError());
-  }
-  if (p->select)
-    GFH_CUDA_TRY(cudaMemsetAsync(p->d_keys, 0, p->key_words * sizeof(unsigned long long), st));
   return GFH_OK;
 }
 
@@ -886,41 +1031,28 @@ static int launch_epilogue(gfh_plan* p) {
 
 int gfh_launch_plan(gfh_plan* p, const gfh_peaks* peaks) {
   GFH_CUDA_TRY(cudaSetDevice(p->ctx->device));
-  const size_t smem = gfh_hough_smem_bytes(p, false);
-  const size_t smem_x = gfh_hough_smem_bytes(p, true);
-  if (smem > kHoughSmemLimit || (p->n_tiles_x > 0 && smem_x > kHoughSmemLimit)) return GFH_ERR_SIZE;
   int rc = launch_prologue(p, peaks);
   if (rc) return rc;
-  GFH_CUDA_TRY(cudaMemsetAsync(p->d_next, 0, 2 * sizeof(int), p->ctx->stream));
-  if (p->n_tiles > 0) {
-    rc = launch_hough(p, peaks, p->d_tiles, p->n_tiles, smem, false);
-    if (rc) return rc;
-  }
-  if (p->n_tiles_x > 0) {
-    rc = launch_hough(p, peaks, p->d_tiles + p->n_tiles, p->n_tiles_x, smem_x, false, true);
-    if (rc) return rc;
-  }
+  rc = launch_hough(p, peaks, kFull);
+  if (!rc && p->n_tiles_x > 0) rc = launch_hough(p, peaks, kFullX);
+  if (rc) return rc;
   return launch_epilogue(p);
 }
 
 int gfh_launch_plan_tiles(gfh_plan* p, const gfh_peaks* peaks, const int32_t* d_coarse, int n_sel,
                           const int32_t* d_full) {
   GFH_CUDA_TRY(cudaSetDevice(p->ctx->device));
-  // the list kernel's tile, plus the FFT sub-ranges of up to sub_cap bins
-  const size_t smem = gfh_hough_smem_bytes(p, false) + (size_t)p->sub_cap * 8 + 16;
-  if (smem > kHoughSmemLimit) return GFH_ERR_SIZE;
-  int rc = launch_prologue(p, peaks, true);
+  int rc = launch_prologue(p, peaks);
   if (rc) return rc;
   const int nct = p->coarse_k * p->coarse_x;
   cudaStream_t st = p->ctx->stream;
-  GFH_CUDA_TRY(cudaMemsetAsync(p->d_sel_count, 0, 2 * sizeof(int), st));
   const int gx = n_sel > 0 ? n_sel : 1;
   if (n_sel > 0 || d_full) {
     k_gather_tiles<<<dim3(gx, p->n_maps), 128, 0, st>>>(p->d_fine, p->d_coarse_first, d_coarse,
                                                        d_full, n_sel, nct, p->d_sel_tiles,
                                                        p->d_sel_count, p->sel_cap, p->ctx->d_flag);
     GFH_CUDA_TRY(cudaGetLastError());
-    rc = launch_hough(p, peaks, p->d_sel_tiles, -1, smem, false);
+    rc = launch_hough(p, peaks, kList);
     if (rc) return rc;
   }
   return launch_epilogue(p);

@@ -13,8 +13,16 @@
 
 // Largest dynamic shared memory a block may use on sm_103a (227 KB).
 constexpr size_t kMaxSmemBytes = 227 * 1024;
+constexpr size_t kSmemPerSm = 228 * 1024;   // shared memory of one SM
 // dynamic shared memory a Hough tile may take: the kernels keep a few static bytes (tile counter)
 constexpr size_t kHoughSmemLimit = kMaxSmemBytes - 64;
+
+// Shared memory of a Hough tile: words between its rows' ends and starts (rows stay 16-byte aligned,
+// and 4 words from row to row spread a line's cells over the banks), spare words per warp.
+constexpr int kHoughPad = 4, kHoughSpare = 4;
+// Room of a planned tile (words of one of its two counts): two blocks of 512 threads per SM, and
+// three of 256 for the coarse-tile search.
+constexpr int64_t kPlannedWords = 12544, kPlannedListWords = 8224;
 
 // Counter-based generator of the statistical peakmap model: the splitmix64 finaliser (Steele, Lea
 // and Flood, "Fast splittable pseudorandom number generators", OOPSLA 2014) applied to a key built
@@ -81,15 +89,25 @@ struct gfh_ctx {
 
 constexpr int kLogTable = 4096;
 
+// One FFT of a map's shift table: its lines move left by S per k row (2^-32 columns).
+// D = ceil(2^89 / S): rows of 2^-57 per column, for S > 2^25 (0 otherwise).
+struct alignas(16) FftRow {
+  int64_t S;
+  uint64_t D;
+};
+
 // One map as the kernels see it.
 struct MapDev {
   int32_t* out;             // [K][ld]
-  const longlong2* UP;      // J: {U[j+1], U[j]} edge positions of bin j (upper f, lower f)
-  const longlong2* BS;      // n_fft: {B_i, S_i}
+  const longlong2* UP;      // J: {U[j+1], U[j] - 1}: first and last position of bin j
+  const FftRow* SD;         // n_fft
+  const int64_t* B;         // n_fft: shift on row 0 (null: all 0, the default k_min = 0)
   const int32_t* col_band;  // ld entries, -1 outside the analysis band / beyond n_x0
   const double* f0c;        // n_x0
   const double* f0n;        // n_x0
-  int64_t* csr;             // J + 1 entries: first peak (absolute index) of bins bin_lo .. bin_hi+1
+  const int64_t* csr;       // J + 1 entries: first peak (absolute index) of bins bin_lo .. bin_hi+1
+  const int32_t* blk;       // [J][nb1]: offset in a bin's peaks of its first of FFT >= 2^shift b
+  int32_t nb1, shift;
   unsigned long long* keys; // n_bands
   unsigned long long* sums; // 2: sum, sum of squares
   gfh_candidate* cands;     // n_bands (may be null)
@@ -103,20 +121,17 @@ struct MapDev {
   int32_t n_fft;
   int32_t list;
   int32_t n_bands;
-  int32_t csr_base;         // index of this map's first CSR entry in the plan-wide numbering
+  // B_i and S_i against i as lines through the table's first and last rows (a bin's windows of FFTs)
+  int64_t b0, s0;           // B_0, S_0
+  float db, ds;             // (B_last - B_0) / (n_fft - 1), (S_last - S_0) / (n_fft - 1)
 };
 
-// Per map, for the coarse-tile search's FFT sub-ranges: an index of each bin's peaks by blocks of
-// kFftBlock FFTs (built per execute, valid when the map's list holds each bin's peaks in FFT
-// order) and the shift B_i + r S_i against i as a line through the table's first and last rows
-// (the starting guess of a bin's FFT window, which the table then confirms).
-constexpr int kFftBlock = 64;
-struct CoarseMapDev {
-  int32_t* fblk;            // [J][nb1]: offset in the bin's peaks of its first peak with FFT >= 64 b
-  int32_t nb1;              // ceil(n_fft / 64) + 1 entries per bin
-  int32_t list;             // the map's peak list
-  int64_t b0, s0;           // B_0, S_0
-  double db, ds;            // (B_last - B_0) / (n_fft - 1), (S_last - S_0) / (n_fft - 1)
+// The index of one peak list, over the bins that some map reads (built per execute, k_index).
+struct ListDev {
+  int64_t* csr;             // n_bins + 1
+  int32_t* blk;             // [n_bins][nb1]
+  int32_t list, bin_lo, n_bins, nb1, shift;
+  int32_t entry0;           // its first bin in the plan-wide numbering
 };
 
 // One tile of the accumulation kernel: k rows [row0, row0+nrows) x columns [col0, col0+ncols).
@@ -130,8 +145,12 @@ struct TileDev {
   int32_t bin_b;
   int32_t band_lo;    // candidate bands present in the tile's columns (band_hi < 0: none)
   int32_t band_hi;
-  int32_t sub;        // coarse-tile search: walk only each bin's FFT sub-range (see hough_tile)
-  int32_t reserved;
+};
+
+// Tile shapes of a plan's maps.
+struct TilePlan {
+  int rows = 0, cols = 0;       // uniform tiles, or rows = 0:
+  int64_t words = 0;            // shapes chosen by the work they make, within this room
 };
 
 struct gfh_plan {
@@ -139,6 +158,10 @@ struct gfh_plan {
   int n_maps = 0;
   std::vector<gfh_grid> grids;
   gfh_tile_config cfg{};
+  TilePlan shape;              // of uniform tiles
+  bool planned = false;        // tile shapes chosen by their work (the default shape)
+  size_t cells = 0, cells_x = 0, cells_list = 0;   // shared memory of the largest tile's counts: full
+                                                   // search's two lists, coarse tiles
   void* d_buf = nullptr;       // tables, map descriptors, tiles
   size_t buf_bytes = 0;
   MapDev* d_maps = nullptr;
@@ -147,13 +170,20 @@ struct gfh_plan {
   int n_tiles_x = 0;                   // tiles of maps moving > 2 columns per k row: along x0
   std::vector<char> map_xd;            // per map: drawn in the x-direction form
   int max_tile_bands = 0;
-  unsigned long long* d_keys = nullptr;  // all maps' keys and sums (zeroed per execute)
-  size_t key_words = 0;
-  int32_t csr_entries = 0;                // total CSR entries over maps
-  int32_t* d_csr_map = nullptr;           // per CSR entry: map index
+  // zeroed per execute, in one piece: all maps' keys and sums, the lists' order states, the tile
+  // counters (full search's two launches; coarse-tile list length and next tile)
+  void* d_zeroed = nullptr;
+  size_t zeroed_bytes = 0;
+  unsigned long long* d_keys = nullptr;
+  int* d_list_state = nullptr;            // per peak list a map reads: order bits (k_check_sorted)
+  int n_list_states = 0;                  // largest list index + 1
+  int* d_next = nullptr;
+  int* d_sel_count = nullptr;
+  ListDev* d_lists = nullptr;             // the peak lists that maps read
+  int32_t csr_entries = 0;                // their bins in all
+  int32_t* d_csr_list = nullptr;          // per bin: its entry of d_lists
   bool select = false;
   int64_t* d_offsets_single = nullptr;    // scratch offsets for gfh_hough
-  int* d_next = nullptr;                  // tile counters of the full search's two launches
   // the bound outputs, kept so that the autotuner can rebuild the plan with another tile shape
   std::vector<int32_t*> h_maps;
   std::vector<gfh_candidate*> h_cands;
@@ -165,14 +195,7 @@ struct gfh_plan {
   TileDev* d_fine = nullptr;           // fine tiles, grouped by (map, coarse tile)
   int32_t* d_coarse_first = nullptr;   // n_maps * (coarse_k * coarse_x + 1) + 1 group offsets
   TileDev* d_sel_tiles = nullptr;      // the gathered tile list (worst case: every map in full)
-  int* d_sel_count = nullptr;          // [0] list length, [1] next tile (persistent blocks)
   int sel_cap = 0;                     // capacity of d_sel_tiles
-  CoarseMapDev* d_cmaps = nullptr;     // per map: FFT block index and shift line
-  int* d_fft_unsorted = nullptr;       // per peak list: 1 if some bin's peaks are not in FFT order
-  int n_list_flags = 0;                // entries of d_fft_unsorted (largest list index + 1)
-  int sub_cap = 0;                     // bins per tile the sub-range walk holds in shared memory
-  int fblk_entries = 0;                // largest J * nb1 over the maps (index build grid)
-  int n_sub_tiles = 0;                 // coarse-group fine tiles flagged for the sub-range walk
 };
 
 // Host-side planning (gfh_host.cpp).
