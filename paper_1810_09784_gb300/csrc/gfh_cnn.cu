@@ -1219,21 +1219,48 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
 }
 
-// dst[e] += sum_{c < chunks} part[c * n + e], chunks in increasing order (deterministic).
-__global__ void k_sum_chunks(const float* __restrict__ part, int chunks, int n,
-                             float* __restrict__ dst) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
+// dst[e] += sum_{c < chunks} part[c * stride + e] for e < n, and the same of part2 (n2 entries per
+// chunk, their own stride) into dst2: the weights' and the biases' partial sums of a layer in one launch.
+// Chunks are added in increasing order (deterministic); their loads go out kSumAhead at a time, since
+// a sum that waits for each load in turn took 20 us for 304 chunks.
+constexpr int kSumAhead = 32;
+__device__ __forceinline__ float sum_chunks(const float* __restrict__ p, int chunks, int64_t stride) {
   float s = 0.f;
-  for (int c = 0; c < chunks; ++c) s += part[(int64_t)c * n + e];
-  dst[e] += s;
+  int c = 0;
+  for (; c + kSumAhead <= chunks; c += kSumAhead) {
+    float v[kSumAhead];
+#pragma unroll
+    for (int q = 0; q < kSumAhead; ++q) v[q] = __ldg(p + (c + q) * stride);
+#pragma unroll
+    for (int q = 0; q < kSumAhead; ++q) s += v[q];
+  }
+  for (; c < chunks; ++c) s += __ldg(p + c * stride);
+  return s;
+}
+__global__ void k_sum_chunks(const float* __restrict__ part, int chunks, int n, float* __restrict__ dst,
+                             const float* __restrict__ part2, int n2, float* __restrict__ dst2) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < n) dst[e] += sum_chunks(part + e, chunks, n);
+  else if (e < n + n2) dst2[e - n] += sum_chunks(part2 + (e - n), chunks, n2);
 }
 
 // g[i] = dout[i] where out[i] > 0, else 0 (the gradient in a layer's pre-activation), n elements.
+// vec (16-byte aligned arrays, n a multiple of 8): eight elements per thread and array.
+__device__ __forceinline__ uint32_t mask2(uint32_t d, uint32_t o) {   // two bf16 of each
+  const bool lo = __uint_as_float(o << 16) > 0.f, hi = __uint_as_float(o & 0xffff0000u) > 0.f;
+  return (lo ? d & 0xffffu : 0u) | (hi ? d & 0xffff0000u : 0u);
+}
 __global__ void k_mask_grad(const __nv_bfloat16* __restrict__ dout,
                             const __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ g,
-                            int64_t n) {
+                            int64_t n, bool vec) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (vec) {
+    if (i * 8 >= n) return;
+    const uint4 d = __ldcs(reinterpret_cast<const uint4*>(dout) + i);
+    const uint4 o = __ldcs(reinterpret_cast<const uint4*>(out) + i);
+    reinterpret_cast<uint4*>(g)[i] = make_uint4(mask2(d.x, o.x), mask2(d.y, o.y), mask2(d.z, o.z), mask2(d.w, o.w));
+    return;
+  }
   if (i < n) g[i] = __bfloat162float(out[i]) > 0.f ? dout[i] : __float2bfloat16_rn(0.f);
 }
 
@@ -1247,25 +1274,33 @@ __global__ void k_pad_channels(const uint32_t* __restrict__ img, int4* __restric
 }
 
 // dst[co][tap][ci] += sum_{c < chunks} part[c][co][tap][ci8] for ci < 2 (the padded layout has 8
-// input channels), chunks in increasing order.
-__global__ void k_sum_chunks_l1(const float* __restrict__ part, int chunks, float* __restrict__ dst) {
+// input channels), and the 32 biases from part2[c][co], chunks in increasing order.
+__global__ void k_sum_chunks_l1(const float* __restrict__ part, int chunks, float* __restrict__ dst,
+                                const float* __restrict__ part2, float* __restrict__ dst2) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;   // (co, tap, ci) of 32 x 9 x 2
-  if (e >= 576) return;
   const int ci = e & 1, ct = e >> 1;
-  float s = 0.f;
-  for (int c = 0; c < chunks; ++c) s += part[(int64_t)c * 32 * 9 * 8 + ct * 8 + ci];
-  dst[e] += s;
+  if (e < 576) dst[e] += sum_chunks(part + ct * 8 + ci, chunks, 32 * 9 * 8);
+  else if (e < 576 + 32) dst2[e - 576] += sum_chunks(part2 + (e - 576), chunks, 32);
 }
 
 // ---- mean over t, head, loss --------------------------------------------------------------------
-// pooled[b][f][c] = mean_t a5[b][t][f][c]
+// pooled[b][f][c] = mean_t a5[b][t][f][c], four channels per thread, t ascending
 __global__ void k_pool(const __nv_bfloat16* __restrict__ a5, float* __restrict__ pooled, int B) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;   // (b, f, c)
-  if (e >= B * 64 * 64) return;
-  const int b = e / 4096, fc = e % 4096;
-  float s = 0.f;
-  for (int tt = 0; tt < 64; ++tt) s += __bfloat162float(a5[((int64_t)b * 64 + tt) * 4096 + fc]);
-  pooled[e] = s * (1.0f / 64.0f);
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;   // (b, f, c / 4)
+  if (e >= B * 1024) return;
+  const int b = e / 1024, q = e % 1024;
+  const uint2* p = reinterpret_cast<const uint2*>(a5) + (int64_t)b * 64 * 1024 + q;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 16
+  for (int tt = 0; tt < 64; ++tt) {
+    const uint2 v = __ldg(p + tt * 1024);
+    s.x += __uint_as_float(v.x << 16);
+    s.y += __uint_as_float(v.x & 0xffff0000u);
+    s.z += __uint_as_float(v.y << 16);
+    s.w += __uint_as_float(v.y & 0xffff0000u);
+  }
+  constexpr float k = 1.0f / 64.0f;
+  reinterpret_cast<float4*>(pooled)[e] = make_float4(s.x * k, s.y * k, s.z * k, s.w * k);
 }
 
 // logits[b][kt * 64 + f] = bh[kt] + sum_{d, c} wh[kt][d][c] pooled[b][f + d - 1][c]; logits[b][4096]
@@ -1344,55 +1379,124 @@ __global__ void k_softmax_ce(const float* __restrict__ logits, const int32_t* __
       dlogits[(int64_t)b * kClasses + c] = (expf(l[c] - lse) - (c == y ? 1.f : 0.f)) / (float)B;
 }
 
-// Head weight/bias gradients: one thread per (kt, d, c) weight, plus bias and null bias, summing
-// the images of chunk blockIdx.y (kHeadImgs images) into part[chunk][weight] (k_sum_chunks adds the
-// chunks in order).
-constexpr int kHeadImgs = 16, kHeadParams = 64 * 3 * 64 + 65;
-__global__ void k_head_wgrad(const float* __restrict__ dlogits, const float* __restrict__ pooled,
-                             float* __restrict__ part, int B) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+// Head weight/bias gradients, the images of chunk blockIdx.y (kHeadImgs images) summed into
+// part[chunk][weight] (k_sum_chunks adds the chunks in order); every sum takes its images, and the f of
+// each, in increasing order.  Block x < 8: the weights of 8 k tiles; a thread owns a channel c and four
+// k tiles with their three taps, so that one pooled value and one 16-byte read of four k tiles'
+// gradients serve 12 products (0.148 ms per 256 images with a thread per weight and two global reads
+// per product).  Block x = 8: the biases.
+constexpr int kHeadImgs = 16, kHeadParams = 64 * 3 * 64 + 65, kHeadKt = 8;
+__global__ void __launch_bounds__(128) k_head_wgrad(const float* __restrict__ dlogits,
+                                                    const float* __restrict__ pooled,
+                                                    float* __restrict__ part, int B) {
+  __shared__ __align__(16) float pp[64 * 64];            // [f][c]
+  __shared__ __align__(16) float dl[64 * kHeadKt];       // [f][k tile of the block]
+  const int tid = threadIdx.x;
   const int b0 = blockIdx.y * kHeadImgs, b1 = min(B, b0 + kHeadImgs);
-  float s = 0.f;
-  if (e < 64 * 3 * 64) {
-    const int kt = e / 192, d = (e / 64) % 3, c = e % 64;
-    for (int b = b0; b < b1; ++b)
-      for (int f = 0; f < 64; ++f) {
-        const int ff = f + d - 1;
-        if (ff < 0 || ff >= 64) continue;
-        s += dlogits[(int64_t)b * kClasses + kt * 64 + f] * pooled[((int64_t)b * 64 + ff) * 64 + c];
-      }
-  } else if (e < 64 * 3 * 64 + 64) {
-    const int kt = e - 64 * 3 * 64;
-    for (int b = b0; b < b1; ++b)
-      for (int f = 0; f < 64; ++f) s += dlogits[(int64_t)b * kClasses + kt * 64 + f];
-  } else if (e == 64 * 3 * 64 + 64) {
-    for (int b = b0; b < b1; ++b) s += dlogits[(int64_t)b * kClasses + kClasses - 1];
-  } else {
+  float* const out = part + (int64_t)blockIdx.y * kHeadParams;
+  if (blockIdx.x == 64 / kHeadKt) {                      // biases: pp holds [kt][f], rows padded by hand
+    float s = 0.f;
+    for (int b = b0; b < b1; ++b) {
+      const float* g = dlogits + (int64_t)b * kClasses;
+      __syncthreads();
+      for (int e = tid; e < 64 * 64; e += 128) pp[(e & ~63) | ((e + (e >> 6)) & 63)] = g[e];   // rotated rows
+      __syncthreads();
+      if (tid < 64) for (int f = 0; f < 64; ++f) s += pp[tid * 64 + ((f + tid) & 63)];
+      else if (tid == 64) s += g[kClasses - 1];
+    }
+    if (tid < 65) out[64 * 3 * 64 + tid] = s;
     return;
   }
-  part[(int64_t)blockIdx.y * kHeadParams + e] = s;
+  const int c = tid & 63, half = tid >> 6, kt0 = blockIdx.x * kHeadKt;
+  float acc[4][3] = {};
+  for (int b = b0; b < b1; ++b) {
+    __syncthreads();
+    for (int e = tid; e < 1024; e += 128)
+      reinterpret_cast<float4*>(pp)[e] = __ldg(reinterpret_cast<const float4*>(pooled + (int64_t)b * 4096) + e);
+    for (int e = tid; e < 64 * kHeadKt; e += 128)
+      dl[(e & 63) * kHeadKt + (e >> 6)] = __ldg(dlogits + (int64_t)b * kClasses + kt0 * 64 + e);
+    __syncthreads();
+    auto grads = [&](int f) { return *reinterpret_cast<const float4*>(dl + f * kHeadKt + 4 * half); };
+    // tap d pairs pooled row ff with f = ff - d + 1
+    auto add = [&](int d, const float4& g, float v) {
+      acc[0][d] += g.x * v;
+      acc[1][d] += g.y * v;
+      acc[2][d] += g.z * v;
+      acc[3][d] += g.w * v;
+    };
+    float4 prev = make_float4(0.f, 0.f, 0.f, 0.f), cur = grads(0), next = grads(1);
+    add(0, next, pp[c]);
+    add(1, cur, pp[c]);
+#pragma unroll 2
+    for (int ff = 1; ff < 63; ++ff) {
+      prev = cur;
+      cur = next;
+      next = grads(ff + 1);
+      const float v = pp[ff * 64 + c];
+      add(0, next, v);
+      add(1, cur, v);
+      add(2, prev, v);
+    }
+    add(1, next, pp[63 * 64 + c]);
+    add(2, cur, pp[63 * 64 + c]);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) out[((kt0 + 4 * half + q) * 3 + d) * 64 + c] = acc[q][d];
 }
 
 // d a5[b][t][f][c] = (1/64) sum_{kt, d} dlogits[b][kt * 64 + f - d + 1] wh[kt][d][c]  (same for all t),
-// stored masked by a5 > 0: the gradient in layer 5's pre-activation
-__global__ void k_head_dgrad(const float* __restrict__ dlogits, const float* __restrict__ wh,
-                             const __nv_bfloat16* __restrict__ a5, __nv_bfloat16* __restrict__ da5,
-                             int B) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;   // (b, f, c)
-  if (e >= B * 4096) return;
-  const int b = e / 4096, f = (e / 64) % 64, c = e % 64;
-  float s = 0.f;
-  for (int kt = 0; kt < 64; ++kt)
-    for (int d = 0; d < 3; ++d) {
-      const int fo = f - d + 1;
-      if (fo < 0 || fo >= 64) continue;
-      s += dlogits[(int64_t)b * kClasses + kt * 64 + fo] * wh[(kt * 3 + d) * 64 + c];
+// stored masked by a5 > 0: the gradient in layer 5's pre-activation.  Block (b, y): image b, rows
+// f = 16 y .. 16 y + 15; a thread owns a channel and four rows (kt, then d ascending in every sum),
+// then the block streams its part of all 64 t, 16 bytes per thread and access.  Bound by those 268 MB
+// per 256 images (0.127 ms with 2-byte accesses and a pass over the weights per output).
+__global__ void __launch_bounds__(256) k_head_dgrad(const float* __restrict__ dlogits,
+                                                    const float* __restrict__ wh,
+                                                    const __nv_bfloat16* __restrict__ a5,
+                                                    __nv_bfloat16* __restrict__ da5) {
+  constexpr int kKt = 32;                                // k tiles staged at a time
+  __shared__ __align__(16) float ws[kKt * 192];
+  __shared__ float dl[kKt * 18];                         // f = 16 y - 1 .. 16 y + 16
+  __shared__ __align__(16) __nv_bfloat16 v[16 * 64];
+  const int b = blockIdx.x, f0 = blockIdx.y * 16, tid = threadIdx.x;
+  const int c = tid & 63, fg = (tid >> 6) * 4;
+  float s[4] = {};
+  for (int k0 = 0; k0 < kTiles; k0 += kKt) {
+    __syncthreads();
+    for (int e = tid; e < kKt * 48; e += 256)
+      reinterpret_cast<float4*>(ws)[e] = __ldg(reinterpret_cast<const float4*>(wh + k0 * 192) + e);
+    for (int e = tid; e < kKt * 18; e += 256) {
+      const int kt = e / 18, f = f0 - 1 + e % 18;
+      dl[e] = f >= 0 && f < 64 ? __ldg(dlogits + (int64_t)b * kClasses + (k0 + kt) * 64 + f) : 0.f;
     }
-  const __nv_bfloat16 v = __float2bfloat16_rn(s * (1.0f / 64.0f));
-  const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-  for (int tt = 0; tt < 64; ++tt) {
-    const int64_t i = ((int64_t)b * 64 + tt) * 4096 + f * 64 + c;
-    da5[i] = __bfloat162float(a5[i]) > 0.f ? v : zero;
+    __syncthreads();
+    for (int kt = 0; kt < kKt; ++kt) {
+      const float w0 = ws[kt * 192 + c], w1 = ws[kt * 192 + 64 + c], w2 = ws[kt * 192 + 128 + c];
+      float g[6];
+#pragma unroll
+      for (int j = 0; j < 6; ++j) g[j] = dl[kt * 18 + fg + j];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int f = f0 + fg + j;
+        if (f < 63) s[j] += g[j + 2] * w0;
+        s[j] += g[j + 1] * w1;
+        if (f > 0) s[j] += g[j] * w2;
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[(fg + j) * 64 + c] = __float2bfloat16_rn(s[j] * (1.0f / 64.0f));
+  __syncthreads();
+  // 128 vectors of 8 channels per t
+  const uint4 mine = reinterpret_cast<const uint4*>(v)[tid & 127];
+  const int64_t base = (int64_t)b * 64 * 512 + f0 * 8 + (tid & 127);
+  const uint4* src = reinterpret_cast<const uint4*>(a5) + base;
+  uint4* dst = reinterpret_cast<uint4*>(da5) + base;
+#pragma unroll 8
+  for (int tt = tid >> 7; tt < 64; tt += 2) {
+    const uint4 o = __ldg(src + tt * 512);
+    dst[tt * 512] = make_uint4(mask2(mine.x, o.x), mask2(mine.y, o.y), mask2(mine.z, o.z), mask2(mine.w, o.w));
   }
 }
 
@@ -1618,6 +1722,14 @@ int wgrad_launch(const __nv_bfloat16* G, const __nv_bfloat16* in, int B, int H, 
   return GFH_OK;
 }
 
+cudaError_t mask_grad(const __nv_bfloat16* dout, const __nv_bfloat16* out, __nv_bfloat16* g, int64_t n,
+                      cudaStream_t st) {
+  const bool vec = n % 8 == 0 && ((uintptr_t)dout | (uintptr_t)out | (uintptr_t)g) % 16 == 0;
+  const int64_t threads = vec ? n / 8 : n;
+  k_mask_grad<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(dout, out, g, n, vec);
+  return cudaGetLastError();
+}
+
 // Weight gradient on tcgen05 (k_wgrad_tma) added into dw and bias gradient into db, from the
 // gradient in the pre-activation G (masked); output rows and columns a multiple of 64.
 template <int CIN, int COUT, int S>
@@ -1626,9 +1738,7 @@ int conv_wgrad_tc(const __nv_bfloat16* G, const __nv_bfloat16* in, float* dw, fl
   const int rc = wgrad_launch<CIN, COUT, S>(G, in, B, H, part, st, flag);
   if (rc) return rc;
   const int n = COUT * 9 * CIN, chunks = wgrad_chunks(CIN);
-  k_sum_chunks<<<(n + 255) / 256, 256, 0, st>>>(part, chunks, n, dw);
-  GFH_CUDA_TRY(cudaGetLastError());
-  k_sum_chunks<<<1, 64, 0, st>>>(part + (size_t)chunks * n, chunks, COUT, db);
+  k_sum_chunks<<<(n + COUT + 127) / 128, 128, 0, st>>>(part, chunks, n, dw, part + (size_t)chunks * n, COUT, db);
   GFH_CUDA_TRY(cudaGetLastError());
   return GFH_OK;
 }
@@ -1646,9 +1756,8 @@ int conv1_wgrad(const __nv_bfloat16* g1, const __nv_bfloat16* in, __nv_bfloat16*
   }
   const int rc = wgrad_launch<8, 32, 1>(g1, img8, B, H, part, st, flag);
   if (rc) return rc;
-  k_sum_chunks_l1<<<(576 + 255) / 256, 256, 0, st>>>(part, WT_CHUNKS1, dw);
-  GFH_CUDA_TRY(cudaGetLastError());
-  k_sum_chunks<<<1, 64, 0, st>>>(part + (size_t)WT_CHUNKS1 * 32 * 9 * 8, WT_CHUNKS1, 32, db);
+  k_sum_chunks_l1<<<(576 + 32 + 63) / 64, 64, 0, st>>>(part, WT_CHUNKS1, dw,
+                                                       part + (size_t)WT_CHUNKS1 * 32 * 9 * 8, db);
   GFH_CUDA_TRY(cudaGetLastError());
   return GFH_OK;
 }
@@ -1722,7 +1831,7 @@ int forward(gfh_cnn* n, const __nv_bfloat16* img, int B, bool masks) {
   if (!rc) rc = conv_fwd<64, 64, 1>(n->act[4], n->wb[4], n->w + L.b[4], nullptr, nullptr, n->act[5],
                                     B, 64, sms, st, flag);
   if (rc) return rc;
-  k_pool<<<(B * 4096 + 255) / 256, 256, 0, st>>>(n->act[5], n->pooled, B);
+  k_pool<<<(B * 1024 + 127) / 128, 128, 0, st>>>(n->act[5], n->pooled, B);
   k_head_fwd<<<dim3(kTiles / kHeadKtPerBlock, B), 256, 0, st>>>(n->pooled, n->w + L.wh, n->w + L.bh,
                                                                 n->w + L.bnull, n->logits);
   GFH_CUDA_TRY(cudaGetLastError());
@@ -1738,9 +1847,9 @@ int backward(gfh_cnn* n, const __nv_bfloat16* img, const int32_t* labels, int B)
   GFH_CUDA_TRY(cudaMemsetAsync(n->gw, 0, L.total * sizeof(float), st));
   k_softmax_ce<<<B, 256, 0, st>>>(n->logits, labels, n->dlogits, n->loss, B);
   const int hchunks = (B + kHeadImgs - 1) / kHeadImgs;
-  k_head_wgrad<<<dim3((kHeadParams + 255) / 256, hchunks), 256, 0, st>>>(n->dlogits, n->pooled, n->part, B);
-  k_sum_chunks<<<(kHeadParams + 255) / 256, 256, 0, st>>>(n->part, hchunks, kHeadParams, n->gw + L.wh);
-  k_head_dgrad<<<(B * 4096 + 255) / 256, 256, 0, st>>>(n->dlogits, n->w + L.wh, n->act[5], n->dact[5], B);
+  k_head_wgrad<<<dim3(64 / kHeadKt + 1, hchunks), 128, 0, st>>>(n->dlogits, n->pooled, n->part, B);
+  k_sum_chunks<<<(kHeadParams + 127) / 128, 128, 0, st>>>(n->part, hchunks, kHeadParams, n->gw + L.wh, nullptr, 0, nullptr);
+  k_head_dgrad<<<dim3(B, 4), 256, 0, st>>>(n->dlogits, n->w + L.wh, n->act[5], n->dact[5]);
   GFH_CUDA_TRY(cudaGetLastError());
   int rc = conv_wgrad_tc<64, 64, 1>(n->dact[5], n->act[4], n->gw + L.w[4], n->gw + L.b[4], B, 64, n->part, st, flag);
   if (!rc) rc = conv_fwd<64, 64, 1, 1>(n->dact[5], n->wb[4], nullptr, n->mbits[4], nullptr, n->dact[4], B, 64, sms, st, flag);
@@ -2063,16 +2172,14 @@ extern "C" int gfh_conv3x3(gfh_ctx* ctx, int32_t mode, int32_t cin, int32_t cout
     if (mode == 1) {                                                                               \
       const int64_t n_el = (int64_t)batch * (h / S) * (h / S) * CO;                                \
       __nv_bfloat16* g = (__nv_bfloat16*)ctx->pm_buf;                                              \
-      k_mask_grad<<<(unsigned)((n_el + 255) / 256), 256, 0, st>>>(dout, out, g, n_el);              \
-      GFH_CUDA_TRY(cudaGetLastError());                                                            \
+      GFH_CUDA_TRY(mask_grad(dout, out, g, n_el, st));                                              \
       return conv_fwd<CO, CI, 1, S == 1 ? 1 : 2>(g, w, nullptr, nullptr, nullptr, (__nv_bfloat16*)d_res, \
                                                  batch, h, sms, st, ctx->d_flag);                  \
     }                                                                                              \
     if (mode == 2) {                                                                               \
       const int64_t n_el = (int64_t)batch * (h / S) * (h / S) * CO;                                \
       __nv_bfloat16* g = (__nv_bfloat16*)((char*)ctx->pm_buf + part_bytes);                       \
-      k_mask_grad<<<(unsigned)((n_el + 255) / 256), 256, 0, st>>>(dout, out, g, n_el);              \
-      GFH_CUDA_TRY(cudaGetLastError());                                                            \
+      GFH_CUDA_TRY(mask_grad(dout, out, g, n_el, st));                                              \
       return conv_wgrad_tc<CI, CO, S>(g, in, (float*)d_res, d_db, batch, h, part, st, ctx->d_flag); \
     }                                                                                              \
     return GFH_ERR_ARG;                                                                            \
@@ -2085,8 +2192,7 @@ extern "C" int gfh_conv3x3(gfh_ctx* ctx, int32_t mode, int32_t cin, int32_t cout
       const int64_t n_el = (int64_t)batch * h * h * 32;
       __nv_bfloat16* g = (__nv_bfloat16*)((char*)ctx->pm_buf + part_bytes);
       __nv_bfloat16* img8 = g + n_el;
-      k_mask_grad<<<(unsigned)((n_el + 255) / 256), 256, 0, st>>>(dout, out, g, n_el);
-      GFH_CUDA_TRY(cudaGetLastError());
+      GFH_CUDA_TRY(mask_grad(dout, out, g, n_el, st));
       return conv1_wgrad(g, in, img8, (float*)d_res, d_db, batch, h, part, st, ctx->d_flag, false);
     }
     return GFH_ERR_ARG;
