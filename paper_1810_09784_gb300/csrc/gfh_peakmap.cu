@@ -4,9 +4,10 @@
 //
 // The equaliser is one sequential recurrence per FFT.  A warp owns 32 FFTs (one per lane); tiles
 // of 32 FFTs x 32 bins are staged through shared memory with coalesced loads and every lane walks
-// its own spectrum.  Each step's peak decisions of the warp form one 32-bit ballot word, stored in
+// its own spectrum.  The peak decisions of a warp on one bin form one 32-bit ballot word, stored in
 // a bin-major bit matrix that the compaction kernels turn into sorted lists.
 #include <mutex>
+#include <type_traits>
 
 #include "gfh_internal.h"
 
@@ -49,156 +50,147 @@ struct BandIn {
   }
 };
 
-// Asynchronous copy of one raw element (4 or 8 bytes) to shared memory; ok = false fills zeros
-// (the source is then not read).
+// Asynchronous copy of one raw element (4 or 8 bytes) to shared memory.
 template <class Raw>
-__device__ __forceinline__ void eq_copy(Raw* dst, const Raw* src, bool ok) {
+__device__ __forceinline__ void eq_copy(Raw* dst, const Raw* src) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src),
-               "n"((int)sizeof(Raw)), "r"(ok ? (int)sizeof(Raw) : 0)
-               : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"((int)sizeof(Raw)) : "memory");
 }
+
+// One step of the clipped mean: S + w (min(G P, 2.5 G S) - S).
+// FAST needs S >= 2^-100: the difference is then a multiple of 2^-142 or above 2^-118 in size, so its
+// product with 2^-7 is exact and one fused multiply-add rounds as the multiply and the add do (four
+// dependent operations per bin, 18 cycles against 22).
+template <bool FAST>
+__device__ __forceinline__ float mean_step(float S, float P) {
+  const float u = fminf(__fmul_rn(P, kGain), __fmul_rn(S, kClipGain));
+  const float d = __fsub_rn(u, S);
+  return FAST ? __fmaf_rn(kArWeight, d, S) : __fadd_rn(S, __fmul_rn(kArWeight, d));
+}
+// a mean that cannot fall below 2^-100 within 32 steps (each keeps at least 1 - 2^-7 of it); not for NaN
+__device__ __forceinline__ bool fast_mean(float S) { return S >= 0x1p-98f; }
 
 // bits[(b - bin_lo) * n_words + w], bit l: FFT 32 w + l has a peak in bin b.
 //
-// One block of kEqWarps warps per 32 FFTs (lane l = FFT 32 w + l), over chunks of 32 bins:
-//   warp 0      runs only the recurrence of chunk c (the mean each bin is divided by, then the
-//               update: four dependent operations per bin, the one serial part) and leaves the
-//               means in shared memory;
-//   warps 1..H  copy chunk c + kEqDepth into a ring in shared memory (asynchronous copies, one
-//               group per chunk, each helper its own rows), divide chunk c-1 (helper h takes bins
-//               h-1, h-1+H, ...), meet at a named barrier, take the peak decisions of chunk c-1 one
-//               bin late (bin b needs R at b+1, one ballot word per bin), then wait for their rows
-//               of chunk c+1 and turn them into powers for the recurrence.
-// Rings: kEqDepth + 1 raw tiles, three power tiles, two mean tiles, two equalised tiles; one block
-// barrier per chunk.  The copies run kEqDepth chunks ahead so that memory latency stays off the
-// recurrence, and a full chunk past the warm-up is one straight-line run of 32 updates, its loads
-// issued ahead of the chain.
-constexpr int kEqWarps = 16;
-constexpr int kEqHelpers = kEqWarps - 1;
-constexpr int kEqDepth = 4;
-constexpr int kEqRing = kEqDepth + 1;
+// One block per 32 FFTs (lane l = FFT 32 w + l), over chunks of 32 bins, a barrier per chunk:
+//   warp 0      runs only the recurrence, one chunk per turn, and leaves the mean before every fourth
+//               bin in shared memory;
+//   kEqCopy     warps copy the spectra kEqDepth chunks ahead into a ring (asynchronous copies, each
+//               warp its own rows) and turn the next chunk into powers, bin-major;
+//   kEqSel      warps, two chunks behind, take four bins each: they repeat the recurrence from the mean
+//               before the first, divide, and decide (bin b needs R at b - 1 .. b + 1, so six steps).
+// Bound by the chunk's slowest warp: the recurrence (7930 dependent steps of four operations, 18 cycles
+// each, for a 50-2000 Hz band) beside about 2300 warp instructions per chunk; 161 us while every SM
+// holds one block (4864 FFTs), more where 6 SMs hold two.  Before, the division and the decisions of a
+// chunk were spread bin by bin over 15 warps, 4300 warp instructions per chunk.
+// For 5039 FFTs x 7930 bins: 0.440 ms then, 0.207 ms now; 1799 x 730: 33 us then, 18 us now.
+constexpr int kEqCopy = 3, kEqSel = 8, kEqWarps = 1 + kEqCopy + kEqSel;
+constexpr int kEqDepth = 6, kEqRing = kEqDepth + 1;
+constexpr int kEqSub = 32 / kEqSel;              // bins per deciding warp
 
 template <class In>
 size_t eq_smem_bytes() { return (size_t)kEqRing * 32 * 32 * sizeof(typename In::Raw); }
 
 template <class In>
-__global__ void __launch_bounds__(32 * kEqWarps) k_equalise(In in, int n_fft, int bin_lo,
-                                                            int bin_hi, float theta,
-                                                            uint32_t* __restrict__ bits,
+__global__ void __launch_bounds__(32 * kEqWarps) k_equalise(In in, int n_fft, int bin_lo, int bin_hi,
+                                                            float theta, uint32_t* __restrict__ bits,
                                                             int n_words) {
   using Raw = typename In::Raw;
+  constexpr int kWarmChunks = kWarm / 32, kRows = (32 + kEqCopy - 1) / kEqCopy;
   extern __shared__ __align__(16) unsigned char eq_dyn[];
-  Raw* raw = reinterpret_cast<Raw*>(eq_dyn);   // [kEqRing][32 ffts][32 bins]
-  __shared__ float Pt[3][32][33];   // [chunk ring][fft][bin]
-  __shared__ float Sm[2][32][33];   // [chunk ring][fft][bin]: mean each bin is divided by
-  __shared__ float Rt[2][32][32];   // [chunk ring][bin][fft]: equalised values
+  Raw* raw = reinterpret_cast<Raw*>(eq_dyn);     // [kEqRing][32 ffts][32 bins]
+  __shared__ float Pt[4][32][33];                // [chunk ring][bin][fft]
+  __shared__ float Sm[4][kEqSel][32];            // [chunk ring][deciding warp][fft]: mean before its bins
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x;        // word index: FFTs 32 gw .. 32 gw + 31
-  const int fft0 = gw * 32;
-  const int my_fft = fft0 + lane;
-  const int j0 = bin_lo - 1 - kWarm;    // first warm-up bin
-  const int j_end = bin_hi + 1;         // last equalised bin
-  const int n_chunks = (j_end - j0 + 32) / 32;
-  constexpr int kRowsPerHelper = (32 + kEqHelpers - 1) / kEqHelpers;
-  const int h = warp - 1;
-  // helper: copy its rows of chunk x (zeros past the last FFT or bin), as one commit group
+  const int gw = blockIdx.x, fft0 = gw * 32;
+  const bool live = fft0 + lane < n_fft;
+  const int j0 = bin_lo - 1 - kWarm;             // first warm-up bin
+  const int n_chunks = (bin_hi + 1 - j0 + 32) / 32;
+  // rows past the last FFT and bins past bin_hi + 1 repeat the last (their decisions are not taken)
+  const int h = warp - 1;                        // copying warp
   auto issue = [&](int x) {
     if (x < n_chunks) {
       Raw* slot = raw + (x % kEqRing) * 32 * 32;
+      const int j = min(j0 + 32 * x + lane, bin_hi + 1);
 #pragma unroll
-      for (int i = 0; i < kRowsPerHelper; ++i) {
-        const int r = h + i * kEqHelpers;
-        if (r < 32) {
-          const int f = fft0 + r, j = j0 + 32 * x + lane;
-          const bool ok = f < n_fft && j <= j_end;
-          eq_copy(slot + r * 32 + lane, ok ? in.src(f, j) : in.src(0, j0), ok);
-        }
+      for (int i = 0; i < kRows; ++i) {
+        const int r = h + i * kEqCopy;
+        if (r < 32) eq_copy(slot + r * 32 + lane, in.src(min(fft0 + r, n_fft - 1), j));
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  // helper: its rows of chunk x, raw -> power tile
   auto convert = [&](int x) {
     if (x < n_chunks) {
       const Raw* slot = raw + (x % kEqRing) * 32 * 32;
 #pragma unroll
-      for (int i = 0; i < kRowsPerHelper; ++i) {
-        const int r = h + i * kEqHelpers;
-        if (r < 32) Pt[x % 3][r][lane] = In::power(slot[r * 32 + lane]);
+      for (int i = 0; i < kRows; ++i) {
+        const int r = h + i * kEqCopy;
+        if (r < 32) Pt[x & 3][lane][r] = In::power(slot[r * 32 + lane]);
       }
     }
   };
-  if (warp > 0) {
+  const bool copier = warp >= 1 && warp <= kEqCopy;
+  if (copier) {
     for (int x = 0; x < kEqDepth; ++x) issue(x);
     asm volatile("cp.async.wait_group %0;" ::"n"(kEqDepth - 1) : "memory");   // chunk 0
     convert(0);
   }
   __syncthreads();
-  float S = 0.f;                        // warp 0: running mean of FFT my_fft
-  for (int c = 0; c <= n_chunks; ++c) {
+  float S = 0.f;                                 // warp 0: running mean of FFT fft0 + lane
+  for (int c = 0; c < n_chunks + 2; ++c) {
     if (warp == 0) {
       if (c < n_chunks) {
-        const int cb = j0 + 32 * c;
-        const int nq = min(32, j_end - cb + 1);
-        const float* row = Pt[c % 3][lane];
-        float* srow = Sm[c & 1][lane];
-        if (nq == 32 && cb >= bin_lo - 1) {
-          // a full chunk past the warm-up (all but a few): straight-line code, so the chunk's
-          // loads and the P-only products run ahead of the chain of dependent updates
-          float P[32];
+        float P[32];
 #pragma unroll
-          for (int q = 0; q < 32; ++q) P[q] = row[q];
+        for (int q = 0; q < 32; ++q) P[q] = Pt[c & 3][q][lane];
+        auto steps = [&](auto fast) {
 #pragma unroll
           for (int q = 0; q < 32; ++q) {
-            srow[q] = S;
-            const float u = fminf(__fmul_rn(P[q], kGain), __fmul_rn(S, kClipGain));
-            S = __fadd_rn(S, __fmul_rn(kArWeight, __fsub_rn(u, S)));
+            if (q % kEqSub == 0) Sm[c & 3][q / kEqSub][lane] = S;
+            S = mean_step<decltype(fast)::value>(S, P[q]);
           }
+        };
+        if (c < kWarmChunks) {
+#pragma unroll
+          for (int q = 0; q < 32; ++q) S = __fadd_rn(S, P[q]);
+          if (c == kWarmChunks - 1) S = __fmul_rn(S, 1.0f / kWarm);
+        } else if (__all_sync(0xffffffffu, fast_mean(S))) {
+          steps(std::true_type{});
         } else {
-#pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            if (q < nq) {
-              const int j = cb + q;
-              const float P = row[q];
-              srow[q] = S;
-              if (j < bin_lo - 1) {
-                S = __fadd_rn(S, P);
-                if (j == bin_lo - 2) S = __fmul_rn(S, 1.0f / kWarm);
-              } else {
-                const float u = fminf(__fmul_rn(P, kGain), __fmul_rn(S, kClipGain));
-                S = __fadd_rn(S, __fmul_rn(kArWeight, __fsub_rn(u, S)));
-              }
-            }
-          }
+          steps(std::false_type{});
         }
       }
-    } else {
+    } else if (copier) {
       issue(c + kEqDepth);
-      if (c >= 1) {
-        const int cp = c - 1;
-        const int cb = j0 + 32 * cp;
-        const int nq = min(32, j_end - cb + 1);
-        // equalised values of this helper's bins: R_j = P_j / S_(j-1)
-        for (int q = h; q < nq; q += kEqHelpers)
-          if (cb + q >= bin_lo - 1)
-            Rt[cp & 1][q][lane] = __fdiv_rn(Pt[cp % 3][lane][q], Sm[cp & 1][lane][q]);
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kEqHelpers));
-        // decisions for bins b = cb + q - 1: neighbours b-1, b, b+1 (the first two may sit in
-        // the previous chunk's tile)
-        for (int q = h; q < nq; q += kEqHelpers) {
-          const int b = cb + q - 1;
-          if (b < bin_lo || b > bin_hi) continue;
-          const float rl = q >= 2 ? Rt[cp & 1][q - 2][lane] : Rt[(cp + 1) & 1][q + 30][lane];
-          const float rc = q >= 1 ? Rt[cp & 1][q - 1][lane] : Rt[(cp + 1) & 1][31][lane];
-          const float rr = Rt[cp & 1][q][lane];
-          const bool pk = my_fft < n_fft && rc > theta && rc > rl && rc > rr;
-          const uint32_t word = __ballot_sync(0xffffffffu, pk);
-          if (lane == 0) bits[(int64_t)(b - bin_lo) * n_words + gw] = word;
-        }
-      }
-      asm volatile("cp.async.wait_group %0;" ::"n"(kEqDepth - 1) : "memory");   // chunk c+1
+      asm volatile("cp.async.wait_group %0;" ::"n"(kEqDepth - 1) : "memory");   // chunk c + 1
       convert(c + 1);
+    } else {
+      const int y = c - 2, w = warp - 1 - kEqCopy;
+      if (y >= kWarmChunks) {
+        const int jb = j0 + 32 * y + kEqSub * w; // bin of the first step
+        float s = Sm[y & 3][w][lane], R[kEqSub + 2];
+        auto steps = [&](auto fast) {
+#pragma unroll
+          for (int q = 0; q < kEqSub + 2; ++q) {
+            const int at = kEqSub * w + q;
+            const float P = Pt[(y + (at >> 5)) & 3][at & 31][lane];
+            R[q] = __fdiv_rn(P, s);              // a bin is divided by the mean before it
+            s = mean_step<decltype(fast)::value>(s, P);
+          }
+        };
+        if (__all_sync(0xffffffffu, fast_mean(s))) steps(std::true_type{});
+        else steps(std::false_type{});
+        uint32_t mine = 0;                       // lane i: bin jb + 1 + i
+#pragma unroll
+        for (int i = 0; i < kEqSub; ++i) {
+          const uint32_t word =
+              __ballot_sync(0xffffffffu, live && R[i + 1] > theta && R[i + 1] > R[i] && R[i + 1] > R[i + 2]);
+          if (lane == i) mine = word;
+        }
+        const int b = jb + 1 + lane;
+        if (lane < kEqSub && b <= bin_hi) bits[(int64_t)(b - bin_lo) * n_words + gw] = mine;
+      }
     }
     __syncthreads();
   }
@@ -243,39 +235,43 @@ __global__ void k_count(const uint32_t* __restrict__ bits, int n_bins, int n_wor
   if (lane == 0) counts[b] = c;
 }
 
-// Exclusive scan of counts[0..n) into counts (in place) and counts[n] = total; one block.
+// Exclusive scan of counts[0..n) into counts (in place) and counts[n] = total; one block.  Eight
+// consecutive counts per thread and turn: one turn for 8192 bins, where one count per thread took
+// eight turns of four barriers (10 us for 7800 bins).
 __global__ void __launch_bounds__(1024) k_scan(int64_t* counts, int n) {
+  constexpr int kPer = 8;
   __shared__ long long part[32];
-  __shared__ long long carry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < n; base += 1024) {
-    const int i = base + tid;
-    const long long v = i < n ? counts[i] : 0;
-    long long x = v;
+  long long carry = 0;
+  for (int base = 0; base < n; base += 1024 * kPer) {
+    const int i0 = base + tid * kPer;
+    long long v[kPer], sum = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) v[q] = i0 + q < n ? counts[i0 + q] : 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) sum += v[q];
+    long long x = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const long long u = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += u;
     }
+    __syncthreads();                             // the previous turn's sums are read
     if (lane == 31) part[warp] = x;
     __syncthreads();
-    if (warp == 0) {
-      long long y = part[lane];
+    long long y = part[lane], below = lane < warp ? y : 0;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long u = __shfl_up_sync(0xffffffffu, y, o);
-        if (lane >= o) y += u;
-      }
-      part[lane] = y;
+    for (int o = 16; o > 0; o >>= 1) {
+      below += __shfl_xor_sync(0xffffffffu, below, o);
+      y += __shfl_xor_sync(0xffffffffu, y, o);
     }
-    __syncthreads();
-    const long long excl = carry + (warp ? part[warp - 1] : 0) + x - v;
-    if (i < n) counts[i] = excl;
-    __syncthreads();
-    if (tid == 0) carry += part[31];
-    __syncthreads();
+    long long run = carry + below + x - sum;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      if (i0 + q < n) counts[i0 + q] = run;
+      run += v[q];
+    }
+    carry += y;
   }
   if (tid == 0) counts[n] = carry;
 }
