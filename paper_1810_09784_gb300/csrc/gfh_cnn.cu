@@ -464,7 +464,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 
 // ---- tcgen05 helpers (5th-generation tensor cores, accumulator in tensor memory) --------------------
 //
-// Operands live in shared memory K-major without swizzle: "core matrices" of 8 rows x 16 bytes
+// Operands without swizzle live in shared memory K-major: "core matrices" of 8 rows x 16 bytes
 // (8 bf16 along K); within a 16-wide K slice the two K halves are 128 bytes apart (leading byte
 // offset) and consecutive 8-row groups 256 bytes apart (stride byte offset).
 
@@ -484,6 +484,12 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo = 128u
                                               uint32_t sbo = 256u) {
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+}
+
+// Layout field of a descriptor whose operand was copied with the 64- or 128-byte swizzle (rows of
+// that many bytes, the 16-byte chunks of a row permuted by the address bits above them).
+__host__ __device__ constexpr uint64_t umma_swizzle(int row_bytes) {
+  return (row_bytes == 128 ? 2ull : 4ull) << 61;
 }
 
 // Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, both K-major, M x N.
@@ -568,15 +574,14 @@ __device__ __forceinline__ void async_proxy_fence() {
 // ---- forward layers and input gradients on tcgen05, TMA-fed and pipelined ---------------------------
 // Implicit GEMM out[m][n] = relu(bias[n] + sum_k A[m][k] W[n][k]): m = output pixel (b, y, x),
 // k = tap * CIN + ci (tap = 3 dy + dx), A[m][k] = in[b][y S + dy - 1][x S + dx - 1][ci] (zero outside
-// the image); tcgen05.mma M = 128 output pixels x N = COUT x K = 16 (8-channel chunks as 16-byte
-// rows of K-major core matrices, taps addressed through descriptor offsets into the staged input
-// rows).  The first layer runs on its image padded to 8 channels (CIN = 8): a K slice is then two
+// the image); tcgen05.mma M = 128 output pixels x N = COUT x K = 16 (K-major,
+// taps addressed through descriptor offsets into the staged input rows).  The first layer runs on its image padded to 8 channels (CIN = 8): a K slice is then two
 // taps of one row, one input entry apart.  One output row of CW <= 128 columns per tile, with the
 // roles of a block split so that copies, tensor-core work and the accumulator read-back of
 // different tiles overlap:
 //   warp 0      issues the tile's input copies with the tensor memory accelerator (TMA) into one of
-//               NS stage buffers: one box per (8-channel chunk, parity) of 3 input rows x NP
-//               entries x 16 bytes, zero-filled outside the image by the copy itself;
+//               NS stage buffers: one box per column parity of 3 input rows x NP entries (pixels)
+//               with all CIN channels, swizzled, zero-filled outside the image by the copy itself;
 //   warp 1      holds the tensor memory (four accumulators of COUT columns) and issues the tile's
 //               MMAs (tap by tap, K = 16 per MMA) once its stage is full and its accumulator free;
 //               their completion frees the stage and marks the accumulator full;
@@ -600,6 +605,15 @@ __device__ __forceinline__ void async_proxy_fence() {
 // rows) and G columns x0 - 1 + j (entry j); each parity class's 1, 2, 2 or 4 taps are its only
 // MMAs (a quarter of the multiply-adds of the zero-inserted form), into one accumulator per column
 // parity, and the tile's 2 CW output pixels are one contiguous run of the row.
+// What bounds it: the copies move about one row of a box per cycle and SM whatever its width, so boxes
+// of 16-byte rows (one per 8-channel chunk) held the wide layers at 1 byte in 4 or 8 of that rate: an
+// entry's channels are one 64- or 128-byte row now, in the swizzled K-major layout, whose pattern
+// follows the address bits, so that a tap's operand may start at any entry.  Then the MMAs' operand
+// reads (64 channels) and the epilogue's chain of waits (the input gradients of strided layers, whose
+// tiles are 2 to 8 MMAs: the mask words are fetched before the accumulator is waited for, and two
+// blocks share an SM where registers, tensor memory and two stages each allow).  Input gradient of
+// the first strided layer, 64 images: 190 -> 132 us; gradients of 256 images 5.50 -> 5.15 ms, logits
+// of 51 images 374 -> 354 us.
 constexpr int kTmaThreads = 320, kTmaGroupWarps = 4, kTmaAcc = 4, kTmaMaxStages = 4;
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -655,9 +669,23 @@ __device__ __forceinline__ bool group_any(int id, bool c) {
   return r != 0;
 }
 
-// Bytes of one TMA box in shared memory (rows x np entries x 16 bytes, 128-byte aligned).
-__host__ __device__ constexpr int tma_box_bytes(int np, int rows) {
-  return (rows * np * 16 + 127) / 128 * 128;
+// Bytes of one input entry (pixel) of k_conv_tma in shared memory: all its channels.
+__host__ __device__ constexpr int tma_entry_bytes(int cin) { return cin * 2; }
+
+// Bytes of one TMA box in shared memory: rows x np entries, aligned to the swizzle atom (1024 bytes
+// also where it is smaller), or to 128 bytes for the unswizzled 16-byte entries of the first layer.
+__host__ __device__ constexpr int tma_box_bytes(int cin, int np, int rows) {
+  const int align = cin == 8 ? 128 : 1024;
+  return (rows * np * tma_entry_bytes(cin) + align - 1) / align * align;
+}
+
+// Bytes the MMAs of the last stage can read past it (the dropped rows of a tile of under 128
+// columns).  The swizzled layers' over-read ends in the output staging that follows.
+__host__ __device__ constexpr int tma_over_read(int cin) { return cin == 8 ? 128 * 16 : 0; }
+
+// Blocks per SM that k_conv_tma is built for.
+__host__ __device__ constexpr int tma_blocks(int cin, int mode) {
+  return cin == 8 ? 3 : (cin == 32 && mode == 2 ? 2 : 1);
 }
 
 // Taps of the stride-2 input gradient's parity class c = 2 py + px (see k_conv_tma): tap index
@@ -669,9 +697,11 @@ __device__ __constant__ const int8_t kParityTaps[4][4][3] = {
     {{0, 0, 1}, {2, 0, 2}, {6, 1, 1}, {8, 1, 2}}};
 
 // The first layer (CIN == 8: the image padded to 8 channels, 51 KB of shared memory) keeps to 64
-// registers so that three blocks share an SM; the others are held to one block by shared memory.
+// registers so that three blocks share an SM, the first strided layer's input gradient to 96 for two
+// (its tiles are short on MMAs and long on the epilogue's chain of waits); the others are held to
+// one block by shared memory.
 template <int CIN, int COUT, int S, int MODE>
-__global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(const __grid_constant__ CUtensorMap tmap,
+__global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma(const __grid_constant__ CUtensorMap tmap,
                                                              const __grid_constant__ CUtensorMap omap,
                                                              const __nv_bfloat16* __restrict__ w,
                                                              const float* __restrict__ bias,
@@ -686,7 +716,7 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
   // taps (dx = 2 s, 2 s + 1) of one tap row, one entry apart, so a row takes 2 slices (the tap
   // dx = 3 has zero weights): 6 slices
   constexpr bool L1 = CIN == 8;
-  constexpr int KR = 9 * CIN, SPT = CIN / 16, QC = L1 ? 1 : CIN / 8;
+  constexpr int KR = 9 * CIN, SPT = CIN / 16, EB = tma_entry_bytes(CIN);
   constexpr int NSLW = L1 ? 6 : KR / 16;             // weight K slices
   constexpr int B_SL = COUT / 8 * 256;
   constexpr uint32_t IDESC = umma_idesc_bf16(128, COUT);
@@ -703,7 +733,7 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
   constexpr int ROWS = MODE == 2 ? 2 : 3;
   const int Ho = H / S, Wt = MODE == 2 ? H / 2 : Ho;   // output rows, columns per tile row
   const int CW = Wt > 128 ? 128 : Wt, NCB = Wt / CW, NP = CW + 2;
-  const int BOXB = tma_box_bytes(NP, ROWS), STAGE = QC * S * BOXB;
+  const int BOXB = tma_box_bytes(CIN, NP, ROWS), STAGE = S * BOXB;
   const int n_tiles = B * Ho * NCB;
   // tile t: image b, output row y, first column x0 of the block (of G columns in MODE 2)
   auto geo = [&](int t, int& b, int& y, int& x0) {
@@ -712,12 +742,15 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
     y = r / NCB;
     x0 = (r - y * NCB) * CW;
   };
-  const uint32_t sb32 = smem_u32(smem_tc), sa32 = sb32 + (uint32_t)(NSLW * B_SL);
+  // stages start on the swizzle atom
+  constexpr uint32_t AT = L1 ? 128u : 1024u;
+  const uint32_t sb32 = smem_u32(smem_tc);
+  const uint32_t sa32 = (sb32 + (uint32_t)(NSLW * B_SL) + AT - 1u) & ~(AT - 1u);
   // output staging of the two epilogue groups, after the stages and the MMA over-read pad, aligned
   // to the 1024-byte swizzle atom: 128 rows (pixels) of COUT bf16, 16-byte chunks swizzled as the
   // output tensor map's 128-byte (COUT = 64) or 64-byte (COUT = 32) mode expects
   constexpr int RB = COUT * 2;
-  const uint32_t ob32 = (sa32 + (uint32_t)(ns * STAGE + 128 * 16) + 1023u) & ~1023u;
+  const uint32_t ob32 = (sa32 + (uint32_t)(ns * STAGE + tma_over_read(CIN)) + 1023u) & ~1023u;
   auto fail = [&]() {
     s_fail = 1;
     atomicOr(flag, GFH_FLAG_TIMEOUT);
@@ -753,7 +786,7 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
   if (L1) {
     // the zero-weight tap dx = 3 of the last row reads one entry past its box: zeros, not stale
     // bits (0 x NaN would poison the pixel), in the slack no copy writes
-    for (int i = tid; i < (ns * STAGE + 128 * 16) / 16; i += blockDim.x)
+    for (int i = tid; i < (ns * STAGE + tma_over_read(CIN)) / 16; i += blockDim.x)
       *reinterpret_cast<int4*>(smem_tc + NSLW * B_SL + i * 16) = make_int4(0, 0, 0, 0);
   }
   if (tid == 0) {
@@ -778,20 +811,15 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
         if (s_fail) break;
         int b, y, x0;
         geo(t, b, y, x0);
-        mbar_expect_tx(&full[slot], (uint32_t)(QC * S * ROWS * 16 * NP));
+        mbar_expect_tx(&full[slot], (uint32_t)(S * ROWS * EB * NP));
         const uint32_t dst = sa32 + (uint32_t)(slot * STAGE);
-#pragma unroll
-        for (int q = 0; q < QC; ++q) {
-          if constexpr (MODE == 2) {
-            tma_load_4d(dst + (uint32_t)(q * BOXB), &tmap, &full[slot], 8 * q, x0 - 1, y >> 1, b);
-          } else if constexpr (S == 1) {
-            tma_load_4d(dst + (uint32_t)(q * BOXB), &tmap, &full[slot], 8 * q, x0 - 1, y - 1, b);
-          } else {   // parity 0: odd columns 2 (x0 + j) - 1; parity 1: even columns 2 (x0 + j)
-            tma_load_5d(dst + (uint32_t)(2 * q * BOXB), &tmap, &full[slot], 8 * q, 1, x0 - 1,
-                        2 * y - 1, b);
-            tma_load_5d(dst + (uint32_t)((2 * q + 1) * BOXB), &tmap, &full[slot], 8 * q, 0, x0,
-                        2 * y - 1, b);
-          }
+        if constexpr (MODE == 2) {
+          tma_load_4d(dst, &tmap, &full[slot], 0, x0 - 1, y >> 1, b);
+        } else if constexpr (S == 1) {
+          tma_load_4d(dst, &tmap, &full[slot], 0, x0 - 1, y - 1, b);
+        } else {   // parity 0: odd columns 2 (x0 + j) - 1; parity 1: even columns 2 (x0 + j)
+          tma_load_5d(dst, &tmap, &full[slot], 0, 1, x0 - 1, 2 * y - 1, b);
+          tma_load_5d(dst + (uint32_t)BOXB, &tmap, &full[slot], 0, 0, x0, 2 * y - 1, b);
         }
         ++issued;
       }
@@ -806,9 +834,11 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
         if (!mbar_wait(&full[slot], (uint32_t)(issued / ns) & 1u)) { fail(); break; }
         if (s_fail) break;
         tc_fence_after();
-        // descriptors: the stage's first entry plus the (chunk, parity, row, entry) offset of each
-        // tap and K slice, in 16-byte units (all offsets stay inside the 14-bit address field)
-        const uint64_t ad0 = umma_desc(sa32 + (uint32_t)(slot * STAGE), (uint32_t)(S * BOXB), 128u);
+        // descriptors: the stage's first entry plus the (parity, row, entry, channel) offset of each
+        // tap and K slice, in 16-byte units (all offsets stay inside the 14-bit address field);
+        // 8-entry groups follow each other
+        const uint64_t ad0 = umma_desc(sa32 + (uint32_t)(slot * STAGE), 16u, 8u * EB) |
+                             (L1 ? 0ull : umma_swizzle(EB));
         const uint32_t d_tmem = tmem + (uint32_t)(acc * NPAR * COUT);
         if constexpr (L1) {
           // K halves one entry apart: the descriptor's leading byte offset is 16 bytes
@@ -831,7 +861,7 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
 #pragma unroll
                 for (int sp = 0; sp < SPT; ++sp)
                   umma_bf16(d_tmem + (uint32_t)(px * COUT),
-                            ad0 + (uint64_t)((2 * sp * BOXB + (row * NP + jo) * 16) >> 4),
+                            ad0 + (uint64_t)(((row * NP + jo) * EB + sp * 32) >> 4),
                             bd0 + (uint64_t)(((tap * SPT + sp) * B_SL) >> 4), IDESC,
                             (k > 0 || sp > 0) ? 1u : 0u);
               }
@@ -846,7 +876,7 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
 #pragma unroll
           for (int sp = 0; sp < SPT; ++sp) {
             const int sl = tap * SPT + sp;
-            umma_bf16(d_tmem, ad0 + (uint64_t)(((2 * sp * S + par) * BOXB + (dy * NP + jo) * 16) >> 4),
+            umma_bf16(d_tmem, ad0 + (uint64_t)((par * BOXB + (dy * NP + jo) * EB + sp * 32) >> 4),
                       bd0 + (uint64_t)((sl * B_SL) >> 4), IDESC, sl > 0 ? 1u : 0u);
           }
         }
@@ -863,15 +893,21 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
     const uint32_t obuf = ob32 + (uint32_t)(grp * NPAR * 128 * RB);
     for (int i = grp, t = blockIdx.x + grp * gridDim.x; t < n_tiles; i += 2, t += 2 * gridDim.x) {
       const int acc = i % kTmaAcc;
+      int b, y, x0;
+      geo(t, b, y, x0);
+      const bool valid = p < CW;
+      const bool live = quarter * 32 < CW;           // warp-uniform: a row of the quarter is inside
+      // first output pixel of this lane; its ReLU mask is under way while the MMAs run
+      const int64_t m0 = ((int64_t)b * Ho + y) * Ho + NPAR * (x0 + p);
+      uint32_t mw[NPAR * BW];
+#pragma unroll
+      for (int k = 0; k < NPAR * BW; ++k)
+        mw[k] = (MODE != 0 && mbits && valid) ? __ldg(mbits + m0 * BW + k) : 0xffffffffu;
       const bool got = mbar_wait(&accf[acc], (uint32_t)(i / kTmaAcc) & 1u);
       if (!got) fail();
       // the whole group leaves together (it shares barriers), on its own timeout or another's
       if (group_any(1 + grp, !got || s_fail != 0)) break;
       tc_fence_after();
-      int b, y, x0;
-      geo(t, b, y, x0);
-      const bool valid = p < CW;
-      const bool live = quarter * 32 < CW;           // warp-uniform: a row of the quarter is inside
       // the staging buffer is free once the group's previous store has read it
       if (leader) bulk_wait_read0();
       group_bar(1 + grp);
@@ -879,7 +915,6 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
       for (int px = 0; px < NPAR; ++px) {
         // output pixel of this lane and parity: row q of the tile's staging (q = p, or 2 p + px)
         const int q = NPAR * p + px;
-        const int64_t m = ((int64_t)b * Ho + y) * Ho + NPAR * x0 + q;
         const int swz = COUT == 64 ? (q & 7) : ((q >> 1) & 3);
         uint32_t v[COUT];
         if (live) {
@@ -896,12 +931,7 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
           if (lane == 0) mbar_arrive(&acce[acc]);
         }
         if (live && valid) {
-          uint32_t mw[BW > 0 ? BW : 1], pw[BW > 0 ? BW : 1];
-#pragma unroll
-          for (int k = 0; k < BW; ++k) {
-            pw[k] = 0u;
-            mw[k] = (MODE != 0 && mbits) ? __ldg(mbits + m * BW + k) : 0xffffffffu;
-          }
+          uint32_t pw[BW] = {};
 #pragma unroll
           for (int c0 = 0; c0 < COUT; c0 += 8) {     // one 16-byte chunk: 8 channels
             uint32_t pk[4];
@@ -913,7 +943,7 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
                 pw[c0 >> 5] |= pos_bits(pk[j]) << ((c0 & 31) + 2 * j);
               }
             } else {
-              const uint32_t b8 = mw[c0 >> 5] >> (c0 & 31);
+              const uint32_t b8 = mw[px * BW + (c0 >> 5)] >> (c0 & 31);
 #pragma unroll
               for (int j = 0; j < 4; ++j)
                 pk[j] = keep_by_bits(
@@ -926,7 +956,7 @@ __global__ void __launch_bounds__(kTmaThreads, CIN == 8 ? 3 : 1) k_conv_tma(cons
           }
           if (MODE == 0 && bits) {
 #pragma unroll
-            for (int k = 0; k < BW; ++k) bits[m * BW + k] = pw[k];
+            for (int k = 0; k < BW; ++k) bits[(m0 + px) * BW + k] = pw[k];
           }
         }
       }
@@ -1549,29 +1579,33 @@ int conv_tma(const __nv_bfloat16* in, const __nv_bfloat16* w, const float* bias,
   if (!encode) return GFH_ERR_CUDA;
   alignas(64) CUtensorMap map;
   const cuuint64_t e = 2;                            // bf16 bytes
+  constexpr CUtensorMapSwizzle iswz = CIN == 8 ? CU_TENSOR_MAP_SWIZZLE_NONE
+                                      : CIN == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                                  : CU_TENSOR_MAP_SWIZZLE_128B;
+  static_assert(CIN == 8 || CIN == 32 || CIN == 64, "entries of 16, 64 or 128 bytes");
   CUresult r;
   if (MODE == 2) {
     const cuuint64_t hg = (cuuint64_t)H / 2;
     const cuuint64_t dims[4] = {(cuuint64_t)CIN, hg, hg, (cuuint64_t)B};
     const cuuint64_t strides[3] = {CIN * e, hg * CIN * e, hg * hg * CIN * e};
-    const cuuint32_t box[4] = {8, (cuuint32_t)NP, 2, 1}, es[4] = {1, 1, 1, 1};
+    const cuuint32_t box[4] = {CIN, (cuuint32_t)NP, 2, 1}, es[4] = {1, 1, 1, 1};
     r = encode(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)in, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, iswz,
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   } else if (S == 1) {
     const cuuint64_t dims[4] = {(cuuint64_t)CIN, (cuuint64_t)H, (cuuint64_t)H, (cuuint64_t)B};
     const cuuint64_t strides[3] = {CIN * e, (cuuint64_t)H * CIN * e, (cuuint64_t)H * H * CIN * e};
-    const cuuint32_t box[4] = {8, (cuuint32_t)NP, 3, 1}, es[4] = {1, 1, 1, 1};
+    const cuuint32_t box[4] = {CIN, (cuuint32_t)NP, 3, 1}, es[4] = {1, 1, 1, 1};
     r = encode(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)in, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, iswz,
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   } else {
     const cuuint64_t dims[5] = {(cuuint64_t)CIN, 2, (cuuint64_t)H / 2, (cuuint64_t)H, (cuuint64_t)B};
     const cuuint64_t strides[4] = {CIN * e, 2 * CIN * e, (cuuint64_t)H * CIN * e,
                                    (cuuint64_t)H * H * CIN * e};
-    const cuuint32_t box[5] = {8, 1, (cuuint32_t)NP, 3, 1}, es[5] = {1, 1, 1, 1, 1};
+    const cuuint32_t box[5] = {CIN, 1, (cuuint32_t)NP, 3, 1}, es[5] = {1, 1, 1, 1, 1};
     r = encode(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)in, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, iswz,
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   }
   if (r != CUDA_SUCCESS) return GFH_ERR_CUDA;
@@ -1596,13 +1630,19 @@ int conv_tma(const __nv_bfloat16* in, const __nv_bfloat16* w, const float* bias,
   // weights, stages, the over-read of the dropped MMA rows past the last stage, then (aligned to
   // 1024 bytes) the two epilogue groups' output staging of 128 rows x COUT bf16
   const size_t w_bytes = (size_t)(CIN == 8 ? 6 : 9 * CIN / 16) * (COUT / 8 * 256);
-  const size_t stage = (size_t)(CIN / 8) * S * tma_box_bytes(NP, ROWS);
+  const size_t stage = (size_t)S * tma_box_bytes(CIN, NP, ROWS);
   const size_t o_bytes = 2 * NPAR * 128 * COUT * 2 + 1024;
+  static_assert(CIN == 8 || 2 * NPAR * 128 * COUT * 2 >= 128 * CIN * 2, "the staging takes the over-read");
+  // the shared memory of one of the blocks the kernel is built for, if two stages fit in it
+  constexpr int want = tma_blocks(CIN, MODE);
   const size_t room = kMaxSmemBytes - fa.sharedSizeBytes - 1024;
+  const size_t share = std::min(room, kSmemPerSm / want - fa.sharedSizeBytes - 1024);
+  const size_t fixed = w_bytes + tma_over_read(CIN) + o_bytes;
   int ns = kTmaMaxStages;
-  while (ns >= 2 && w_bytes + ns * stage + 128 * 16 + o_bytes > room) --ns;
+  while (ns > 2 && fixed + ns * stage > share) --ns;
+  while (ns >= 2 && fixed + ns * stage > room) --ns;
   if (ns < 2) return GFH_ERR_SIZE;
-  const size_t smem = w_bytes + ns * stage + 128 * 16 + o_bytes;
+  const size_t smem = fixed + ns * stage;
   GFH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   GFH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   const int regs = std::max(1, (fa.numRegs + 7) / 8 * 8);
