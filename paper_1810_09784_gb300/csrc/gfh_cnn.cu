@@ -1000,17 +1000,22 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
 // fit): block (chunk, dy) keeps the taps (dy, 0..2) and G is read once per tap row.  A tile is
 // WT_ROWS output rows x 64 columns of one image, its K-steps 16 output pixels of one row.  Warp 0
 // copies each tile with the tensor memory accelerator into one of WT_STAGES stages:
-//   G: one box per 8-co chunk c of WT_ROWS rows x 64 pixels  -> [c][row][64 px] x 16 bytes;
-//   X: one box per 8-ci chunk c (and column parity for S = 2) of the input rows the tile's taps
-//      read, x NP entries, zero-filled outside the image -> [c][par][row][NP] x 16 bytes: rows
+//   G: one box of WT_ROWS rows x 64 pixels, swizzled          -> [row][64 px] x COUT;
+//   X: one box (per column parity for S = 2) of the input rows the tile's taps read, x NP entries,
+//      swizzled, zero-filled outside the image -> [par][row][NP] x CIN: rows
 //      (y0 + r) S + dy - 1 for DYB = 1, or all rows y0 S - 1 .. (y0 + WT_ROWS - 1) S + 1 for
 //      DYB = 3 (tap row dy of output row r is row r S + dy of the box); entry j of parity 0 is
 //      input column x0 S - 1 + j (S = 1), 2 (x0 + j) - 1 (S = 2), of parity 1 column 2 (x0 + j).
 // Warp 1 issues the MMAs once a stage is full and frees it with their commit.  Tap dx's B operand is
-// the same array started dx entries later (S = 1) or in the other parity (S = 2); for CIN = 8 the
-// three taps are one MMA of N = 24 whose N-adjacent core matrices are one entry (16 bytes) apart.
-// Core matrices: 8 pixels x 16 bytes, K-adjacent ones 128 bytes apart (the descriptor's leading
-// byte offset), M/N-adjacent ones one chunk apart (its stride byte offset).  In the blocks whose
+// the same array started dx entries later (S = 1: the three taps) or the other parity (S = 2: dx = 1,
+// beside dx = 0 and 2); taps of one array are one MMA of N = 3 CIN or 2 CIN whose N-adjacent pieces
+// of CIN channels lie one entry apart (the descriptor's leading byte offset in the swizzled layouts,
+// whose 8-pixel groups along K are the stride byte offset apart; the padded image's 16-byte
+// entries have no swizzle, and the two fields the other way round).
+// What bounds it: the copies' box rows (one of 16 bytes per pixel and 8 channels before, one of 64 or
+// 128 bytes per pixel now) and the MMAs' operand reads from shared memory (the 64 gradient rows were
+// read again for each of a row's three taps).  Gradients of 256 images 5.15 -> 4.48 ms.
+// In the blocks whose
 // tiles cover every output pixel once (all blocks for DYB = 3, the dy = 1 ones for DYB = 1),
 // warps 2-3 also sum each staged G tile over its pixels
 // (the bias gradient) before they release the stage with the MMA commit.  At the end the four
@@ -1036,16 +1041,15 @@ __device__ __forceinline__ int wgrad_row_of_lane(int lane) {
 
 template <int CIN, int COUT, int S, int DYB>
 struct WgradTc {
-  static constexpr int NP = S == 1 ? 66 : 65;                         // entries per (chunk, parity, row)
+  static constexpr int NP = S == 1 ? 66 : 65;                         // entries per (parity, row)
   static constexpr int XROWS = DYB == 1 ? WT_ROWS : (WT_ROWS - 1) * S + 3;   // input rows per tile
-  static constexpr int GBOX = WT_ROWS * 64 * 16;                      // one G box
-  static constexpr int XBOX = (XROWS * NP * 16 + 127) / 128 * 128;    // one X box (128-aligned)
-  static constexpr int GB = (COUT / 8) * GBOX;
-  static constexpr int XB = (CIN / 8) * S * XBOX;
-  static constexpr int STAGE = (GB + XB + 127) / 128 * 128;
-  // A reads 8 co chunks (64 rows): the padding chunks past G reach into X or the next stage
-  static constexpr int PAD = (64 - COUT) / 8 * GBOX;
-  static constexpr int SMEM = WT_STAGES * STAGE + PAD;
+  static constexpr int GE = COUT * 2, XE = CIN * 2;                   // bytes of a G pixel, an X entry
+  static constexpr int GB = WT_ROWS * 64 * GE;                        // the G box
+  static constexpr int XBOX = (XROWS * NP * XE + 1023) / 1024 * 1024; // one X box (on the swizzle atom)
+  static constexpr int XB = S * XBOX;
+  static constexpr int STAGE = GB + XB;
+  static constexpr int SMEM = WT_STAGES * STAGE + 1024;               // stages start on the atom
+  static_assert(GB % 1024 == 0 && (COUT == 32 || COUT == 64), "G pixels of 64 or 128 bytes");
 };
 
 template <int CIN, int COUT, int S, int DYB>
@@ -1056,9 +1060,10 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
                                                           int chunks, unsigned int* flag) {
   using T = WgradTc<CIN, COUT, S, DYB>;
   constexpr int NP = T::NP;
-  constexpr int NMMA = CIN == 8 ? 3 * CIN : CIN;
-  constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                             ((uint32_t)(NMMA >> 3) << 17) | ((uint32_t)(64 >> 4) << 24);
+  auto idesc = [](int n) {                           // M = 64 x N, both operands MN-major
+    return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) |
+           ((uint32_t)(64 >> 4) << 24);
+  };
   constexpr int NACC = DYB * 3 * CIN;               // accumulator columns: (dy, dx, ci)
   constexpr uint32_t TCOLS = NACC <= 128 ? 128 : (NACC <= 256 ? 256 : 512);
   static_assert(NACC <= 512, "tensor memory holds the block's taps");
@@ -1075,7 +1080,7 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
   const int Ho = H / S;
   const int tiles_per_img = (Ho / WT_ROWS) * (Ho / 64);
   const int n_tiles = B * tiles_per_img;
-  const uint32_t s32 = smem_u32(smem_w);
+  const uint32_t align = (0u - smem_u32(smem_w)) & 1023u, s32 = smem_u32(smem_w) + align;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tslot)), "r"(TCOLS));
@@ -1108,22 +1113,17 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
       const int rg = rem / (Ho / 64), cb = rem - rg * (Ho / 64);
       const int y0 = rg * WT_ROWS, x0 = cb * 64;
       const uint32_t st = s32 + (uint32_t)(slot * T::STAGE);
-      mbar_expect_tx(&full[slot], (uint32_t)(T::GB + (CIN / 8) * S * T::XROWS * NP * 16));
-#pragma unroll
-      for (int c = 0; c < COUT / 8; ++c)
-        tma_load_4d(st + (uint32_t)(c * T::GBOX), &gmap, &full[slot], 8 * c, x0, y0, b);
-#pragma unroll
-      for (int c = 0; c < CIN / 8; ++c) {
-        const uint32_t xs = st + (uint32_t)(T::GB + c * S * T::XBOX);
-        // first input row: y0 S - 1 (all tap rows), or (y0 S) + dy - 1 for one tap row, whose
-        // S = 2 rows 2 (y0 + r) + dy - 1 come through the row traversal stride of 2
-        const int yr = y0 * S - 1 + (DYB == 1 ? dy1 : 0);
-        if constexpr (S == 1) {
-          tma_load_4d(xs, &xmap, &full[slot], 8 * c, x0 - 1, yr, b);
-        } else {
-          tma_load_5d(xs, &xmap, &full[slot], 8 * c, 1, x0 - 1, yr, b);
-          tma_load_5d(xs + (uint32_t)T::XBOX, &xmap, &full[slot], 8 * c, 0, x0, yr, b);
-        }
+      mbar_expect_tx(&full[slot], (uint32_t)(T::GB + S * T::XROWS * NP * T::XE));
+      tma_load_4d(st, &gmap, &full[slot], 0, x0, y0, b);
+      const uint32_t xs = st + (uint32_t)T::GB;
+      // first input row: y0 S - 1 (all tap rows), or (y0 S) + dy - 1 for one tap row, whose
+      // S = 2 rows 2 (y0 + r) + dy - 1 come through the row traversal stride of 2
+      const int yr = y0 * S - 1 + (DYB == 1 ? dy1 : 0);
+      if constexpr (S == 1) {
+        tma_load_4d(xs, &xmap, &full[slot], 0, x0 - 1, yr, b);
+      } else {
+        tma_load_5d(xs, &xmap, &full[slot], 0, 1, x0 - 1, yr, b);
+        tma_load_5d(xs + (uint32_t)T::XBOX, &xmap, &full[slot], 0, 0, x0, yr, b);
       }
       ++issued;
     }
@@ -1142,9 +1142,9 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
       for (int r = 0; r < WT_ROWS; ++r)
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
-          // A: [c][row][64 px]; B: [c][par][row][NP]
+          // A: [row][64 px], its 8-pixel groups one after the other (M rows past COUT read G again)
           const uint64_t ad =
-              umma_desc(st + (uint32_t)((r * 64 + ks * 16) * 16), 128u, (uint32_t)T::GBOX);
+              umma_desc(st + (uint32_t)((r * 64 + ks * 16) * T::GE), 0u, 8u * T::GE) | umma_swizzle(T::GE);
           // every accumulator column group starts with the block's first K-step
           const uint32_t acc_on = (issued > 0 || r > 0 || ks > 0) ? 1u : 0u;
 #pragma unroll
@@ -1152,19 +1152,17 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
             // box row of this output row's tap row, accumulator columns of the tap row
             const int xr = DYB == 1 ? r : r * S + d;
             const uint32_t tcol = tmem + (uint32_t)(d * 3 * CIN);
+            // B: [par][row][NP]; the taps of one parity are one entry apart
+            const uint32_t b_addr = st + (uint32_t)(T::GB + (xr * NP + ks * 16) * T::XE);
             if constexpr (CIN == 8) {
-              const uint32_t b_addr = st + (uint32_t)(T::GB + (xr * NP + ks * 16) * 16);
-              umma_bf16(tcol, ad, umma_desc(b_addr, 128u, 16u), IDESC, acc_on);
+              umma_bf16(tcol, ad, umma_desc(b_addr, 128u, 16u), idesc(3 * CIN), acc_on);
             } else {
-#pragma unroll
-              for (int dx = 0; dx < 3; ++dx) {
-                const int par = S == 1 ? 0 : (dx == 1 ? 1 : 0);
-                const int jo = S == 1 ? dx : (dx == 2 ? 1 : 0);
-                const uint32_t b_addr =
-                    st + (uint32_t)(T::GB + par * T::XBOX + (xr * NP + ks * 16 + jo) * 16);
-                umma_bf16(tcol + (uint32_t)(dx * CIN), ad,
-                          umma_desc(b_addr, 128u, (uint32_t)(S * T::XBOX)), IDESC, acc_on);
-              }
+              umma_bf16(tcol, ad, umma_desc(b_addr, (uint32_t)T::XE, 8u * T::XE) | umma_swizzle(T::XE),
+                        idesc((S == 1 ? 3 : 2) * CIN), acc_on);
+              if constexpr (S == 2)                    // dx = 1: the other parity
+                umma_bf16(tcol + 2u * CIN, ad,
+                          umma_desc(b_addr + (uint32_t)T::XBOX, 0u, 8u * T::XE) | umma_swizzle(T::XE),
+                          idesc(CIN), acc_on);
             }
           }
         }
@@ -1187,9 +1185,10 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
         break;
       }
       if (__shfl_sync(0xffffffffu, s_fail, 0)) break;
-      const unsigned char* g = smem_w + slot * T::STAGE + c * T::GBOX;
+      const unsigned char* g = smem_w + align + slot * T::STAGE;
       for (int px = j; px < WT_ROWS * 64; px += TPC) {
-        const uint4 w4 = *reinterpret_cast<const uint4*>(g + px * 16);
+        const int swz = COUT == 64 ? (px & 7) : ((px >> 1) & 3);
+        const uint4 w4 = *reinterpret_cast<const uint4*>(g + px * T::GE + ((c ^ swz) << 4));
         const uint32_t wv[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -1233,7 +1232,8 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
   for (int d = 0; d < DYB; ++d)
     for (int dx = 0; dx < 3; ++dx)
       for (int c0 = 0; c0 < CIN; c0 += 16) {
-        const int tap = (DYB == 1 ? dy1 : d) * 3 + dx;
+        // accumulator columns dx of a tap row: taps 0, 1, 2, or with stride 2 0, 2, 1
+        const int tap = (DYB == 1 ? dy1 : d) * 3 + (S == 2 ? (3 - dx) % 3 : dx);
         uint32_t v[16];
         if (have)
           tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((d * 3 + dx) * CIN + c0), v);
@@ -1564,6 +1564,12 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
+// Swizzle of the pixels of `c` bf16 channels in shared memory: 64- or 128-byte rows; the 16-byte
+// rows of the padded image have none.
+constexpr CUtensorMapSwizzle swizzle_of(int c) {
+  return c == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : c == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE;
+}
+
 // Launch of k_conv_tma (see there): the input view's tensor map, the stage count that fits in shared
 // memory next to the weights (4, 3 or 2), persistent blocks.
 template <int CIN, int COUT, int S, int MODE>
@@ -1579,10 +1585,7 @@ int conv_tma(const __nv_bfloat16* in, const __nv_bfloat16* w, const float* bias,
   if (!encode) return GFH_ERR_CUDA;
   alignas(64) CUtensorMap map;
   const cuuint64_t e = 2;                            // bf16 bytes
-  constexpr CUtensorMapSwizzle iswz = CIN == 8 ? CU_TENSOR_MAP_SWIZZLE_NONE
-                                      : CIN == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
-                                                  : CU_TENSOR_MAP_SWIZZLE_128B;
-  static_assert(CIN == 8 || CIN == 32 || CIN == 64, "entries of 16, 64 or 128 bytes");
+  constexpr CUtensorMapSwizzle iswz = swizzle_of(CIN);
   CUresult r;
   if (MODE == 2) {
     const cuuint64_t hg = (cuuint64_t)H / 2;
@@ -1699,8 +1702,8 @@ size_t grad_partial_floats(int B) {
   return most;
 }
 
-// Tensor maps of the weight-gradient kernel's operands: G (COUT, Ho, Ho, B) in boxes of 8 co x 64
-// pixels x WT_ROWS rows; X (CIN, H, H, B) in boxes of 8 ci x NP entries x XROWS rows, or for S = 2
+// Tensor maps of the weight-gradient kernel's operands: G (COUT, Ho, Ho, B) in boxes of 64
+// pixels x WT_ROWS rows; X (CIN, H, H, B) in boxes of NP entries x XROWS rows, or for S = 2
 // the column-parity view (CIN, 2, H/2, H, B), its rows traversed with a stride of 2 for one tap row.
 template <int CIN, int COUT, int S, int DYB>
 int wgrad_maps(const __nv_bfloat16* G, const __nv_bfloat16* in, int B, int H, CUtensorMap* gmap,
@@ -1712,9 +1715,9 @@ int wgrad_maps(const __nv_bfloat16* G, const __nv_bfloat16* in, int B, int H, CU
   {
     const cuuint64_t dims[4] = {(cuuint64_t)COUT, Ho, Ho, (cuuint64_t)B};
     const cuuint64_t strides[3] = {COUT * e, Ho * COUT * e, Ho * Ho * COUT * e};
-    const cuuint32_t box[4] = {8, 64, WT_ROWS, 1}, es[4] = {1, 1, 1, 1};
+    const cuuint32_t box[4] = {COUT, 64, WT_ROWS, 1}, es[4] = {1, 1, 1, 1};
     if (encode(gmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)G, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(COUT),
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return GFH_ERR_CUDA;
   }
@@ -1723,19 +1726,19 @@ int wgrad_maps(const __nv_bfloat16* G, const __nv_bfloat16* in, int B, int H, CU
   if (S == 1) {
     const cuuint64_t dims[4] = {(cuuint64_t)CIN, h, h, (cuuint64_t)B};
     const cuuint64_t strides[3] = {CIN * e, h * CIN * e, h * h * CIN * e};
-    const cuuint32_t box[4] = {8, (cuuint32_t)NP, XROWS, 1}, es[4] = {1, 1, 1, 1};
+    const cuuint32_t box[4] = {CIN, (cuuint32_t)NP, XROWS, 1}, es[4] = {1, 1, 1, 1};
     r = encode(xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)in, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(CIN),
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   } else {
     const cuuint64_t dims[5] = {(cuuint64_t)CIN, 2, h / 2, h, (cuuint64_t)B};
     const cuuint64_t strides[4] = {CIN * e, 2 * CIN * e, h * CIN * e, h * h * CIN * e};
     // one tap row: rows 2 (y0 + r) + dy - 1 (stride 2); all tap rows: XROWS consecutive rows
     const cuuint32_t rstride = DYB == 1 ? 2 : 1;
-    const cuuint32_t box[5] = {8, 1, (cuuint32_t)NP, (cuuint32_t)XROWS * rstride, 1},
+    const cuuint32_t box[5] = {CIN, 1, (cuuint32_t)NP, (cuuint32_t)XROWS * rstride, 1},
                      es[5] = {1, 1, 1, rstride, 1};
     r = encode(xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)in, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(CIN),
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   }
   return r == CUDA_SUCCESS ? GFH_OK : GFH_ERR_CUDA;
