@@ -536,21 +536,27 @@ __device__ __forceinline__ void umma_commit(uint32_t e, uint64_t* mbar) {
       "r"(smem_u32(mbar)));
 }
 
+__device__ __forceinline__ bool mbar_try(uint64_t* mbar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(smem_u32(mbar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
 // Waits for the phase of parity `parity` of the mbarrier, at most `budget` cycles (default about a
-// second at the maximum clock).
-__device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity,
+// second at the maximum clock) and no longer than until *stop is set (nullable: another role of the
+// block gave up).  A phase that is over already costs one test: clock and flag are read after it.
+__device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, const volatile int* stop = nullptr,
                                           long long budget = 2000000000ll) {
+  if (mbar_try(mbar, parity)) return true;
   const long long t0 = clock64();
   for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(smem_u32(mbar)), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (clock64() - t0 > budget) return false;
+    if (mbar_try(mbar, parity)) return true;
+    if ((stop && *stop) || clock64() - t0 > budget) return false;
   }
 }
 
@@ -560,7 +566,7 @@ __global__ void k_wait_unsignalled(long long budget, unsigned int* flag) {
   __shared__ __align__(8) uint64_t mbar;
   if (threadIdx.x == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar)), "r"(1));
   __syncthreads();
-  if (threadIdx.x == 0 && !mbar_wait(&mbar, 0, budget)) atomicOr(flag, GFH_FLAG_TIMEOUT);
+  if (threadIdx.x == 0 && !mbar_wait(&mbar, 0, nullptr, budget)) atomicOr(flag, GFH_FLAG_TIMEOUT);
 }
 
 // 16 consecutive 32-bit accumulator columns of the warp's 32 lanes into v[0..15]; the values are
@@ -833,8 +839,7 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
       for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         const int slot = issued % ns, use = issued / ns;
-        if (use > 0 && !mbar_wait(&empty[slot], (uint32_t)(use - 1) & 1u)) { fail(); break; }
-        if (s_fail) break;
+        if (use > 0 && !mbar_wait(&empty[slot], (uint32_t)(use - 1) & 1u, &s_fail)) { fail(); break; }
         int b, y, x0;
         geo(t, b, y, x0);
         mbar_expect_tx(&full[slot], (uint32_t)(S * ROWS * EB * NP));
@@ -856,10 +861,9 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
       const UmmaDesc bd0 = umma_desc(sb32);
       for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         const int slot = issued % ns, acc = issued % kTmaAcc;
-        bool got = issued < kTmaAcc || mbar_wait(&acce[acc], (uint32_t)(issued / kTmaAcc - 1) & 1u);
-        got = got && mbar_wait(&full[slot], (uint32_t)(issued / ns) & 1u);
+        bool got = issued < kTmaAcc || mbar_wait(&acce[acc], (uint32_t)(issued / kTmaAcc - 1) & 1u, &s_fail);
+        got = got && mbar_wait(&full[slot], (uint32_t)(issued / ns) & 1u, &s_fail);
         if (!__all_sync(0xffffffffu, got)) { fail(); break; }
-        if (__any_sync(0xffffffffu, s_fail != 0)) break;
         tc_fence_after();
         // descriptors: the stage's first entry plus the (parity, row, entry, channel) offset of each
         // tap and K slice, in 16-byte units (all offsets stay inside the 14-bit address field);
@@ -930,14 +934,13 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
 #pragma unroll
       for (int k = 0; k < NPAR * BW; ++k)
         mw[k] = (MODE != 0 && mbits && valid) ? __ldg(mbits + m0 * BW + k) : 0xffffffffu;
-      const bool got = mbar_wait(&accf[acc], (uint32_t)(i / kTmaAcc) & 1u);
+      const bool got = mbar_wait(&accf[acc], (uint32_t)(i / kTmaAcc) & 1u, &s_fail);
       if (!got) fail();
-      // the whole group leaves together (it shares barriers), on its own timeout or another's
-      if (group_any(1 + grp, !got || s_fail != 0)) break;
-      tc_fence_after();
       // the staging buffer is free once the group's previous store has read it
       if (leader) bulk_wait_read0();
-      group_bar(1 + grp);
+      // the whole group leaves together (it shares barriers), on its own timeout or another's
+      if (group_any(1 + grp, !got)) break;
+      tc_fence_after();
 #pragma unroll
       for (int px = 0; px < NPAR; ++px) {
         // output pixel of this lane and parity: row q of the tile's staging (q = p, or 2 p + px)
@@ -1131,7 +1134,7 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&xmap)) : "memory");
     for (int q = chunk; q < n_tiles; q += chunks) {
       const int slot = issued % WT_STAGES, use = issued / WT_STAGES;
-      if (use > 0 && !mbar_wait(&empty[slot], (uint32_t)(use - 1) & 1u)) {
+      if (use > 0 && !mbar_wait(&empty[slot], (uint32_t)(use - 1) & 1u, &s_fail)) {
         s_fail = 1;
         atomicOr(flag, GFH_FLAG_TIMEOUT);
         break;
@@ -1158,12 +1161,11 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
     const uint32_t e = elect_one(), tm = __shfl_sync(0xffffffffu, tmem, 0);
     for (int q = chunk; q < n_tiles; q += chunks) {
       const int slot = issued % WT_STAGES;
-      if (!__all_sync(0xffffffffu, mbar_wait(&full[slot], (uint32_t)(issued / WT_STAGES) & 1u))) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&full[slot], (uint32_t)(issued / WT_STAGES) & 1u, &s_fail))) {
         s_fail = 1;
         atomicOr(flag, GFH_FLAG_TIMEOUT);
         break;
       }
-      if (__any_sync(0xffffffffu, s_fail != 0)) break;
       tc_fence_after();
       const uint32_t st = s32 + (uint32_t)(slot * T::STAGE);
 #pragma unroll
@@ -1207,12 +1209,11 @@ __global__ void __launch_bounds__(WT_THREADS) k_wgrad_tma(const __grid_constant_
     int n = 0;
     for (int q = chunk; q < n_tiles; q += chunks, ++n) {
       const int slot = n % WT_STAGES;
-      const bool got = mbar_wait(&full[slot], (uint32_t)(n / WT_STAGES) & 1u);
+      const bool got = mbar_wait(&full[slot], (uint32_t)(n / WT_STAGES) & 1u, &s_fail);
       if (!__all_sync(0xffffffffu, got)) {
         if (lane == 0) { s_fail = 1; atomicOr(flag, GFH_FLAG_TIMEOUT); }
         break;
       }
-      if (__shfl_sync(0xffffffffu, s_fail, 0)) break;
       const unsigned char* g = smem_w + align + slot * T::STAGE;
       for (int px = j; px < WT_ROWS * 64; px += TPC) {
         const int swz = COUT == 64 ? (px & 7) : ((px >> 1) & 3);
