@@ -445,20 +445,32 @@ __global__ void __launch_bounds__(1024) k_line_scores(const uint32_t* __restrict
 
 // ---- tensor-core helpers --------------------------------------------------------------------------
 
-// Bit 0 / bit 1: whether the low / high bf16 half of w is positive (where a ReLU passes gradient).
-__device__ __forceinline__ uint32_t pos_bits(uint32_t w) {
-  const uint32_t lo = w & 0xffffu, hi = w >> 16;
-  return (uint32_t)((lo & 0x7fffu) != 0u && !(lo & 0x8000u)) |
-         ((uint32_t)((hi & 0x7fffu) != 0u && !(hi & 0x8000u)) << 1);
+// ReLU mask of 32 channels in one word: bit j for channel 2 j, bit 16 + j for channel 2 j + 1, as the
+// two halves of a bf16 pair shift into place together (3 instructions a pair, 10 bit by bit).
+// Bits of pair j (two bf16, neither negative nor NaN): a half that is not 0 carries into its top bit.
+__device__ __forceinline__ uint32_t pos_bits(uint32_t w, int j) {
+  return ((w + 0x7fff7fffu) >> (15 - j)) & (0x10001u << j);
 }
 
-// Keeps each bf16 half of g whose bit (0: low half, 1: high half) is set in b2.
-__device__ __forceinline__ uint32_t keep_by_bits(uint32_t g, uint32_t b2) {
-  return g & (((b2 & 1u) ? 0xffffu : 0u) | ((b2 & 2u) ? 0xffff0000u : 0u));
+// Keeps each bf16 half of pair j whose bit is set.
+__device__ __forceinline__ uint32_t keep_by_bits(uint32_t g, uint32_t bits, int j) {
+  return g & (((bits >> j) & 0x10001u) * 0xffffu);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// bf16 of max(lo + blo, 0) and max(hi + bhi, 0): one paired add, one conversion, one paired maximum
+// (rounding keeps the order, so the maximum may follow it; a NaN becomes 0 either way).
+__device__ __forceinline__ uint32_t bias_relu_bf16(uint32_t lo, uint32_t hi, float2 b) {
+  float x, y;
+  asm("{\n.reg .b64 v, b, r;\nmov.b64 v, {%2, %3};\nmov.b64 b, {%4, %5};\nadd.rn.f32x2 r, v, b;\n"
+      "mov.b64 {%0, %1}, r;\n}\n"
+      : "=f"(x), "=f"(y)
+      : "r"(lo), "r"(hi), "f"(b.x), "f"(b.y));
+  const __nv_bfloat162 v = __hmax2(__floats2bfloat162_rn(x, y), __nv_bfloat162(0.f, 0.f));
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
@@ -758,7 +770,7 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
   __shared__ __align__(8) uint64_t full[kTmaMaxStages], empty[kTmaMaxStages], accf[kTmaAcc],
       acce[kTmaAcc];
   __shared__ uint32_t tslot;
-  __shared__ float sbias[COUT];
+  __shared__ __align__(16) float sbias[COUT];
   __shared__ volatile int s_fail;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   // MODE 2: Ho = H output rows, each with two column parities of Hg = H / 2 columns
@@ -968,17 +980,16 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
             if (MODE == 0) {
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
-                pk[j] = pack_bf16(fmaxf(__uint_as_float(v[c0 + 2 * j]) + sbias[c0 + 2 * j], 0.f),
-                                  fmaxf(__uint_as_float(v[c0 + 2 * j + 1]) + sbias[c0 + 2 * j + 1], 0.f));
-                pw[c0 >> 5] |= pos_bits(pk[j]) << ((c0 & 31) + 2 * j);
+                pk[j] = bias_relu_bf16(v[c0 + 2 * j], v[c0 + 2 * j + 1],
+                                       *reinterpret_cast<const float2*>(sbias + c0 + 2 * j));
+                pw[c0 >> 5] |= pos_bits(pk[j], (c0 & 31) / 2 + j);
               }
             } else {
-              const uint32_t b8 = mw[px * BW + (c0 >> 5)] >> (c0 & 31);
 #pragma unroll
               for (int j = 0; j < 4; ++j)
                 pk[j] = keep_by_bits(
                     pack_bf16(__uint_as_float(v[c0 + 2 * j]), __uint_as_float(v[c0 + 2 * j + 1])),
-                    b8 >> (2 * j));
+                    mw[px * BW + (c0 >> 5)], (c0 & 31) / 2 + j);
             }
             const uint32_t dst = obuf + (uint32_t)(q * RB + (((c0 >> 3) ^ swz) << 4));
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(pk[0]),
