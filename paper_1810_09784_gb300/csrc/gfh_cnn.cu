@@ -628,7 +628,11 @@ __device__ __forceinline__ void async_proxy_fence() {
 //               with all CIN channels, swizzled, zero-filled outside the image by the copy itself;
 //   warp 1      holds the tensor memory (four accumulators of COUT columns) and, all its lanes
 //               together, issues the tile's MMAs (tap by tap, K = 16 per MMA) once its stage is full and its accumulator free;
-//               their completion frees the stage and marks the accumulator full;
+//               their completion frees the stage and marks the accumulator full.  MMAs of N = 64
+//               (32) are issued at the rate of their operand reads, 48 (41) cycles each by the
+//               warp's clock, with no queue to speak of, and 750 cycles of waits, fences and commits
+//               per tile left the tensor core idle: in the layers that this bounds a second MMA
+//               warp (warp 10) takes every other tile;
 //   warps 2-9   two groups of four that take alternate tiles: read the tile's accumulator back
 //               (warp w: lanes 32 (w % 4) .., all COUT columns, one wait for all the loads) and
 //               release it, add the bias and apply the ReLU (MODE 0; with `bits`, also store one
@@ -732,6 +736,20 @@ __host__ __device__ constexpr int tma_blocks(int cin, int mode) {
   return cin == 8 ? 3 : (cin == 32 && mode == 2 ? 2 : 1);
 }
 
+// Its MMA warps: a second one for the 64-channel stride-1 forms, whose tensor-core work per tile (36
+// MMAs, 12 to 24 in MODE 2) is what bounds them (256 images: 147 -> 114 us, 180 -> 137 us, MODE 2
+// 280 -> 203 us).  The others did not gain: they wait for their copies (two or three stages fit) or
+// for the epilogue.  With two warps the number of stages must be even: a stage then always meets the
+// same warp, as its mbarrier's parity wants (a warp two phases ahead of a barrier would take the
+// phase before for the one it waits for).
+__host__ __device__ constexpr int tma_mma_warps(int cin, int cout, int s) {
+  return cin == 64 && cout == 64 && s == 1 ? 2 : 1;
+}
+__host__ __device__ constexpr int tma_threads(int cin, int cout, int s) {
+  return kTmaThreads + 32 * (tma_mma_warps(cin, cout, s) - 1);
+}
+static_assert(kTmaAcc % 2 == 0, "an accumulator always meets the same MMA warp");
+
 // Taps of the stride-2 input gradient's parity class c = 2 py + px (see k_conv_tma): tap index
 // 3 dy + dx, box row (0: G row y / 2, 1: the next) and entry offset jo; class c has 1, 2, 2, 4 taps.
 __device__ __constant__ const int8_t kParityTaps[4][4][3] = {
@@ -745,7 +763,7 @@ __device__ __constant__ const int8_t kParityTaps[4][4][3] = {
 // (its tiles are short on MMAs and long on the epilogue's chain of waits); the others are held to
 // one block by shared memory.
 template <int CIN, int COUT, int S, int MODE>
-__global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma(const __grid_constant__ CUtensorMap tmap,
+__global__ void __launch_bounds__(tma_threads(CIN, COUT, S), tma_blocks(CIN, MODE)) k_conv_tma(const __grid_constant__ CUtensorMap tmap,
                                                              const __grid_constant__ CUtensorMap omap,
                                                              const __nv_bfloat16* __restrict__ w,
                                                              const float* __restrict__ bias,
@@ -844,7 +862,9 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tslot;
-  int issued = 0;                                    // stages (warp 0) or tiles (warp 1) issued
+  int issued = 0;        // stages (warp 0) or tiles up to the warp's last one (MMA warps) issued
+  constexpr int MW = tma_mma_warps(CIN, COUT, S);
+  const bool second = MW == 2 && warp == kTmaThreads / 32;   // the second MMA warp
 
   if (warp == 0) {
     if (lane == 0) {
@@ -867,14 +887,15 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
         ++issued;
       }
     }
-  } else if (warp == 1) {
+  } else if (warp == 1 || second) {
     {
       const uint32_t e = elect_one(), tm = __shfl_sync(0xffffffffu, tmem, 0);
       const UmmaDesc bd0 = umma_desc(sb32);
-      for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-        const int slot = issued % ns, acc = issued % kTmaAcc;
-        bool got = issued < kTmaAcc || mbar_wait(&acce[acc], (uint32_t)(issued / kTmaAcc - 1) & 1u, &s_fail);
-        got = got && mbar_wait(&full[slot], (uint32_t)(issued / ns) & 1u, &s_fail);
+      // the block's tiles i = 0, 1, ..: alternate ones where there are two MMA warps
+      for (int i = second, t = blockIdx.x + i * gridDim.x; t < n_tiles; i += MW, t += MW * gridDim.x) {
+        const int slot = i % ns, acc = i % kTmaAcc;
+        bool got = i < kTmaAcc || mbar_wait(&acce[acc], (uint32_t)(i / kTmaAcc - 1) & 1u, &s_fail);
+        got = got && mbar_wait(&full[slot], (uint32_t)(i / ns) & 1u, &s_fail);
         if (!__all_sync(0xffffffffu, got)) { fail(); break; }
         tc_fence_after();
         // descriptors: the stage's first entry plus the (parity, row, entry, channel) offset of each
@@ -926,7 +947,7 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
         }
         umma_commit(e, &empty[slot]);                // the stage is free once these MMAs complete
         umma_commit(e, &accf[acc]);
-        ++issued;
+        issued = i + 1;
       }
     }
   } else {
@@ -1020,7 +1041,7 @@ __global__ void __launch_bounds__(kTmaThreads, tma_blocks(CIN, MODE)) k_conv_tma
         mbar_wait(&full[s], (uint32_t)(last / ns) & 1u);
       }
     }
-    if (tid == 32 && issued > 0)
+    if ((warp == 1 || second) && lane == 0 && issued > 0)
       mbar_wait(&accf[(issued - 1) % kTmaAcc], (uint32_t)((issued - 1) / kTmaAcc) & 1u);
     __syncthreads();
   }
@@ -1685,16 +1706,18 @@ int conv_tma(const __nv_bfloat16* in, const __nv_bfloat16* w, const float* bias,
   while (ns > 2 && fixed + ns * stage > share) --ns;
   while (ns >= 2 && fixed + ns * stage > room) --ns;
   if (ns < 2) return GFH_ERR_SIZE;
+  if (tma_mma_warps(CIN, COUT, S) == 2) ns &= ~1;
   const size_t smem = fixed + ns * stage;
   GFH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   GFH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+  constexpr int threads = tma_threads(CIN, COUT, S);
   const int regs = std::max(1, (fa.numRegs + 7) / 8 * 8);
   const int per_sm = std::max(1, std::min({(int)(kSmemPerSm / (smem + fa.sharedSizeBytes + 1024)),
-                                           65536 / (regs * kTmaThreads), 2048 / kTmaThreads,
+                                           65536 / (regs * threads), 2048 / threads,
                                            512 / (kTmaAcc * NPAR * COUT)}));
   const int64_t tiles = (int64_t)B * Ho * (Wt / CW);
   const int grid = (int)std::min<int64_t>(tiles, (int64_t)sms * per_sm);
-  fn<<<grid, kTmaThreads, smem, st>>>(map, omap, w, bias, mbits, bits, out, B, H, ns, flag);
+  fn<<<grid, threads, smem, st>>>(map, omap, w, bias, mbits, bits, out, B, H, ns, flag);
   GFH_CUDA_TRY(cudaGetLastError());
   return GFH_OK;
 }
