@@ -333,9 +333,11 @@ __device__ __forceinline__ void fill_tile(const MapDev& md, const TileDev& t, in
 // events' integer instructions, about 7 per event, and the increments' bank conflicts (2.4 wavefronts
 // each): 4.68 ms against 7.56 ms for the row-by-row form on flat 16 x 3072 tiles.  On sparse maps
 // (11 braking indices, 1.76e9 cells, 1.3 peak rows per cell) the tiles' chain of dependent loads and
-// barriers: 5.63 against 5.67 ms.  Small maps gain from the split tiles: 500 rows x 51,695 columns
-// 129 against 215 us, the 32 rows of a followed-up candidate 26 against 70 us, 12 uneven peakmaps
-// 0.50 against 1.36 ms.
+// barriers: 5.63 against 5.67 ms; there and on small steep maps it can be the slower of the two (five
+// maps of 228-1858 rows x 85,654-164,343 columns 1.68 against 1.46 ms, 1672 x 2494 cells of 383 FFTs
+// 91 against 72 us).  Small maps gain from the planned tiles (whole calls): 500 rows x 51,695
+// columns 134 against 234 us, the 32 rows of a followed-up candidate 42 against 86 us, 12 uneven
+// peakmaps 0.49 against 1.42 ms.
 //
 // Shared memory: tot[32] row-0 chunk sums | spare words | skey[bands] candidate keys | sums per warp
 // | ent[2 batch] | G.
