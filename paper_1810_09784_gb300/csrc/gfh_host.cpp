@@ -385,6 +385,26 @@ struct HostMap {
   int64_t ana_lo = 0, ana_hi = -1;   // first and last analysis column (contiguous: f0 falls with the column)
 };
 
+// max |v_i - line| over a table, in whole units rounded up, of the line through its ends.
+float line_error(const std::vector<int64_t>& v) {
+  const int64_t n = (int64_t)v.size() - 1;
+  if (n < 1) return 0.f;
+  const __int128 d = (__int128)v[n] - v[0];
+  __int128 most = 0;
+  for (int64_t i = 1; i < n; ++i) {
+    const __int128 e = ((__int128)v[i] - v[0]) * n - d * i;
+    most = std::max(most, e < 0 ? -e : e);
+  }
+  const int64_t up = (int64_t)((most + n - 1) / n);
+  const float f = (float)up;
+  return (int64_t)f < up ? std::nextafter(f, INFINITY) : f;
+}
+
+ShiftLine shift_line(const HostMap& hm) {
+  return ShiftLine{hm.B[0], hm.S[0], hm.B.back() - hm.B[0], hm.S.back() - hm.S[0],
+                   line_error(hm.B), line_error(hm.S), (int32_t)hm.B.size()};
+}
+
 void find_analysis_columns(HostMap& hm) {
   const int64_t n = (int64_t)hm.band.size();
   int64_t a = 0, b = n - 1;
@@ -814,10 +834,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
     md.UP = (const longlong2*)(base + o_U[m]);
     md.SD = (const FftRow*)(base + o_SD[m]);
     md.B = g.k_min != 0.0 ? (const int64_t*)(base + o_B[m]) : nullptr;
-    md.b0 = hm.B[0];
-    md.s0 = hm.S[0];
-    md.db = g.n_fft > 1 ? (float)((double)(hm.B[g.n_fft - 1] - hm.B[0]) / (g.n_fft - 1)) : 0.f;
-    md.ds = g.n_fft > 1 ? (float)((double)(hm.S[g.n_fft - 1] - hm.S[0]) / (g.n_fft - 1)) : 0.f;
+    md.line = shift_line(hm);
     md.col_band = (const int32_t*)(base + o_band[m]);
     md.f0c = (const double*)(base + o_f0[m]);
     md.f0n = (const double*)(base + o_f0n[m]);

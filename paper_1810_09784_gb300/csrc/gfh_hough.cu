@@ -388,18 +388,6 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
     const int64_t* const Bt = md.B;
     const longlong2* const UP = md.UP + bin0;
     const bool window = !XD && !(state & kListFftUnsorted);
-    const int64_t r0 = t.row0, r1 = r0 + t.nrows - 1;
-    // The shift of FFT i on row r is the line base + i slope within 2 r + 4 lattice units and the
-    // rounding of float32, so the FFTs whose shift is at most (at least) x are those up to (from)
-    // (x - base) / slope within `slack`, the other way round where k < 0 (n = 0) makes the shift
-    // fall with the FFT; with slope 0 every FFT may meet the tile and none is known to cover it.
-    const int64_t base0 = md.b0 + r0 * md.s0, base1 = md.b0 + r1 * md.s0;
-    const float sl0 = md.db + (float)r0 * md.ds, sl1 = md.db + (float)r1 * md.ds;
-    const float inv0 = sl0 != 0.f ? 1.f / sl0 : 0.f, inv1 = sl1 != 0.f ? 1.f / sl1 : 0.f;
-    const float ffts = (float)md.n_fft;
-    const float slack0 = 2.f + (float)(2 * r0 + 4) * fabsf(inv0) + ffts * 0x1p-20f;
-    const float slack1 = 2.f + (float)(2 * r1 + 4) * fabsf(inv1) + ffts * 0x1p-20f;
-    auto clampf = [&](float x) { return (int)fminf(fmaxf(x, -1.f), ffts); };
     for (int q0 = 0; q0 < (fits ? nbw : 0); q0 += batch) {
       const int nq = min(batch, nbw - q0);
       // per bin (one thread each): its peaks that have an edge in the tile, in one or two pieces
@@ -419,29 +407,15 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
           auto to = [&](int i) {
             return i <= 0 ? 0 : (i >= md.n_fft ? n : __ldg(blk + ((i - 1) >> md.shift) + 1));
           };
-          auto col = [](int c) { return (int64_t)c << GFH_FRAC_BITS; };
           if (__ldg(fl + st1 + n - 1) >= nfft) atomicOr(flag, GFH_FLAG_FFT_RANGE);
-          // right edge on the first row reaches the tile (shift0 <= x); left edge on the last row is
-          // not past it (shift1 >= y)
-          const float x = (float)(up.y - col(c0) - base0) * inv0;
-          const float y = (float)(up.x - col(c0 + ub + 1) - base1) * inv1;
-          float lo = -1.f, hi = ffts;
-          if (inv0 > 0.f) hi = x + slack0;
-          if (inv0 < 0.f) lo = x - slack0;
-          if (inv1 > 0.f) lo = fmaxf(lo, y - slack1);
-          if (inv1 < 0.f) hi = fminf(hi, y + slack1);
-          const int o0 = from(clampf(lo)), o1 = max(to(clampf(hi) + 1), o0);
+          const TileLine line = tile_line(md.line, t.row0, (int64_t)t.row0 + t.nrows - 1);
+          const BinFfts w = bin_ffts(line, up.x, up.y, c0, ub, ub == C - 1, md.n_fft);
+          const int o0 = from(w.lo), o1 = max(to(w.hi + 1), o0);
           st1 += o0;
           cnt1 = o1 - o0;
-          // a bin wider than the tile: the FFTs c_lo .. c_hi cover the tile on every row (left edge
-          // at or before its first column on the first row, right edge at or past its last on the
-          // last) and are counted without a walk
-          if (((up.y - up.x) >> GFH_FRAC_BITS) >= ub && ub == C - 1 && cnt1 > 0 && inv0 != 0.f && inv1 != 0.f) {
-            const float cx = (float)(up.x - col(c0 + 1) - base0) * inv0;
-            const float cy = (float)(up.y - col(c0 + ub) - base1) * inv1;
-            const float c_lo = fmaxf(inv0 > 0.f ? cx + slack0 : -1.f, inv1 < 0.f ? cy + slack1 : -1.f);
-            const float c_hi = fminf(inv1 > 0.f ? cy - slack1 : ffts, inv0 < 0.f ? cx - slack0 : ffts);
-            const int m1 = max(to(clampf(c_lo) + 1), o0), m2 = min(from(clampf(c_hi)), o1);
+          // the FFTs that cover the tile on every row are counted without a walk
+          if (w.c_lo < w.c_hi && cnt1 > 0) {
+            const int m1 = max(to(w.c_lo + 1), o0), m2 = min(from(w.c_hi), o1);
             if (m1 < m2) {
               carry += m2 - m1;
               cnt1 = m1 - o0;

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 #include <cufft.h>
+#include <cmath>
 #include <cstdint>
 #include <cstddef>
 #include <vector>
@@ -96,6 +97,76 @@ struct alignas(16) FftRow {
   uint64_t D;
 };
 
+// A map's shifts B_i + r S_i against the FFT i: the line through the tables' ends, in whole lattice
+// units, and the largest distance of the tables from it.
+struct ShiftLine {
+  int64_t b0, s0;           // B_0, S_0
+  int64_t db, ds;           // B_last - B_0, S_last - S_0
+  float eb, es;             // max |B_i - line|, max |S_i - line|, rounded up
+  int32_t n_fft;
+};
+
+// The line on a tile's first and last row: FFT i is shifted by base + i / inv, within `slack` FFTs
+// (the tables' distance from the line, and float32's rounding of what bin_ffts computes).
+// inv = 0 where the line is level: every FFT may then meet the tile and none is known to cover it.
+struct TileLine {
+  int64_t base0, base1;
+  float inv0, inv1, slack0, slack1;
+};
+
+// The slope is the difference of the ends on that row, formed in whole units: where db and r ds have
+// opposite signs (k < 0) it can be a few units out of 2^40, and as a sum of two float32 slopes was
+// rounding alone.  With a level line's few units the slack is all FFTs.
+__host__ __device__ __forceinline__ TileLine tile_line(const ShiftLine& l, int64_t row0, int64_t row1) {
+  const int64_t d0 = l.db + row0 * l.ds, d1 = l.db + row1 * l.ds;
+  const float ffts = (float)l.n_fft, last = (float)(l.n_fft - 1);
+  TileLine t;
+  t.base0 = l.b0 + row0 * l.s0;
+  t.base1 = l.b0 + row1 * l.s0;
+  t.inv0 = d0 != 0 ? last / (float)d0 : 0.f;
+  t.inv1 = d1 != 0 ? last / (float)d1 : 0.f;
+  t.slack0 = 2.f + (l.eb + (float)row0 * l.es) * fabsf(t.inv0) + ffts * 0x1p-20f;
+  t.slack1 = 2.f + (l.eb + (float)row1 * l.es) * fabsf(t.inv1) + ffts * 0x1p-20f;
+  return t;
+}
+
+// The FFTs of one bin at a tile: those outside lo .. hi have no edge in it on any row and do not
+// cover it; those strictly between c_lo and c_hi cover it on every row.  All in -1 .. n_fft.
+struct BinFfts {
+  int lo, hi, c_lo, c_hi;
+};
+
+// left, right: the bin's first and last position; c0, ub: the tile's first column and its last one
+// inside the map, counted from c0; wide: the tile has no column past the map.
+__host__ __device__ __forceinline__ BinFfts bin_ffts(const TileLine& t, int64_t left, int64_t right,
+                                                     int64_t c0, int ub, bool wide, int n_fft) {
+  const float ffts = (float)n_fft;
+  auto clamp = [&](float x) { return (int)fminf(fmaxf(x, -1.f), ffts); };
+  BinFfts b;
+  // right edge on the first row reaches the tile (shift0 <= x); left edge on the last row is not
+  // past it (shift1 >= y)
+  const float x = (float)(right - (c0 << GFH_FRAC_BITS) - t.base0) * t.inv0;
+  const float y = (float)(left - ((c0 + ub + 1) << GFH_FRAC_BITS) - t.base1) * t.inv1;
+  float lo = -1.f, hi = ffts;
+  if (t.inv0 > 0.f) hi = x + t.slack0;
+  if (t.inv0 < 0.f) lo = x - t.slack0;
+  if (t.inv1 > 0.f) lo = fmaxf(lo, y - t.slack1);
+  if (t.inv1 < 0.f) hi = fminf(hi, y + t.slack1);
+  b.lo = clamp(lo);
+  b.hi = clamp(hi);
+  // a bin wider than the tile: left edge at or before its first column on the first row, right edge
+  // at or past its last on the last
+  b.c_lo = (int)ffts;
+  b.c_hi = -1;
+  if (wide && ((right - left) >> GFH_FRAC_BITS) >= ub && t.inv0 != 0.f && t.inv1 != 0.f) {
+    const float cx = (float)(left - ((c0 + 1) << GFH_FRAC_BITS) - t.base0) * t.inv0;
+    const float cy = (float)(right - ((c0 + ub) << GFH_FRAC_BITS) - t.base1) * t.inv1;
+    b.c_lo = clamp(fmaxf(t.inv0 > 0.f ? cx + t.slack0 : -1.f, t.inv1 < 0.f ? cy + t.slack1 : -1.f));
+    b.c_hi = clamp(fminf(t.inv1 > 0.f ? cy - t.slack1 : ffts, t.inv0 < 0.f ? cx - t.slack0 : ffts));
+  }
+  return b;
+}
+
 // One map as the kernels see it.
 struct MapDev {
   int32_t* out;             // [K][ld]
@@ -121,9 +192,7 @@ struct MapDev {
   int32_t n_fft;
   int32_t list;
   int32_t n_bands;
-  // B_i and S_i against i as lines through the table's first and last rows (a bin's windows of FFTs)
-  int64_t b0, s0;           // B_0, S_0
-  float db, ds;             // (B_last - B_0) / (n_fft - 1), (S_last - S_0) / (n_fft - 1)
+  ShiftLine line;           // a bin's windows of FFTs
 };
 
 // The index of one peak list, over the bins that some map reads (built per execute, k_index).
