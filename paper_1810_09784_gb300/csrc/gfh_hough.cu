@@ -399,15 +399,17 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
         cnt1 = (int)(md.csr[bin0 + q + 1] - s);
         if (window && cnt1 > 0) {
           const longlong2 up = __ldg(UP + q);
-          const int n = cnt1;
           const int32_t* const blk = md.blk + (int64_t)(bin0 + q) * md.nb1;
+          const int n = cnt1;
+          // indices past the table are flagged; they end the bin and are drawn nowhere
+          const bool past = __ldg(fl + st1 + n - 1) >= nfft;
+          if (past) atomicOr(flag, GFH_FLAG_FFT_RANGE);
           // first peaks of the FFT block that holds FFT i, and of the first block that starts there
           // or later (i <= 0: 0; i >= n_fft: all)
           auto from = [&](int i) { return i <= 0 ? 0 : (i >= md.n_fft ? n : __ldg(blk + (i >> md.shift))); };
           auto to = [&](int i) {
             return i <= 0 ? 0 : (i >= md.n_fft ? n : __ldg(blk + ((i - 1) >> md.shift) + 1));
           };
-          if (__ldg(fl + st1 + n - 1) >= nfft) atomicOr(flag, GFH_FLAG_FFT_RANGE);
           const TileLine line = tile_line(md.line, t.row0, (int64_t)t.row0 + t.nrows - 1);
           const BinFfts w = bin_ffts(line, up.x, up.y, c0, ub, ub == C - 1, md.n_fft);
           const int o0 = from(w.lo), o1 = max(to(w.hi + 1), o0);
@@ -415,7 +417,8 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
           cnt1 = o1 - o0;
           // the FFTs that cover the tile on every row are counted without a walk
           if (w.c_lo < w.c_hi && cnt1 > 0) {
-            const int m1 = max(to(w.c_lo + 1), o0), m2 = min(from(w.c_hi), o1);
+            const int m1 = max(to(w.c_lo + 1), o0);
+            const int m2 = min(from(past ? min(w.c_hi, md.n_fft - 1) : w.c_hi), o1);
             if (m1 < m2) {
               carry += m2 - m1;
               cnt1 = m1 - o0;
