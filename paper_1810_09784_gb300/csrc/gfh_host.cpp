@@ -658,6 +658,30 @@ size_t tile_bytes(const std::vector<TileDev>& tiles, int rows_x, int* bands) {
   return (size_t)words * 8;
 }
 
+constexpr gfh_tile_config kDefaultShape{16, 3072, 512, 0};
+
+bool same_shape(const gfh_tile_config& a, const gfh_tile_config& b) {
+  return a.rows == b.rows && a.cols == b.cols && a.threads == b.threads;
+}
+
+// The shape a plan takes for the requested one (null or zero fields: the default's).  form selects
+// nothing and is not kept, so that it tells no two shapes apart.
+int tile_config(const gfh_tile_config* cfg, gfh_tile_config* tc) {
+  *tc = kDefaultShape;
+  if (cfg) {
+    if (cfg->rows) tc->rows = cfg->rows;
+    if (cfg->cols) tc->cols = cfg->cols;
+    if (cfg->threads) tc->threads = cfg->threads;
+    if (!(cfg->form == 0 || cfg->form == 1)) return GFH_ERR_ARG;
+  }
+  if (!(tc->rows == 4 || tc->rows == 8 || tc->rows == 16 || tc->rows == 32) || tc->cols < 128 || tc->cols % 128 ||
+      tc->cols > 4096 || !(tc->threads == 256 || tc->threads == 512 || (tc->threads == 1024 && tc->rows >= 16)))
+    return GFH_ERR_ARG;
+  const int nwarps = tc->threads / 32;
+  if ((tc->cols / 128 + nwarps - 1) / nwarps > 4) return GFH_ERR_ARG;  // <= 4 chunks per warp
+  return GFH_OK;
+}
+
 }  // namespace
 
 extern "C" int gfh_plan_destroy(gfh_plan* p) {
@@ -678,22 +702,11 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
                                gfh_plan** out) {
   if (!ctx || !out || n_maps < 1 || !grids || !h_maps) return GFH_ERR_ARG;
   *out = nullptr;
-  gfh_tile_config tc{16, 3072, 512, 0};
-  if (cfg) {
-    if (cfg->rows) tc.rows = cfg->rows;
-    if (cfg->cols) tc.cols = cfg->cols;
-    if (cfg->threads) tc.threads = cfg->threads;
-    tc.form = cfg->form;
-  }
-  if (!(tc.rows == 4 || tc.rows == 8 || tc.rows == 16 || tc.rows == 32) || tc.cols < 128 || tc.cols % 128 ||
-      tc.cols > 4096 || !(tc.form == 0 || tc.form == 1) ||
-      !(tc.threads == 256 || tc.threads == 512 || (tc.threads == 1024 && tc.rows >= 16)))
-    return GFH_ERR_ARG;
+  gfh_tile_config tc;
+  if (tile_config(cfg, &tc) != GFH_OK) return GFH_ERR_ARG;
   // The default shape stands for tiles planned by their work (512 threads, two blocks per SM); any
   // other is taken as it is, in strips of half its columns (a cell has two counts).
-  const bool planned = tc.rows == 16 && tc.cols == 3072 && tc.threads == 512 && tc.form == 0;
-  const int nwarps = tc.threads / 32;
-  if ((tc.cols / 128 + nwarps - 1) / nwarps > 4) return GFH_ERR_ARG;  // <= 4 chunks per warp
+  const bool planned = same_shape(tc, kDefaultShape);
 
   std::vector<HostMap> hms(n_maps);
   std::vector<TileDev> tiles, tiles_x;
@@ -1080,10 +1093,6 @@ int time_plan(gfh_plan* q, const gfh_peaks* peaks, int reps, float* ms) {
 }
 
 // Rebuilds plan p with tile shape `shape` (same grids and outputs; coarse tiles follow the shape).
-bool same_shape(const gfh_tile_config& a, const gfh_tile_config& b) {
-  return a.rows == b.rows && a.cols == b.cols && a.threads == b.threads && a.form == b.form;
-}
-
 int reshape_plan(gfh_plan* p, const gfh_tile_config& shape) {
   if (same_shape(shape, p->cfg)) return GFH_OK;
   gfh_plan* q = nullptr;
