@@ -134,16 +134,15 @@ typedef struct gfh_peaks {
   int32_t n_lists;
 } gfh_peaks;
 
-/* Tile shape of the Hough kernel; zero fields pick the library default (16 x 3072, 512).  The
- * default stands for tiles planned by the library: their rows and columns follow each region's
- * estimated work, and heavy tiles are split until every block has its share.  Any other shape is
- * taken as it is, drawn in strips of half its columns (a cell has two counts while it is drawn).  A
- * shape of which rows x (cols + 2) int32 plus the candidate keys exceed 227 KB is refused.
- * form is accepted for compatibility (0 or 1) and selects nothing: every warp draws edge event by
- * edge event.  The maps do not depend on the shape. */
+/* Tile shape of the Hough kernel; zero fields pick the library default (16 x 3072, 512).  It gives a
+ * block's threads and the shared memory of its tiles; their rows and columns are planned by the
+ * library, by each region's estimated work, and heavy tiles are split until every block has its share.
+ * A shape of which rows x (cols + 2) int32 plus the candidate keys exceed 227 KB is refused.
+ * form is accepted for compatibility (0 or 1) and selects nothing.  The maps do not depend on the
+ * shape. */
 typedef struct gfh_tile_config {
-  int32_t rows;     /* k rows per tile: 4, 8, 16 or 32 */
-  int32_t cols;     /* x0 columns per tile: multiple of 128, at most 4096 */
+  int32_t rows;     /* 4, 8, 16 or 32 */
+  int32_t cols;     /* multiple of 128, at most 4096 */
   int32_t threads;  /* threads per block: 256 or 512, or 1024 with 16 or 32 rows */
   int32_t form;     /* 0 or 1, no effect */
 } gfh_tile_config;

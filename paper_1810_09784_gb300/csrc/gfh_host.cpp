@@ -382,6 +382,7 @@ struct HostMap {
   std::vector<int32_t> band;
   std::vector<double> f0, f0n;
   int64_t cells = 0;
+  bool one = false;                  // sparse: one count per cell
   int64_t ana_lo = 0, ana_hi = -1;   // first and last analysis column (contiguous: f0 falls with the column)
 };
 
@@ -412,6 +413,19 @@ void find_analysis_columns(HostMap& hm) {
   while (b >= a && hm.band[b] < 0) --b;
   hm.ana_lo = a;
   hm.ana_hi = b;
+}
+
+// Peaks per (FFT, bin) of noise (threshold 2.5, local maxima).
+constexpr double kNoisePeaks = 0.0755;
+
+// Whether a map is drawn with one count per cell (+1 and -1) and not with two (+1 each).  Two halve a
+// tile, one makes lanes that leave the same column wait for each other.  Tiles of a map with few peaks
+// per column cost what their cells and chains of loads cost: fewer, larger ones are faster below two
+// (x0 columns counted, each peak of the band on each of them once): 51 half-hour maps (0.85) 7.00 ->
+// 4.73 ms, 11 braking indices (1.3) 5.78 -> 3.83 ms, one half-hour map (1.6) 138 -> 105 us.  Above,
+// 0.81 to 0.92 of the speed at 2.9 to 3.1, half at 50 (75 drawn plans, 12 uneven peakmaps).
+bool sparse_map(const gfh_grid& g) {
+  return kNoisePeaks * g.n_fft * (double)(g.bin_hi - g.bin_lo + 1) < 2.0 * (double)g.n_x0;
 }
 
 // Bin range [ja, jb] of the peaks that can touch columns [c0, c1) on rows [r0, r1) (tile planning).
@@ -472,6 +486,7 @@ TileDev make_tile(const gfh_grid& g, const HostMap& hm, int m, int r0, int nr, i
   t.ncols = nc;
   tile_bins(g, hm, s_min, s_max, c0, c0 + nc, &t.bin_a, &t.bin_b);
   column_bands(hm, c0, c0 + nc, &t.band_lo, &t.band_hi);
+  t.one = hm.one;
   return t;
 }
 
@@ -519,34 +534,34 @@ double tile_work(const gfh_grid& g, const HostMap& hm, const TileDev& t) {
     ffts += len;
     moved += len * shift * (t.nrows - 1);
   }
-  const double runs = 0.0755 / 32.0 * nb / samples;
+  const double runs = kNoisePeaks / 32.0 * nb / samples;
   if (ffts <= 0.0) return fill;
   return 8000.0 + cells / 128.0 * 50.0 + 8.0 * nb + runs * (190.0 * ffts + 16.0 * moved);
 }
 
-// Rows x columns of a tile with a given room (words of one of its two counts).
+// Words of one count of a tile; its columns for given rows and words of one count.
 int64_t tile_words(int rows, int cols) { return (int64_t)rows * (cols + kHoughPad); }
 int cols_for(int rows, int64_t words) {
   return (int)std::min<int64_t>(4096, std::max<int64_t>(64, (words / rows - kHoughPad) / 64 * 64));
 }
 
-// Tiles of map m over rows [r0, r1) x columns [c_lo, c_hi) (both multiples of 4).  Chosen shapes: per
-// region of kTall rows by the columns of the flattest shape, the shape of least work.  Tall, narrow
-// tiles halve the peaks' fixed work with every doubling of the rows, flat wide ones suit regions with
-// few edges, whose cost is the cells'.
-void map_tiles(const gfh_grid& g, const HostMap& hm, int m, const TilePlan& tp, int r0, int r1,
+// Uniform tiles of map m over rows [r0, r1) x columns [c_lo, c_hi) (both multiples of 4).
+void cut_tiles(const gfh_grid& g, const HostMap& hm, int m, int r0, int r1, int64_t c_lo, int64_t c_hi,
+               int rows, int cols, std::vector<TileDev>& out) {
+  for (int r = r0; r < r1; r += rows)
+    for (int64_t x = c_lo; x < c_hi; x += cols)
+      out.push_back(make_tile(g, hm, m, r, std::min(rows, r1 - r), x, (int)std::min<int64_t>(cols, c_hi - x)));
+}
+
+// Tiles of map m over rows [r0, r1) x columns [c_lo, c_hi) (both multiples of 4), of at most `room`
+// words: per region of kTall rows by the columns of the flattest shape, the shape of least work.
+// Tall, narrow tiles halve the peaks' fixed work with every doubling of the rows, flat wide ones suit
+// regions with few edges, whose cost is the cells'.
+void map_tiles(const gfh_grid& g, const HostMap& hm, int m, int64_t room, int r0, int r1,
                int64_t c_lo, int64_t c_hi, std::vector<TileDev>& tiles) {
-  auto cut = [&](int a, int b, int64_t c, int64_t d, int rows, int cols, std::vector<TileDev>& out) {
-    for (int r = a; r < b; r += rows)
-      for (int64_t x = c; x < d; x += cols)
-        out.push_back(make_tile(g, hm, m, r, std::min(rows, b - r), x, (int)std::min<int64_t>(cols, d - x)));
-  };
-  if (tp.rows > 0) {
-    cut(r0, r1, c_lo, c_hi, tp.rows, tp.cols, tiles);
-    return;
-  }
+  const int64_t words = hm.one ? room : room / 2;
   constexpr int kTall = 128, kFlat = 8;
-  const int wide = cols_for(kFlat, tp.words);
+  const int wide = cols_for(kFlat, words);
   std::vector<TileDev> best, cand;
   for (int a = r0; a < r1; a += kTall) {
     const int b = std::min(r1, a + kTall);
@@ -555,7 +570,7 @@ void map_tiles(const gfh_grid& g, const HostMap& hm, int m, const TilePlan& tp, 
       double best_work = -1.0;
       for (int rows = kFlat; rows <= kTall; rows *= 2) {
         cand.clear();
-        cut(a, b, c, d, rows, cols_for(rows, tp.words), cand);
+        cut_tiles(g, hm, m, a, b, c, d, rows, cols_for(rows, words), cand);
         double work = 0.0;
         for (const TileDev& t : cand) work += tile_work(g, hm, t);
         if (best_work < 0.0 || work < best_work) { best_work = work; best.swap(cand); }
@@ -647,15 +662,15 @@ void sort_tiles(std::vector<TileDev>& tiles, const std::vector<double>& work) {
   tiles.swap(out);
 }
 
-// Shared-memory bytes of the largest tile's counts (x: the x-direction form, whole tiles of `rows`),
-// and the most bands in a tile.
+// Shared-memory bytes of the largest tile's counts (rows_x: tiles of the x-direction form, all of that
+// many rows), and the most bands in a tile.
 size_t tile_bytes(const std::vector<TileDev>& tiles, int rows_x, int* bands) {
   int64_t words = 0;
   for (const TileDev& t : tiles) {
-    words = std::max(words, tile_words(rows_x > 0 ? rows_x : t.nrows, t.ncols));
+    words = std::max(words, tile_words(rows_x > 0 ? rows_x : t.nrows, t.ncols) * (rows_x == 0 && t.one ? 1 : 2));
     *bands = std::max(*bands, t.band_hi - t.band_lo + 1);
   }
-  return (size_t)words * 8;
+  return (size_t)words * 4;
 }
 
 constexpr gfh_tile_config kDefaultShape{16, 3072, 512, 0};
@@ -704,15 +719,16 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   *out = nullptr;
   gfh_tile_config tc;
   if (tile_config(cfg, &tc) != GFH_OK) return GFH_ERR_ARG;
-  // The default shape stands for tiles planned by their work (512 threads, two blocks per SM); any
-  // other is taken as it is, in strips of half its columns (a cell has two counts).
+  // The shape gives a tile's room and its block's threads; the tiles in that room are planned.  (A tile
+  // leaves 24 KB of shared memory for the chunk sums, band keys and windows.)  The default's room is
+  // that of two blocks per SM.
   const bool planned = same_shape(tc, kDefaultShape);
+  const int64_t room = planned ? kPlannedWords
+                               : std::min<int64_t>(tile_words(tc.rows, tc.cols), (kHoughSmemLimit - 24 * 1024) / 4);
 
   std::vector<HostMap> hms(n_maps);
   std::vector<TileDev> tiles, tiles_x;
-  // (a strip leaves 24 KB of shared memory for the chunk sums, band keys and windows)
-  const TilePlan shape{tc.rows, std::min(tc.cols / 2, cols_for(tc.rows, (int64_t)(kHoughSmemLimit - 24 * 1024) / 8)), 0};
-  const TilePlan chosen{0, 0, kPlannedWords};
+  const int cols_x = std::min(tc.cols / 2, cols_for(tc.rows, (int64_t)(kHoughSmemLimit - 24 * 1024) / 8));
   std::vector<char> map_xd(n_maps, 0);
   int max_tile_bands = 1, cfg_bands = 1;
   std::map<int, ListDev> by_list;           // per list read: the bins and FFTs that its maps cover
@@ -740,13 +756,15 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
     // fewer events differenced along x0 on every row (2 per row) than along k (the columns it
     // crosses): such maps use the x-direction form.
     map_xd[m] = hm.S[g.n_fft - 1] > (int64_t(2) << GFH_FRAC_BITS);
+    hm.one = sparse_map(g);
     find_analysis_columns(hm);
     for (int64_t c = 0; c < g.ld_x0; c += tc.cols) {
       int32_t lo, hi;
       column_bands(hm, c, std::min<int64_t>(c + tc.cols, g.ld_x0), &lo, &hi);
       cfg_bands = std::max(cfg_bands, hi - lo + 1);
     }
-    map_tiles(g, hm, m, planned && !map_xd[m] ? chosen : shape, 0, g.n_k, 0, g.ld_x0, map_xd[m] ? tiles_x : tiles);
+    if (map_xd[m]) cut_tiles(g, hm, m, 0, g.n_k, 0, g.ld_x0, tc.rows, cols_x, tiles_x);
+    else map_tiles(g, hm, m, room, 0, g.n_k, 0, g.ld_x0, tiles);
   }
   // The given tile must fit in shared memory (one count per cell, chunk sums, band keys).
   const bool select = h_cands != nullptr || d_stats != nullptr;
@@ -758,7 +776,9 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   for (size_t q = 0; q < tiles.size(); ++q) work[q] = tile_work(grids[tiles[q].map], hms[tiles[q].map], tiles[q]);
   for (size_t q = 0; q < tiles_x.size(); ++q)
     work_x[q] = (double)std::max(0, tiles_x[q].bin_b - tiles_x[q].bin_a + 1) * tiles_x[q].nrows;
-  if (planned) balance_tiles(std::vector<gfh_grid>(grids, grids + n_maps), hms, 2 * ctx->num_sms, tiles, work);
+  const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(kSmemPerSm / ((size_t)room * 4 + 8192),
+                                                               tc.threads == 256 ? 3 : 1024 / tc.threads));
+  balance_tiles(std::vector<gfh_grid>(grids, grids + n_maps), hms, per_sm * ctx->num_sms, tiles, work);
   sort_tiles(tiles, work);
   sort_tiles(tiles_x, work_x);
   const size_t cells = tile_bytes(tiles, 0, &max_tile_bands);
@@ -822,7 +842,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   p->grids.assign(grids, grids + n_maps);
   p->cfg = tc;
   p->planned = planned;
-  p->shape = shape;
+  p->list_room = planned ? kPlannedListWords : room;
   p->cells = cells;
   p->cells_x = cells_x;
   if (cudaSetDevice(ctx->device) != cudaSuccess) { delete p; return GFH_ERR_CUDA; }
@@ -942,7 +962,6 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
   std::vector<TileDev> fine;
   std::vector<int32_t> first;
   first.reserve((size_t)p->n_maps * (nct + 1) + 1);
-  const TilePlan tp = p->planned ? TilePlan{0, 0, kPlannedListWords} : p->shape;
   int max_fine = 0, max_bands = p->max_tile_bands;
   size_t worst = 0;                        // longest gathered list: every map at its largest
   for (int m = 0; m < p->n_maps; ++m) {
@@ -952,6 +971,7 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
     if (rc) return rc;
     rc = gfh_host_columns(&g, hm.band, hm.f0, hm.f0n);
     if (rc) return rc;
+    hm.one = sparse_map(g);
     find_analysis_columns(hm);
     // columns of each f0 tile: analysis columns only; f0 falls with the column, so each range is
     // contiguous
@@ -976,7 +996,7 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
           // 16-byte aligned column range (vector stores): neighbouring tiles may share <= 3 columns
           const int64_t c_lo = cmin[xt] & ~int64_t(3);
           const int64_t c_hi = std::min<int64_t>(g.ld_x0, (cmax[xt] + 4) & ~int64_t(3));
-          map_tiles(g, hm, m, tp, r0, r1, c_lo, c_hi, fine);
+          map_tiles(g, hm, m, p->list_room, r0, r1, c_lo, c_hi, fine);
         }
         const int cnt = (int)(fine.size() - before);
         max_fine = std::max(max_fine, cnt);
@@ -986,7 +1006,7 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
     // group nct: the whole map, as gfh_plan_execute tiles it
     first.push_back((int32_t)fine.size());
     const size_t before = fine.size();
-    map_tiles(g, hm, m, tp, 0, g.n_k, 0, g.ld_x0, fine);
+    map_tiles(g, hm, m, p->list_room, 0, g.n_k, 0, g.ld_x0, fine);
     const size_t whole = fine.size() - before;
     std::sort(sizes.begin(), sizes.end(), std::greater<int>());
     size_t top = 0;

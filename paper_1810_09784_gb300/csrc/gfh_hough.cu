@@ -21,7 +21,8 @@ constexpr int kListUnsorted = 1, kListFftUnsorted = 2;   // bits of a peak list'
 constexpr int kFewBands = 4;     // a tile of at most this many bands looks for its best cells only if they can win
 template <int NT> constexpr int kSumBytes = NT / kLane * 16;   // two sums per warp
 constexpr int kRowBits = 57;     // fraction bits of an event's row
-constexpr int kEventUnroll = kHoughSpare;   // events of each edge per turn of the drawing loop
+constexpr int kEventUnroll = 4;  // events of each edge per turn of the drawing loop
+constexpr int kSpareRows = kEventUnroll + 2;   // words for events that are not drawn, in rows of 32
 
 __device__ __forceinline__ int warp_sum(int v) {
 #pragma unroll
@@ -142,31 +143,38 @@ __device__ __forceinline__ void inc_shared(uint32_t p) {
   asm volatile("red.shared.inc.u32 [%0], 0xffffffff;" ::"r"(p) : "memory");
 }
 
-// One event: adds 1 at row v / 2^kRowBits of the column Q before the one p points at; with LIMIT only
-// if n > Q, else to one of the warp's spare words.  (A predicated increment compiles to a branch
+// Counts a column that is left: 1 in the second count, or (TAKE) -1 in the only one.
+template <bool TAKE>
+__device__ __forceinline__ void leave_shared(uint32_t p) {
+  if (TAKE) asm volatile("red.shared.add.u32 [%0], 0xffffffff;" ::"r"(p) : "memory");
+  else inc_shared(p);
+}
+
+// One event: adds 1 (TAKE: -1) at row v / 2^kRowBits of the column Q before the one p points at; with
+// LIMIT only if n > Q, else to one of the warp's spare words.  (A predicated increment compiles to a branch
 // around it, with its reconvergence three instructions more per event; lanes that share the spare
-// word cost nothing.)
-template <int Q, bool LIMIT>
+// word cost nothing where 1 is added; -1 is added to a word of the lane's own: on one word for all it
+// took 6.6 instead of 3.8 ms on 11 braking indices.)
+template <int Q, bool LIMIT, bool TAKE>
 __device__ __forceinline__ void event(uint64_t v, uint32_t p, int n, uint32_t row_bytes,
                                       uint32_t spare) {
   uint32_t at = (uint32_t)(v >> kRowBits) * row_bytes + p;
   if (LIMIT) at = n > Q ? at : spare;
-  asm volatile("red.shared.inc.u32 [%0 + %1], 0xffffffff;" ::"r"(at),
-               "n"(-4 * Q)
-               : "memory");
+  if (TAKE) asm volatile("red.shared.add.u32 [%0 + %1], 0xffffffff;" ::"r"(at), "n"(-4 * Q) : "memory");
+  else asm volatile("red.shared.inc.u32 [%0 + %1], 0xffffffff;" ::"r"(at), "n"(-4 * Q) : "memory");
 }
 
 // kEventUnroll events of the left and of the right edge.
-template <int Q, bool LIMIT>
+template <int Q, bool LIMIT, bool ONE>
 __device__ __forceinline__ void events(uint64_t& v1, uint64_t& v2, uint64_t D, uint32_t p1,
                                        uint32_t p2, int n1, int n2, uint32_t row_bytes,
-                                       uint32_t spare) {
+                                       uint32_t spare, uint32_t own) {
   if constexpr (Q < kEventUnroll) {
-    event<Q, LIMIT>(v1, p1, n1, row_bytes, spare);
-    event<Q, LIMIT>(v2, p2, n2, row_bytes, spare);
+    event<Q, LIMIT, false>(v1, p1, n1, row_bytes, spare);
+    event<Q, LIMIT, ONE>(v2, p2, n2, row_bytes, ONE ? own : spare);
     v1 += D;
     v2 += D;
-    events<Q + 1, LIMIT>(v1, v2, D, p1, p2, n1, n2, row_bytes, spare);
+    events<Q + 1, LIMIT, ONE>(v1, v2, D, p1, p2, n1, n2, row_bytes, spare, own);
   }
 }
 
@@ -187,8 +195,9 @@ __device__ __forceinline__ void events(uint64_t& v1, uint64_t& v2, uint64_t D, u
 // alike: the loop runs to the warp's largest count.
 // D = 0 marks s <= 2^25 (D would not fit): at most one crossing in the tile's rows (at most 128),
 // placed by an integer division.
+template <bool ONE>
 __device__ __forceinline__ void draw_peaks(uint32_t ge, uint32_t gl, uint32_t row_bytes,
-                                           uint32_t spare, int nr, int C, int ub, bool ok, int64_t a, int64_t b1, int64_t s,
+                                           uint32_t spare, uint32_t own, int nr, int C, int ub, bool ok, int64_t a, int64_t b1, int64_t s,
                                            uint64_t D, int& carry) {
   const int64_t sr = (int64_t)((uint64_t)(uint32_t)(nr - 1) * (uint64_t)s);
   int lo = (int)(a >> GFH_FRAC_BITS), hr = (int)(b1 >> GFH_FRAC_BITS);
@@ -203,7 +212,7 @@ __device__ __forceinline__ void draw_peaks(uint32_t ge, uint32_t gl, uint32_t ro
   const bool on = ok && o1 <= o2;
   carry += on && lo < 0;
   inc_shared(on && lo >= 0 ? ge + 4u * (uint32_t)lo : spare);
-  inc_shared(on && o2 < C - 1 ? gl + 4u * (uint32_t)(o2 + 1) : spare);
+  leave_shared<ONE>(on && o2 < C - 1 ? gl + 4u * (uint32_t)(o2 + 1) : (ONE ? own : spare));
   // events of the left and the right edge: columns entered, lo - 1 down to lo_n, and left, hr down to
   // hr_n + 1; those below 0 are not drawn
   int n1 = ok ? lo - max(lo_n, 0) : 0;
@@ -232,12 +241,12 @@ __device__ __forceinline__ void draw_peaks(uint32_t ge, uint32_t gl, uint32_t ro
   const int least = __reduce_min_sync(0xffffffffu, min(n1, n2));
   int e = 0;
   for (; e + kEventUnroll <= least; e += kEventUnroll) {
-    events<0, false>(v1, v2, D, p1, p2, n1, n2, row_bytes, spare);
+    events<0, false, ONE>(v1, v2, D, p1, p2, n1, n2, row_bytes, spare, own);
     p1 -= 4 * kEventUnroll;
     p2 -= 4 * kEventUnroll;
   }
   for (; e < most; e += kEventUnroll) {
-    events<0, true>(v1, v2, D, p1, p2, n1 - e, n2 - e, row_bytes, spare);
+    events<0, true, ONE>(v1, v2, D, p1, p2, n1 - e, n2 - e, row_bytes, spare, own);
     p1 -= 4 * kEventUnroll;
     p2 -= 4 * kEventUnroll;
   }
@@ -314,7 +323,8 @@ __device__ __forceinline__ void fill_tile(const MapDev& md, const TileDev& t, in
 //              M[0][m] = sum_{m' <= m} G[0][m'];
 //   row r > 0: along k - +1 at each column the interval newly covers on row r, -1 at each column it
 //              covered on row r-1 but no longer does, so that M[r][m] = M[r-1][m] + G[r][m].
-// (Two counts and not one signed one: see inc_shared.)
+// (Two counts and not one signed one: see inc_shared.)  Tiles of sparse maps (TileDev::one) keep one
+// signed count and have twice the cells in the same memory.
 // Along k a peak's interval shifts left by S_i < 1 column per row with the default k step, so on
 // most rows it enters no column and leaves none: rows after the first cost about one event per
 // (peak, row) instead of two.  An interval entering from the left of the tile on row 0 is a
@@ -333,9 +343,8 @@ __device__ __forceinline__ void fill_tile(const MapDev& md, const TileDev& t, in
 // events' integer instructions, about 7 per event, and the increments' bank conflicts (2.4 wavefronts
 // each): 4.68 ms against 7.56 ms for the row-by-row form on flat 16 x 3072 tiles.  On sparse maps
 // (11 braking indices, 1.76e9 cells, 1.3 peak rows per cell) the tiles' chain of dependent loads and
-// barriers: 5.63 against 5.67 ms; there and on small steep maps it can be the slower of the two (five
-// maps of 228-1858 rows x 85,654-164,343 columns 1.68 against 1.46 ms, 1672 x 2494 cells of 383 FFTs
-// 91 against 72 us).  Small maps gain from the planned tiles (whole calls): 500 rows x 51,695
+// barriers: with one count per cell 4.04 against 5.67 ms, five maps of 228-1858 rows x 85,654-164,343
+// columns 1.10 against 1.46 ms.  Small maps gain from the planned tiles (whole calls): 500 rows x 51,695
 // columns 134 against 234 us, the 32 rows of a followed-up candidate 42 against 86 us, 12 uneven
 // peakmaps 0.49 against 1.42 ms.
 //
@@ -354,17 +363,23 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
   const MapDev& md = maps[t.map];
   const int C = t.ncols;
   const int lds = C + kHoughPad;                 // row stride
-  const int gap = (XD ? R : t.nrows) * lds;      // from the columns entered to the columns left
+  const int words = (XD ? R : t.nrows) * lds;
+  const bool one = !XD && t.one;
+  const int gap = one ? 0 : words;               // from the columns entered to the columns left
   int* tot = reinterpret_cast<int*>(smem);
   int* wsum = tot;                               // the warps' sums while windows are laid out
-  unsigned long long* skey = reinterpret_cast<unsigned long long*>(tot + ((XD ? R : 1) + kEventUnroll) * kLane);
+  unsigned long long* skey = reinterpret_cast<unsigned long long*>(tot + ((XD ? R : 1) + kSpareRows) * kLane);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nb_tile = t.band_hi >= t.band_lo ? t.band_hi - t.band_lo + 1 : 0;
   const int c0 = (int)t.col0;
   const int ub = min(C - 1, (int)(md.W - 1 - t.col0));   // last column inside the map
   const uint32_t ge = (uint32_t)__cvta_generic_to_shared(G), gl = ge + 4u * (uint32_t)gap;
   const uint32_t row_bytes = 4u * (uint32_t)lds;
-  const uint32_t spare = (uint32_t)__cvta_generic_to_shared(tot + (XD ? R : 1) * kLane + kEventUnroll * (warp + 1) - 1);
+  // spare words: kEventUnroll per warp, then as many below the lanes' own (an event's offset reaches
+  // them), which the warps share
+  const uint32_t spares = (uint32_t)__cvta_generic_to_shared(tot + (XD ? R : 1) * kLane);
+  const uint32_t spare = spares + 4u * (uint32_t)(kEventUnroll * (warp + 1) - 1);
+  const uint32_t own = spares + 4u * (uint32_t)(kEventUnroll * kLane + kEventUnroll + lane);
   if (SELECT) {
     for (int i = tid; i < nb_tile; i += NT) skey[i] = 0ull;
     if (tid < kFewBands) s_best[tid] = 0;
@@ -437,7 +452,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
       const int before = warp_sum(lane < warp ? ws : 0), total = warp_sum(ws);
       if (total == 0) continue;
       if (!drawn)
-        for (int i = tid; i < gap / 2; i += NT) reinterpret_cast<int4*>(G)[i] = make_int4(0, 0, 0, 0);
+        for (int i = tid; i < (words + gap) / 4; i += NT) reinterpret_cast<int4*>(G)[i] = make_int4(0, 0, 0, 0);
       drawn = true;
       if (tid < nq) {
         const int e0 = before + incl - cnt;
@@ -520,7 +535,8 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
         if constexpr (XD) {
           if (ok) draw_peak_x<R>(ge, gl, row_bytes, a, b1, s, C, ub, carry_x);
         } else {
-          draw_peaks(ge, gl, row_bytes, spare, t.nrows, C, ub, ok, a, b1, s, d, carry);
+          if (one) draw_peaks<true>(ge, gl, row_bytes, spare, own, t.nrows, C, ub, ok, a, b1, s, d, carry);
+          else draw_peaks<false>(ge, gl, row_bytes, spare, own, t.nrows, C, ub, ok, a, b1, s, d, carry);
         }
         interval(sd, B, up);
         ok = ok_nx;
@@ -548,7 +564,9 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
   const int nch = (C + 127) / 128;
   const int nsum = XD ? t.nrows * nch : nch;
   auto load4 = [&](const int* g) {               // entered - left
-    const int4 e = *reinterpret_cast<const int4*>(g), l = *reinterpret_cast<const int4*>(g + gap);
+    const int4 e = *reinterpret_cast<const int4*>(g);
+    if (one) return e;
+    const int4 l = *reinterpret_cast<const int4*>(g + gap);
     return make_int4(e.x - l.x, e.y - l.y, e.z - l.z, e.w - l.w);
   };
   for (int idx = warp; idx < nsum; idx += NW) {
@@ -573,7 +591,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
     const int add = before + warp_incl_scan(g.w, lane) - g.w;
     if (col < C) {
       *reinterpret_cast<int4*>(&G[rr * lds + col]) = make_int4(g.x + add, g.y + add, g.z + add, g.w + add);
-      *reinterpret_cast<int4*>(&G[rr * lds + col + gap]) = make_int4(0, 0, 0, 0);
+      if (!one) *reinterpret_cast<int4*>(&G[rr * lds + col + gap]) = make_int4(0, 0, 0, 0);
     }
   }
   __syncthreads();
@@ -888,7 +906,7 @@ int launch_hough_t(gfh_plan* p, const gfh_peaks* peaks, int which) {
   if (!list && n_tiles == 0) return GFH_OK;
   const TileDev* const tiles = list ? p->d_sel_tiles : p->d_tiles + (XD ? p->n_tiles : 0);
   const size_t cells = list ? p->cells_list : XD ? p->cells_x : p->cells;
-  const size_t head = (size_t)kLane * 4 * (kHoughSpare + (XD ? R : 1)) +
+  const size_t head = (size_t)kLane * 4 * (kSpareRows + (XD ? R : 1)) +
                       (p->select ? (size_t)p->max_tile_bands * 8 : 0);
   // head (chunk sums, spare words, band keys), sums, the windows of as many bins as there are
   // threads, or as fit beside the tile without lowering the blocks per SM, the tile

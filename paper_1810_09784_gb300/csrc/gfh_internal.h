@@ -19,11 +19,11 @@ constexpr size_t kSmemPerSm = 228 * 1024;   // shared memory of one SM
 constexpr size_t kHoughSmemLimit = kMaxSmemBytes - 64;
 
 // Shared memory of a Hough tile: words between its rows' ends and starts (rows stay 16-byte aligned,
-// and 4 words from row to row spread a line's cells over the banks), spare words per warp.
-constexpr int kHoughPad = 4, kHoughSpare = 4;
-// Room of a planned tile (words of one of its two counts): two blocks of 512 threads per SM, and
-// three of 256 for the coarse-tile search.
-constexpr int64_t kPlannedWords = 12544, kPlannedListWords = 8224;
+// and 4 words from row to row spread a line's cells over the banks).
+constexpr int kHoughPad = 4;
+// Room of a planned tile (words): two blocks of 512 threads per SM, and three of 256 for the
+// coarse-tile search.
+constexpr int64_t kPlannedWords = 25088, kPlannedListWords = 16448;
 
 // Counter-based generator of the statistical peakmap model: the splitmix64 finaliser (Steele, Lea
 // and Flood, "Fast splittable pseudorandom number generators", OOPSLA 2014) applied to a key built
@@ -214,12 +214,7 @@ struct TileDev {
   int32_t bin_b;
   int32_t band_lo;    // candidate bands present in the tile's columns (band_hi < 0: none)
   int32_t band_hi;
-};
-
-// Tile shapes of a plan's maps.
-struct TilePlan {
-  int rows = 0, cols = 0;       // uniform tiles, or rows = 0:
-  int64_t words = 0;            // shapes chosen by the work they make, within this room
+  int32_t one;        // drawn with one count per cell, not two
 };
 
 struct gfh_plan {
@@ -227,8 +222,8 @@ struct gfh_plan {
   int n_maps = 0;
   std::vector<gfh_grid> grids;
   gfh_tile_config cfg{};
-  TilePlan shape;              // of uniform tiles
-  bool planned = false;        // tile shapes chosen by their work (the default shape)
+  bool planned = false;        // the default shape (its coarse tiles take 256 threads)
+  int64_t list_room = 0;       // words of a coarse tile's tiles
   size_t cells = 0, cells_x = 0, cells_list = 0;   // shared memory of the largest tile's counts: full
                                                    // search's two lists, coarse tiles
   void* d_buf = nullptr;       // tables, map descriptors, tiles

@@ -29,8 +29,11 @@ int main() {
     if (gfh_host_tables(&g, hm.U, hm.B, hm.S) || gfh_host_columns(&g, hm.band, hm.f0, hm.f0n)) return 1;
     find_analysis_columns(hm);
     std::vector<TileDev> tiles;
-    map_tiles(g, hm, 0, TilePlan{rows, cols, kPlannedWords}, 0, g.n_k, 0, g.ld_x0, tiles);
-    if (rows == 0) {
+    hm.one = sparse_map(g);
+    if (rows > 0) {
+      cut_tiles(g, hm, 0, 0, g.n_k, 0, g.ld_x0, rows, cols, tiles);
+    } else {
+      map_tiles(g, hm, 0, kPlannedWords, 0, g.n_k, 0, g.ld_x0, tiles);
       std::vector<double> work;
       for (const TileDev& t : tiles) work.push_back(tile_work(g, hm, t));
       balance_tiles({g}, hms, 304, tiles, work);
