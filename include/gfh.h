@@ -134,9 +134,10 @@ typedef struct gfh_peaks {
   int32_t n_lists;
 } gfh_peaks;
 
-/* Tile shape of the Hough kernel; zero fields pick the library default (16 x 3072, 512).  It gives a
- * block's threads and the shared memory of its tiles; their rows and columns are planned by the
- * library, by each region's estimated work, and heavy tiles are split until every block has its share.
+/* Tile shape of the Hough kernel; zero fields pick the library default (16 x 3072, 512).  Its shared
+ * memory and threads decide how many blocks share an SM (1024 threads: two blocks of 512); the rows and
+ * columns of the tiles are planned by the library within a block's share, by each region's estimated
+ * work, and heavy tiles are split until every block has its share of the work.
  * A shape of which rows x (cols + 2) int32 plus the candidate keys exceed 227 KB is refused.
  * form is accepted for compatibility (0 or 1) and selects nothing.  The maps do not depend on the
  * shape. */

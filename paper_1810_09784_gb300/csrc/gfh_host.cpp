@@ -697,6 +697,24 @@ int tile_config(const gfh_tile_config* cfg, gfh_tile_config* tc) {
   return GFH_OK;
 }
 
+// The threads and blocks per SM of a plan, and the words that each block has for a tile.
+struct SmShare {
+  int threads, blocks;
+  int64_t room;
+};
+
+// A shape decides how many blocks share an SM, by its shared memory and its threads; tiles of any rows
+// and columns are then planned in a block's share.  (Taken as it is, a shape was up to 1.6 times as
+// slow: 51 half-hour maps at 8 x 3072 8.3 -> 4.7 ms.)  1024 threads are two blocks of 512: one block
+// has nothing to run while it waits at a tile's chain of loads and barriers (the same maps at
+// 16 x 3072 5.7 -> 4.7 ms).
+SmShare sm_share(const gfh_tile_config& tc) {
+  if (tc.threads == 1024 || same_shape(tc, kDefaultShape)) return SmShare{512, 2, kRoom[2]};
+  const size_t bytes = (size_t)tc.rows * (tc.cols + 2) * 4;
+  const int blocks = (int)std::max<size_t>(1, std::min<size_t>(kSmemPerSm / (bytes + 1024), tc.threads == 256 ? 3 : 2));
+  return SmShare{tc.threads, blocks, kRoom[blocks]};
+}
+
 }  // namespace
 
 extern "C" int gfh_plan_destroy(gfh_plan* p) {
@@ -719,12 +737,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   *out = nullptr;
   gfh_tile_config tc;
   if (tile_config(cfg, &tc) != GFH_OK) return GFH_ERR_ARG;
-  // The shape gives a tile's room and its block's threads; the tiles in that room are planned.  (A tile
-  // leaves 24 KB of shared memory for the chunk sums, band keys and windows.)  The default's room is
-  // that of two blocks per SM.
-  const bool planned = same_shape(tc, kDefaultShape);
-  const int64_t room = planned ? kPlannedWords
-                               : std::min<int64_t>(tile_words(tc.rows, tc.cols), (kHoughSmemLimit - 24 * 1024) / 4);
+  const SmShare share = sm_share(tc);
 
   std::vector<HostMap> hms(n_maps);
   std::vector<TileDev> tiles, tiles_x;
@@ -764,7 +777,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
       cfg_bands = std::max(cfg_bands, hi - lo + 1);
     }
     if (map_xd[m]) cut_tiles(g, hm, m, 0, g.n_k, 0, g.ld_x0, tc.rows, cols_x, tiles_x);
-    else map_tiles(g, hm, m, room, 0, g.n_k, 0, g.ld_x0, tiles);
+    else map_tiles(g, hm, m, share.room, 0, g.n_k, 0, g.ld_x0, tiles);
   }
   // The given tile must fit in shared memory (one count per cell, chunk sums, band keys).
   const bool select = h_cands != nullptr || d_stats != nullptr;
@@ -776,9 +789,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   for (size_t q = 0; q < tiles.size(); ++q) work[q] = tile_work(grids[tiles[q].map], hms[tiles[q].map], tiles[q]);
   for (size_t q = 0; q < tiles_x.size(); ++q)
     work_x[q] = (double)std::max(0, tiles_x[q].bin_b - tiles_x[q].bin_a + 1) * tiles_x[q].nrows;
-  const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(kSmemPerSm / ((size_t)room * 4 + 8192),
-                                                               tc.threads == 256 ? 3 : 1024 / tc.threads));
-  balance_tiles(std::vector<gfh_grid>(grids, grids + n_maps), hms, per_sm * ctx->num_sms, tiles, work);
+  balance_tiles(std::vector<gfh_grid>(grids, grids + n_maps), hms, share.blocks * ctx->num_sms, tiles, work);
   sort_tiles(tiles, work);
   sort_tiles(tiles_x, work_x);
   const size_t cells = tile_bytes(tiles, 0, &max_tile_bands);
@@ -841,8 +852,10 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   p->n_maps = n_maps;
   p->grids.assign(grids, grids + n_maps);
   p->cfg = tc;
-  p->planned = planned;
-  p->list_room = planned ? kPlannedListWords : room;
+  p->threads = share.threads;
+  // coarse tiles are small: the default's take three blocks of 256 threads
+  p->list_threads = same_shape(tc, kDefaultShape) ? 256 : share.threads;
+  p->list_room = same_shape(tc, kDefaultShape) ? kRoom[3] : share.room;
   p->cells = cells;
   p->cells_x = cells_x;
   if (cudaSetDevice(ctx->device) != cudaSuccess) { delete p; return GFH_ERR_CUDA; }

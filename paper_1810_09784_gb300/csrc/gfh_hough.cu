@@ -930,23 +930,28 @@ int launch_hough_t(gfh_plan* p, const gfh_peaks* peaks, int which) {
   return GFH_OK;
 }
 
-// The kernels of a plan: f(rows, threads, XD) as compile-time constants.  The threads are the given
-// shape's (a planned one: 512, and 256 for its coarse tiles).
+// The kernels of a plan: f(rows, threads, XD) as compile-time constants.  Only the x-direction form
+// takes the given shape as it is.
 template <class F>
 int with_kernel(const gfh_plan* p, int which, F f) {
-  auto rows = [&](auto nt) -> int {
-    if (which != kFullX) return f(std::integral_constant<int, 1>{}, nt, std::false_type{});
-    switch (p->cfg.rows) {
-      case 4: return f(std::integral_constant<int, 4>{}, nt, std::true_type{});
-      case 8: return f(std::integral_constant<int, 8>{}, nt, std::true_type{});
-      case 16: return f(std::integral_constant<int, 16>{}, nt, std::true_type{});
-      default: return f(std::integral_constant<int, 32>{}, nt, std::true_type{});
-    }
+  if (which != kFullX) {
+    const std::integral_constant<int, 1> any{};
+    if ((which == kList ? p->list_threads : p->threads) == 256)
+      return f(any, std::integral_constant<int, 256>{}, std::false_type{});
+    return f(any, std::integral_constant<int, 512>{}, std::false_type{});
+  }
+  auto threads = [&](auto rows) -> int {
+    if (p->cfg.threads == 256) return f(rows, std::integral_constant<int, 256>{}, std::true_type{});
+    if constexpr (decltype(rows)::value >= 16)
+      if (p->cfg.threads == 1024) return f(rows, std::integral_constant<int, 1024>{}, std::true_type{});
+    return f(rows, std::integral_constant<int, 512>{}, std::true_type{});
   };
-  const int threads = p->planned && which == kList ? 256 : p->cfg.threads;
-  if (threads == 256) return rows(std::integral_constant<int, 256>{});
-  if (threads == 512) return rows(std::integral_constant<int, 512>{});
-  return rows(std::integral_constant<int, 1024>{});
+  switch (p->cfg.rows) {
+    case 4: return threads(std::integral_constant<int, 4>{});
+    case 8: return threads(std::integral_constant<int, 8>{});
+    case 16: return threads(std::integral_constant<int, 16>{});
+    default: return threads(std::integral_constant<int, 32>{});
+  }
 }
 
 int launch_hough(gfh_plan* p, const gfh_peaks* peaks, int which) {

@@ -21,9 +21,9 @@ constexpr size_t kHoughSmemLimit = kMaxSmemBytes - 64;
 // Shared memory of a Hough tile: words between its rows' ends and starts (rows stay 16-byte aligned,
 // and 4 words from row to row spread a line's cells over the banks).
 constexpr int kHoughPad = 4;
-// Room of a planned tile (words): two blocks of 512 threads per SM, and three of 256 for the
-// coarse-tile search.
-constexpr int64_t kPlannedWords = 25088, kPlannedListWords = 16448;
+// Room of a tile (words) with one, two or three blocks per SM; about 43, 15 and 10 KB of a block's shared
+// memory are left for its chunk sums, band keys and windows.
+constexpr int64_t kRoom[4] = {0, 47104, 25088, 16448};
 
 // Counter-based generator of the statistical peakmap model: the splitmix64 finaliser (Steele, Lea
 // and Flood, "Fast splittable pseudorandom number generators", OOPSLA 2014) applied to a key built
@@ -222,7 +222,7 @@ struct gfh_plan {
   int n_maps = 0;
   std::vector<gfh_grid> grids;
   gfh_tile_config cfg{};
-  bool planned = false;        // the default shape (its coarse tiles take 256 threads)
+  int threads = 0, list_threads = 0;   // of a block: full search, coarse tiles
   int64_t list_room = 0;       // words of a coarse tile's tiles
   size_t cells = 0, cells_x = 0, cells_list = 0;   // shared memory of the largest tile's counts: full
                                                    // search's two lists, coarse tiles

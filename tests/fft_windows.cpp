@@ -33,7 +33,7 @@ int main() {
     if (rows > 0) {
       cut_tiles(g, hm, 0, 0, g.n_k, 0, g.ld_x0, rows, cols, tiles);
     } else {
-      map_tiles(g, hm, 0, kPlannedWords, 0, g.n_k, 0, g.ld_x0, tiles);
+      map_tiles(g, hm, 0, kRoom[2], 0, g.n_k, 0, g.ld_x0, tiles);
       std::vector<double> work;
       for (const TileDev& t : tiles) work.push_back(tile_work(g, hm, t));
       balance_tiles({g}, hms, 304, tiles, work);
