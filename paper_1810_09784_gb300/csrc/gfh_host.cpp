@@ -424,8 +424,11 @@ constexpr double kNoisePeaks = 0.0755;
 // (x0 columns counted, each peak of the band on each of them once): 51 half-hour maps (0.85) 7.00 ->
 // 4.73 ms, 11 braking indices (1.3) 5.78 -> 3.83 ms, one half-hour map (1.6) 138 -> 105 us.  Above,
 // 0.81 to 0.92 of the speed at 2.9 to 3.1, half at 50 (75 drawn plans, 12 uneven peakmaps).
-bool sparse_map(const gfh_grid& g) {
-  return kNoisePeaks * g.n_fft * (double)(g.bin_hi - g.bin_lo + 1) < 2.0 * (double)g.n_x0;
+// The x-direction form counts a left column on every row, so there the line lies at one: half-hour map
+// at 3 and 12 columns per row (1.6) 238 -> 176 and 202 -> 186 us with two counts, 11 braking indices at 4
+// columns (0.15 to 12.7) 2.90 -> 2.55 ms with one for the maps below one.
+bool sparse_map(const gfh_grid& g, bool xd) {
+  return kNoisePeaks * g.n_fft * (double)(g.bin_hi - g.bin_lo + 1) < (xd ? 1.0 : 2.0) * (double)g.n_x0;
 }
 
 // Bin range [ja, jb] of the peaks that can touch columns [c0, c1) on rows [r0, r1) (tile planning).
@@ -667,7 +670,7 @@ void sort_tiles(std::vector<TileDev>& tiles, const std::vector<double>& work) {
 size_t tile_bytes(const std::vector<TileDev>& tiles, int rows_x, int* bands) {
   int64_t words = 0;
   for (const TileDev& t : tiles) {
-    words = std::max(words, tile_words(rows_x > 0 ? rows_x : t.nrows, t.ncols) * (rows_x == 0 && t.one ? 1 : 2));
+    words = std::max(words, tile_words(rows_x > 0 ? rows_x : t.nrows, t.ncols) * (t.one ? 1 : 2));
     *bands = std::max(*bands, t.band_hi - t.band_lo + 1);
   }
   return (size_t)words * 4;
@@ -741,8 +744,8 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
 
   std::vector<HostMap> hms(n_maps);
   std::vector<TileDev> tiles, tiles_x;
-  const int cols_x = std::min(tc.cols / 2, cols_for(tc.rows, (int64_t)(kHoughSmemLimit - 24 * 1024) / 8));
   std::vector<char> map_xd(n_maps, 0);
+  double cells_xd = 0.0;
   int max_tile_bands = 1, cfg_bands = 1;
   std::map<int, ListDev> by_list;           // per list read: the bins and FFTs that its maps cover
   std::map<int, int> list_ffts;
@@ -769,15 +772,25 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
     // fewer events differenced along x0 on every row (2 per row) than along k (the columns it
     // crosses): such maps use the x-direction form.
     map_xd[m] = hm.S[g.n_fft - 1] > (int64_t(2) << GFH_FRAC_BITS);
-    hm.one = sparse_map(g);
+    hm.one = sparse_map(g, map_xd[m]);
     find_analysis_columns(hm);
     for (int64_t c = 0; c < g.ld_x0; c += tc.cols) {
       int32_t lo, hi;
       column_bands(hm, c, std::min<int64_t>(c + tc.cols, g.ld_x0), &lo, &hi);
       cfg_bands = std::max(cfg_bands, hi - lo + 1);
     }
-    if (map_xd[m]) cut_tiles(g, hm, m, 0, g.n_k, 0, g.ld_x0, tc.rows, cols_x, tiles_x);
+    if (map_xd[m]) cells_xd += (double)g.n_k * (double)g.ld_x0;
     else map_tiles(g, hm, m, share.room, 0, g.n_k, 0, g.ld_x0, tiles);
+  }
+  // x-direction tiles: uniform strips of 8 rows, four and more to each block of three per SM as far as
+  // 256 columns allow.  (Tiles of 16 rows keep 16 carries in registers and fill an SM with one block,
+  // which spilt or stood at barriers: half-hour map at 3 columns per row 242 us with 16 x 3072, 149 us so;
+  // 11 braking indices at 4 columns 2.25 against 1.97 ms.)
+  for (int m = 0; m < n_maps; ++m) {
+    if (!map_xd[m]) continue;
+    const int cols = std::max(256, (int)std::min(4096.0, cells_xd / (12.0 * ctx->num_sms * kRowsX)) / 64 * 64);
+    cut_tiles(grids[m], hms[m], m, 0, grids[m].n_k, 0, grids[m].ld_x0, kRowsX,
+              std::min(cols, cols_for(kRowsX, hms[m].one ? kRoom[3] : kRoom[3] / 2)), tiles_x);
   }
   // The given tile must fit in shared memory (one count per cell, chunk sums, band keys).
   const bool select = h_cands != nullptr || d_stats != nullptr;
@@ -793,7 +806,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   sort_tiles(tiles, work);
   sort_tiles(tiles_x, work_x);
   const size_t cells = tile_bytes(tiles, 0, &max_tile_bands);
-  const size_t cells_x = tile_bytes(tiles_x, tc.rows, &max_tile_bands);
+  const size_t cells_x = tile_bytes(tiles_x, kRowsX, &max_tile_bands);
   const int n_tiles_k = (int)tiles.size();
   tiles.insert(tiles.end(), tiles_x.begin(), tiles_x.end());
 
@@ -984,7 +997,7 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
     if (rc) return rc;
     rc = gfh_host_columns(&g, hm.band, hm.f0, hm.f0n);
     if (rc) return rc;
-    hm.one = sparse_map(g);
+    hm.one = sparse_map(g, false);
     find_analysis_columns(hm);
     // columns of each f0 tile: analysis columns only; f0 falls with the column, so each range is
     // contiguous

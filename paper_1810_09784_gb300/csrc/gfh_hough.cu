@@ -255,7 +255,7 @@ __device__ __forceinline__ void draw_peaks(uint32_t ge, uint32_t gl, uint32_t ro
 // Events of one peak on the R rows of a tile in the x-direction form: every row differenced along
 // x0 (entered at its first column, left after its last), so a row costs two events whatever the
 // shift per row; an interval entering from the left of the tile counts in that row's carry.
-template <int R>
+template <int R, bool ONE>
 __device__ __forceinline__ void draw_peak_x(uint32_t ge, uint32_t gl, uint32_t row_bytes, int64_t a,
                                             int64_t b1, int64_t s, int C, int ub, int (&carry)[R]) {
 #pragma unroll
@@ -266,7 +266,7 @@ __device__ __forceinline__ void draw_peak_x(uint32_t ge, uint32_t gl, uint32_t r
     if (o1 <= hi) {
       if (lo < 0) carry[rr] += 1;
       else inc_shared(ge + rr * row_bytes + 4u * (uint32_t)o1);
-      if (hi < C - 1) inc_shared(gl + rr * row_bytes + 4u * (uint32_t)(hi + 1));
+      if (hi < C - 1) leave_shared<ONE>(gl + rr * row_bytes + 4u * (uint32_t)(hi + 1));
     }
     a -= s;
     b1 -= s;
@@ -364,7 +364,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
   const int C = t.ncols;
   const int lds = C + kHoughPad;                 // row stride
   const int words = (XD ? R : t.nrows) * lds;
-  const bool one = !XD && t.one;
+  const bool one = t.one;
   const int gap = one ? 0 : words;               // from the columns entered to the columns left
   int* tot = reinterpret_cast<int*>(smem);
   int* wsum = tot;                               // the warps' sums while windows are laid out
@@ -402,7 +402,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
     const FftRow* const SD = md.SD;
     const int64_t* const Bt = md.B;
     const longlong2* const UP = md.UP + bin0;
-    const bool window = !XD && !(state & kListFftUnsorted);
+    const bool window = !(state & kListFftUnsorted);
     for (int q0 = 0; q0 < (fits ? nbw : 0); q0 += batch) {
       const int nq = min(batch, nbw - q0);
       // per bin (one thread each): its peaks that have an edge in the tile, in one or two pieces
@@ -431,7 +431,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
           st1 += o0;
           cnt1 = o1 - o0;
           // the FFTs that cover the tile on every row are counted without a walk
-          if (w.c_lo < w.c_hi && cnt1 > 0) {
+          if (!XD && w.c_lo < w.c_hi && cnt1 > 0) {
             const int m1 = max(to(w.c_lo + 1), o0);
             const int m2 = min(from(past ? min(w.c_hi, md.n_fft - 1) : w.c_hi), o1);
             if (m1 < m2) {
@@ -533,7 +533,11 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
         has_nx = v + 2 * kLane < vend;
         if (has_nx) fetch(v + 2 * kLane, f_nx, j_nx);
         if constexpr (XD) {
-          if (ok) draw_peak_x<R>(ge, gl, row_bytes, a, b1, s, C, ub, carry_x);
+          // the interval meets the tile on some row (see draw_peaks)
+          if (ok && (b1 >> GFH_FRAC_BITS) >= 0 && ((a - (R - 1) * s) >> GFH_FRAC_BITS) <= ub) {
+            if (one) draw_peak_x<R, true>(ge, gl, row_bytes, a, b1, s, C, ub, carry_x);
+            else draw_peak_x<R, false>(ge, gl, row_bytes, a, b1, s, C, ub, carry_x);
+          }
         } else {
           if (one) draw_peaks<true>(ge, gl, row_bytes, spare, own, t.nrows, C, ub, ok, a, b1, s, d, carry);
           else draw_peaks<false>(ge, gl, row_bytes, spare, own, t.nrows, C, ub, ok, a, b1, s, d, carry);
@@ -559,8 +563,8 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
   }
   __syncthreads();
 
-  // ---- running sums along x0, in place: row 0 only, or every row (XD).  A chunk is 128 columns
-  // (32 lanes x 4).
+  // ---- running sums along x0: of row 0 in place, of every row (XD) as it is stored.  A chunk is 128
+  // columns (32 lanes x 4).
   const int nch = (C + 127) / 128;
   const int nsum = XD ? t.nrows * nch : nch;
   auto load4 = [&](const int* g) {               // entered - left
@@ -581,20 +585,21 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
     if (lane == 0) tot[rr * kLane + ch] = s;
   }
   __syncthreads();
-  for (int idx = warp; idx < nsum; idx += NW) {
-    const int rr = idx / nch, ch = idx - rr * nch;
-    const int col = ch * 128 + lane * 4;
-    const int before = warp_sum((lane < ch) ? tot[rr * kLane + lane] : 0);
-    int4 g = make_int4(0, 0, 0, 0);
-    if (col < C) g = load4(&G[rr * lds + col]);
-    g.y += g.x; g.z += g.y; g.w += g.z;
-    const int add = before + warp_incl_scan(g.w, lane) - g.w;
-    if (col < C) {
-      *reinterpret_cast<int4*>(&G[rr * lds + col]) = make_int4(g.x + add, g.y + add, g.z + add, g.w + add);
-      if (!one) *reinterpret_cast<int4*>(&G[rr * lds + col + gap]) = make_int4(0, 0, 0, 0);
+  if (!XD) {
+    for (int ch = warp; ch < nch; ch += NW) {
+      const int col = ch * 128 + lane * 4;
+      const int before = warp_sum((lane < ch) ? tot[lane] : 0);
+      int4 g = make_int4(0, 0, 0, 0);
+      if (col < C) g = load4(&G[col]);
+      g.y += g.x; g.z += g.y; g.w += g.z;
+      const int add = before + warp_incl_scan(g.w, lane) - g.w;
+      if (col < C) {
+        *reinterpret_cast<int4*>(&G[col]) = make_int4(g.x + add, g.y + add, g.z + add, g.w + add);
+        if (!one) *reinterpret_cast<int4*>(&G[col + gap]) = make_int4(0, 0, 0, 0);
+      }
     }
+    __syncthreads();
   }
-  __syncthreads();
 
   // ---- running sums along k; store; candidates.  A tile of few chunks is split into segments of
   // rows so that every warp has a share: first the column sums of all segments but the last (kept
@@ -620,7 +625,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
   // Candidates.  A tile with columns of at most kFewBands bands (wide bins) first takes each band's
   // largest count only, and looks for its cell in a second walk over the sums if it can win over the
   // map's best so far; with many bands every column tracks its best cell in the one walk.
-  const bool few = nb_tile <= kFewBands;
+  const bool few = !XD && nb_tile <= kFewBands;
   uint64_t s1 = 0, s2 = 0;
   const uint32_t W32 = (uint32_t)md.W;
   // map fields of the store pass read once (a global store could otherwise force a reload)
@@ -636,7 +641,8 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
         const int4 bv = __ldg(reinterpret_cast<const int4*>(col_band + col));
         band[0] = bv.x; band[1] = bv.y; band[2] = bv.z; band[3] = bv.w;
       }
-      const bool any = SELECT && (band[0] & band[1] & band[2] & band[3]) != -1;
+      bool any = SELECT && (band[0] & band[1] & band[2] & band[3]) != -1;
+      if (XD) any = __any_sync(0xffffffffu, any);  // the warp stays together: it scans every row
       const bool all = SELECT && (band[0] | band[1] | band[2] | band[3]) >= 0;
       int4 v = make_int4(0, 0, 0, 0);
       if (!XD && in)
@@ -644,20 +650,31 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
           const int4 g = *reinterpret_cast<const int4*>(seg_sum + q * C + col);
           v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w;
         }
-      const int rb = sg * seg_rows, re = in ? min(rb + seg_rows, t.nrows) : rb;
+      const int rb = sg * seg_rows, re = XD || in ? min(rb + seg_rows, t.nrows) : rb;
       const int* g0 = G + rb * lds + col;
+      const int* tot0 = tot + rb * kLane;
       auto next = [&]() {
-        const int4 g = load4(g0);
+        if (!XD) {
+          const int4 g = load4(g0);
+          v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w;
+        } else {
+          int4 g = make_int4(0, 0, 0, 0);
+          if (in) g = load4(g0);
+          const int before = warp_sum(lane < u - sg * nch ? tot0[lane] : 0);
+          tot0 += kLane;
+          g.y += g.x; g.z += g.y; g.w += g.z;
+          const int add = before + warp_incl_scan(g.w, lane) - g.w;
+          v = make_int4(g.x + add, g.y + add, g.z + add, g.w + add);
+        }
         g0 += lds;
-        if (XD) v = g;
-        else { v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w; }
       };
       if (pass == 1) {                             // the cells that hold a sought band's best count
         int want[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           want[q] = band[q] >= 0 && s_seek[band[q] - t.band_lo] ? s_best[band[q] - t.band_lo] : -1;
-        if ((want[0] & want[1] & want[2] & want[3]) == -1) continue;
+        const bool none = (want[0] & want[1] & want[2] & want[3]) == -1;
+        if (XD ? __all_sync(0xffffffffu, none) : none) continue;
         for (int rr = rb; rr < re; ++rr) {
           next();
           const int vals[4] = {v.x, v.y, v.z, v.w};
@@ -690,14 +707,14 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
       if (!any) {
         for (int rr = rb; rr < re; ++rr) {
           next();
-          __stcs(reinterpret_cast<int4*>(o), v);
+          if (!XD || in) __stcs(reinterpret_cast<int4*>(o), v);
           o += ld_out;
         }
       } else if (few) {
         int best[4] = {0, 0, 0, 0};
         for (int rr = rb; rr < re; ++rr) {
           next();
-          __stcs(reinterpret_cast<int4*>(o), v);
+          if (!XD || in) __stcs(reinterpret_cast<int4*>(o), v);
           o += ld_out;
           sums();
           best[0] = max(best[0], v.x); best[1] = max(best[1], v.y);
@@ -716,7 +733,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
         int bc[4] = {-1, -1, -1, -1}, br[4] = {0, 0, 0, 0};
         for (int rr = rb; rr < re; ++rr) {
           next();
-          __stcs(reinterpret_cast<int4*>(o), v);
+          if (!XD || in) __stcs(reinterpret_cast<int4*>(o), v);
           o += ld_out;
           sums();
           const int vals[4] = {v.x, v.y, v.z, v.w};
@@ -765,7 +782,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
 // together.  The index of a block's next tile is claimed when it starts a tile and read when it has
 // finished it, so the atomic's round trip is hidden behind the tile.
 template <int R, int NT, bool SELECT, bool XD>
-__global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
+__global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
 k_hough(const MapDev* __restrict__ maps, const TileDev* __restrict__ tiles, int n_tiles,
         const int* __restrict__ count, int* __restrict__ next, const uint32_t* __restrict__ fft_idx,
         const int* __restrict__ list_state, unsigned int* __restrict__ flag, int sum_off, int batch) {
@@ -930,28 +947,14 @@ int launch_hough_t(gfh_plan* p, const gfh_peaks* peaks, int which) {
   return GFH_OK;
 }
 
-// The kernels of a plan: f(rows, threads, XD) as compile-time constants.  Only the x-direction form
-// takes the given shape as it is.
+// The kernels of a plan: f(rows, threads, XD) as compile-time constants.
 template <class F>
 int with_kernel(const gfh_plan* p, int which, F f) {
-  if (which != kFullX) {
-    const std::integral_constant<int, 1> any{};
-    if ((which == kList ? p->list_threads : p->threads) == 256)
-      return f(any, std::integral_constant<int, 256>{}, std::false_type{});
-    return f(any, std::integral_constant<int, 512>{}, std::false_type{});
-  }
-  auto threads = [&](auto rows) -> int {
-    if (p->cfg.threads == 256) return f(rows, std::integral_constant<int, 256>{}, std::true_type{});
-    if constexpr (decltype(rows)::value >= 16)
-      if (p->cfg.threads == 1024) return f(rows, std::integral_constant<int, 1024>{}, std::true_type{});
-    return f(rows, std::integral_constant<int, 512>{}, std::true_type{});
-  };
-  switch (p->cfg.rows) {
-    case 4: return threads(std::integral_constant<int, 4>{});
-    case 8: return threads(std::integral_constant<int, 8>{});
-    case 16: return threads(std::integral_constant<int, 16>{});
-    default: return threads(std::integral_constant<int, 32>{});
-  }
+  const std::integral_constant<int, 256> t256{};
+  const std::integral_constant<int, 1> any{};
+  if (which == kFullX) return f(std::integral_constant<int, kRowsX>{}, t256, std::true_type{});
+  if ((which == kList ? p->list_threads : p->threads) == 256) return f(any, t256, std::false_type{});
+  return f(any, std::integral_constant<int, 512>{}, std::false_type{});
 }
 
 int launch_hough(gfh_plan* p, const gfh_peaks* peaks, int which) {

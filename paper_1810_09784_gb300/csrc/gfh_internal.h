@@ -23,6 +23,7 @@ constexpr size_t kHoughSmemLimit = kMaxSmemBytes - 64;
 constexpr int kHoughPad = 4;
 // Room of a tile (words) with one, two or three blocks per SM; about 43, 15 and 10 KB of a block's shared
 // memory are left for its chunk sums, band keys and windows.
+constexpr int kRowsX = 8;   // k rows of a tile in the x-direction form
 constexpr int64_t kRoom[4] = {0, 47104, 25088, 16448};
 
 // Counter-based generator of the statistical peakmap model: the splitmix64 finaliser (Steele, Lea

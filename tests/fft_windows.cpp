@@ -29,7 +29,7 @@ int main() {
     if (gfh_host_tables(&g, hm.U, hm.B, hm.S) || gfh_host_columns(&g, hm.band, hm.f0, hm.f0n)) return 1;
     find_analysis_columns(hm);
     std::vector<TileDev> tiles;
-    hm.one = sparse_map(g);
+    hm.one = sparse_map(g, false);
     if (rows > 0) {
       cut_tiles(g, hm, 0, 0, g.n_k, 0, g.ld_x0, rows, cols, tiles);
     } else {
