@@ -810,15 +810,17 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   const int n_tiles_k = (int)tiles.size();
   tiles.insert(tiles.end(), tiles_x.begin(), tiles_x.end());
 
-  // FFT blocks of 64, or longer so that a bin has at most 256 of them
+  // FFT blocks of 16 to 64, as fine as one per lane of the warp that looks a bin's up allows (a window's
+  // ends are read by whole blocks: 2118 rows x 2540 columns of 652 FFTs 75 -> 71 us); longer ones only
+  // so that a bin has at most 256.
   std::vector<ListDev> lists;
   std::map<int, int> list_at;
   int64_t csr_entries = 0;
   for (auto& kv : by_list) {
     ListDev ld = kv.second;
     ld.n_bins -= ld.bin_lo;
-    ld.shift = 6;
-    while (((list_ffts[kv.first] - 1) >> ld.shift) + 1 > 256) ++ld.shift;
+    ld.shift = 4;
+    while (((list_ffts[kv.first] - 1) >> ld.shift) + 1 > (ld.shift < 6 ? 32 : 256)) ++ld.shift;
     ld.nb1 = ((list_ffts[kv.first] - 1) >> ld.shift) + 2;
     if (csr_entries + ld.n_bins > INT32_MAX) return GFH_ERR_SIZE;
     ld.entry0 = (int32_t)csr_entries;
