@@ -23,7 +23,10 @@
  *     device flag that gfh_check() reads and clears; the GPU context stays usable.
  *   - Peak lists are two parallel uint32 arrays: fft_idx (FFT number i, time t_i = t_first +
  *     i * t_hop from t0) and bin (frequency bin j, f_j = j * df), sorted by bin ascending (the
- *     order within one bin is free).  A peakmap never has two peaks in one (FFT, bin) cell.
+ *     order within one bin is free: tiles read of each bin the FFTs that can have an edge in them,
+ *     and a list whose bins are not in FFT order, as gfh_peakmap emits them, is ordered into the
+ *     plan's memory on the way, which has room for a peak in every eighth (FFT, bin) cell of the
+ *     maps' bins; denser ones are read in full, with the same results).  A peakmap never has two peaks in one (FFT, bin) cell.
  *   - A Hough map is int32 [n_k][ld_x0] row-major: row r is k_r = k_min + r dk, column m is the
  *     x0 interval [x0_min + m dx0, x0_min + (m+1) dx0).  Columns n_x0 .. ld_x0-1 are written 0.
  */
@@ -585,10 +588,8 @@ int gfh_conv3x3(gfh_ctx* ctx, int32_t mode, int32_t cin, int32_t cout, int32_t s
  * in one launch of persistent blocks.  Candidates are the best computed cell of each band (count
  * -1 where no cell of the band was computed).  cr and the statistics come from sums over the
  * computed cells only (a cell computed twice counts twice) with the map's full cell count: they
- * are comparable with those of gfh_plan_execute only for maps searched in full.  A peak list whose
- * bins hold their peaks in FFT order (as gfh_peakmap emits them) lets tiles read only the peaks of
- * the FFTs that can have an edge in them; any other bin-sorted list is read in full, with the same
- * results.  Asynchronous, allocation-free, capturable.
+ * are comparable with those of gfh_plan_execute only for maps searched in full.
+ * Asynchronous, allocation-free, capturable.
  */
 int gfh_plan_set_coarse(gfh_plan* plan, int32_t coarse_k, int32_t coarse_x, int32_t max_sel);
 int gfh_plan_execute_tiles(gfh_plan* plan, const gfh_peaks* peaks, const int32_t* d_coarse,

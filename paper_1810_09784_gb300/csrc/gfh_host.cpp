@@ -762,7 +762,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
     int64_t ana_cols = 0;
     for (int64_t c = 0; c < g.n_x0; ++c) ana_cols += hm.band[c] >= 0;
     hm.cells = ana_cols * g.n_k;
-    auto ins = by_list.insert({g.list, ListDev{nullptr, nullptr, g.list, g.bin_lo, g.bin_hi + 1, 0, 0, 0}});
+    auto ins = by_list.insert({g.list, ListDev{nullptr, nullptr, g.list, g.bin_lo, g.bin_hi + 1, 0, 0, 0, nullptr, 0}});
     ListDev& ld = ins.first->second;             // n_bins holds the end of the bins for now
     ld.bin_lo = std::min(ld.bin_lo, g.bin_lo);
     ld.n_bins = std::max(ld.n_bins, g.bin_hi + 1);
@@ -815,16 +815,19 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   // so that a bin has at most 256.
   std::vector<ListDev> lists;
   std::map<int, int> list_at;
-  int64_t csr_entries = 0;
+  int64_t csr_entries = 0, copy_words = 0;
   for (auto& kv : by_list) {
     ListDev ld = kv.second;
     ld.n_bins -= ld.bin_lo;
     ld.shift = 4;
-    while (((list_ffts[kv.first] - 1) >> ld.shift) + 1 > (ld.shift < 6 ? 32 : 256)) ++ld.shift;
+    while (((list_ffts[kv.first] - 1) >> ld.shift) + 1 > (ld.shift < 6 ? 32 : kMaxFftBlocks)) ++ld.shift;
     ld.nb1 = ((list_ffts[kv.first] - 1) >> ld.shift) + 2;
     if (csr_entries + ld.n_bins > INT32_MAX) return GFH_ERR_SIZE;
     ld.entry0 = (int32_t)csr_entries;
     csr_entries += ld.n_bins;
+    // room to order a list out of FFT order: an eighth of its (FFT, bin) pairs, noise peaks and more
+    ld.cap = (int64_t)ld.n_bins * list_ffts[kv.first] / 8 + 1024;
+    copy_words += ld.cap;
     list_at[kv.first] = (int)lists.size();
     lists.push_back(ld);
   }
@@ -874,14 +877,22 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   p->cells = cells;
   p->cells_x = cells_x;
   if (cudaSetDevice(ctx->device) != cudaSuccess) { delete p; return GFH_ERR_CUDA; }
-  if (cudaMalloc(&p->d_buf, total) != cudaSuccess) { delete p; return GFH_ERR_NOMEM; }
+  // the room to order lists follows what is filled here; without it they are walked whole
+  if (cudaMalloc(&p->d_buf, total + (size_t)copy_words * sizeof(uint32_t)) != cudaSuccess) {
+    cudaGetLastError();
+    for (ListDev& ld : lists) ld.cap = 0;
+    if (cudaMalloc(&p->d_buf, total) != cudaSuccess) { delete p; return GFH_ERR_NOMEM; }
+  }
   p->buf_bytes = total;
   char* base = (char*)p->d_buf;
   std::vector<char> h(total, 0);
   std::vector<MapDev> mds(n_maps);
   std::vector<int32_t> csr_list;
   csr_list.reserve(csr_entries);
+  uint32_t* copy = (uint32_t*)(base + total);
   for (size_t l = 0; l < lists.size(); ++l) {
+    lists[l].copy = copy;
+    copy += lists[l].cap;
     lists[l].csr = (int64_t*)(base + o_csr[l]);
     lists[l].blk = (int32_t*)(base + o_blk[l]);
     csr_list.insert(csr_list.end(), lists[l].n_bins, (int32_t)l);
@@ -902,6 +913,8 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
     const ListDev& ld = lists[list_at[g.list]];
     md.csr = ld.csr + (g.bin_lo - ld.bin_lo);
     md.blk = ld.blk + (size_t)(g.bin_lo - ld.bin_lo) * ld.nb1;
+    md.csr_list = ld.csr;
+    md.copy = ld.copy;
     md.nb1 = ld.nb1;
     md.shift = ld.shift;
     md.keys = (unsigned long long*)(base + o_keys) + key_off;

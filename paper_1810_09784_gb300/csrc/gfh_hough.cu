@@ -17,7 +17,10 @@
 namespace {
 
 constexpr int kLane = 32;
-constexpr int kListUnsorted = 1, kListFftUnsorted = 2;   // bits of a peak list's order state
+// Bits of a peak list's order state: bins not ascending, some bin's peaks not in FFT order, and no copy
+// of its FFT indices by blocks of FFTs.
+constexpr int kListUnsorted = 1, kListFftUnsorted = 2, kListNoCopy = 4;
+constexpr int kIndexWarps = 8;   // bins per block of k_index
 constexpr int kFewBands = 4;     // a tile of at most this many bands looks for its best cells only if they can win
 template <int NT> constexpr int kSumBytes = NT / kLane * 16;   // two sums per warp
 constexpr int kRowBits = 57;     // fraction bits of an event's row
@@ -55,7 +58,7 @@ __device__ __forceinline__ unsigned long long cand_key(int count, uint32_t lin) 
 
 // Order of each peak list (state[l], l < n_states, zeroed before): kListUnsorted when its bins are not ascending
 // (also flagged; such a list is not drawn), kListFftUnsorted when some bin's peaks are not in FFT
-// order (the tiles then read all peaks of their bins).
+// order (k_index then copies them by blocks of FFTs).
 __global__ void k_check_sorted(const uint32_t* __restrict__ bins, const uint32_t* __restrict__ fft,
                                const int64_t* __restrict__ off, unsigned int* flag,
                                int* __restrict__ state, int n_states) {
@@ -78,13 +81,66 @@ __global__ void k_check_sorted(const uint32_t* __restrict__ bins, const uint32_t
   if (bad && l < n_states) atomicOr(&state[l], bad);
 }
 
-// Index of the peak lists, one warp per (list, bin): csr = the bin's first peak (by a 32-way search
-// of the list, five bits a step), and per block of 2^shift FFTs the offset inside the bin of its
-// first peak with FFT index in that block or later (meaningful where the bin is in FFT order).
-__global__ void k_index(const ListDev* __restrict__ lists, const int32_t* __restrict__ entry_list,
-                        int n_entries, const uint32_t* __restrict__ bins,
-                        const uint32_t* __restrict__ fft, const int64_t* __restrict__ off) {
-  const int e = blockIdx.x * (blockDim.x / kLane) + (threadIdx.x >> 5);
+// First of the list's peaks [lo, hi) with bin >= key, by the whole warp (a 32-way search, five bits a
+// step).
+__device__ __forceinline__ int64_t first_of_bin(const uint32_t* __restrict__ bins, int64_t lo, int64_t hi,
+                                                uint32_t key, int lane) {
+  while (lo < hi) {
+    const int64_t step = (hi - lo) / kLane + 1;    // probes lo + step (lane + 1) - 1
+    const int64_t at = lo + step * (lane + 1) - 1;
+    const bool less = at < hi && bins[at] < key;
+    const int64_t l = lo + step * __popc(__ballot_sync(0xffffffffu, less));
+    hi = min(hi, l + step - 1);
+    lo = l;
+  }
+  return lo;
+}
+
+// A bin's n FFT indices f out of order: copied to dst by blocks of 2^shift FFTs, in any order inside one
+// (the tiles read whole blocks), the largest last; begin[b], b < nb1: first of block b.  h: nb1 + 1
+// words of the warp's.
+__device__ __forceinline__ void order_bin(const uint32_t* __restrict__ f, int n, int nb1, int shift,
+                                          int32_t* __restrict__ begin, uint32_t* __restrict__ dst, int* h,
+                                          int lane) {
+  for (int b = lane; b <= nb1; b += kLane) h[b] = 0;
+  __syncwarp();
+  uint32_t top = 0;
+  for (int i = lane; i < n; i += kLane) {
+    const uint32_t v = f[i];
+    top = max(top, v);
+    atomicAdd(&h[min(v >> shift, (uint32_t)(nb1 - 1))], 1);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  __syncwarp();
+  int before = 0;
+  for (int b0 = 0; b0 < nb1; b0 += kLane) {
+    const int b = b0 + lane, c = b < nb1 ? h[b] : 0, incl = warp_incl_scan(c, lane);
+    if (b < nb1) {
+      h[b] = before + incl - c;
+      begin[b] = b + 1 < nb1 ? before + incl - c : n;
+    }
+    before += __shfl_sync(0xffffffffu, incl, kLane - 1);
+  }
+  __syncwarp();
+  for (int i = lane; i < n; i += kLane) {
+    const uint32_t v = f[i];
+    const bool last = v == top && atomicExch(&h[nb1], 1) == 0;
+    dst[last ? n - 1 : atomicAdd(&h[min(v >> shift, (uint32_t)(nb1 - 1))], 1)] = v;
+  }
+}
+
+// Index of the peak lists, one warp per (list, bin): csr = the bin's first peak, and per block of
+// 2^shift FFTs the offset inside the bin of its first peak with FFT index in that block or later.  The
+// bins of a list out of FFT order are also copied by blocks, so that its tiles have their windows too:
+// walked whole by the tiles planned for windows, such lists took up to 4.4 times as long (paper-shaped
+// maps 20.3 ms for 4.64 in order, now 4.69; one half-hour map 186 us for 102, now 105).  A list of more
+// peaks than the copy holds keeps none; its bins are walked whole.
+__global__ void __launch_bounds__(kIndexWarps * kLane)
+k_index(const ListDev* __restrict__ lists, const int32_t* __restrict__ entry_list, int n_entries,
+        const uint32_t* __restrict__ bins, const uint32_t* __restrict__ fft, const int64_t* __restrict__ off,
+        int* __restrict__ state) {
+  __shared__ int s_h[kIndexWarps][kMaxFftBlocks + 2];
+  const int e = blockIdx.x * kIndexWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (e >= n_entries) return;
   const ListDev& ld = lists[entry_list[e]];
@@ -113,6 +169,16 @@ __global__ void k_index(const ListDev* __restrict__ lists, const int32_t* __rest
     if (jl == ld.n_bins - 1) ld.csr[jl + 1] = lo[1];
   }
   const int n = (int)(lo[1] - lo[0]);
+  int32_t* const begin = ld.blk + (int64_t)jl * ld.nb1;
+  const int st = state[ld.list];
+  if ((st & kListFftUnsorted) && !(st & kListUnsorted)) {
+    const int64_t at = lo[0] - first_of_bin(bins, off[ld.list], off[ld.list + 1], (uint32_t)ld.bin_lo, lane);
+    if (at + n <= ld.cap)
+      order_bin(fft + lo[0], n, ld.nb1, ld.shift, begin, ld.copy + at, s_h[threadIdx.x >> 5], lane);
+    else if (lane == 0)
+      atomicOr(&state[ld.list], kListNoCopy);
+    return;
+  }
   for (int b = lane; b < ld.nb1; b += kLane) {
     const uint32_t key = (uint32_t)b << ld.shift;
     int l = 0, h = b + 1 < ld.nb1 ? n : 0;
@@ -120,7 +186,7 @@ __global__ void k_index(const ListDev* __restrict__ lists, const int32_t* __rest
       const int mid = (l + h) >> 1;
       if (__ldg(fft + lo[0] + mid) < key) l = mid + 1; else h = mid;
     }
-    ld.blk[(int64_t)jl * ld.nb1 + b] = b + 1 < ld.nb1 ? l : n;
+    begin[b] = b + 1 < ld.nb1 ? l : n;
   }
 }
 
@@ -334,7 +400,8 @@ __device__ __forceinline__ void fill_tile(const MapDev& md, const TileDev& t, in
 // FFTs' shifts spread far wider than a bin, so of each bin only the FFTs of one window have an edge
 // in the tile: the window comes from the line that the shifts follow, its peaks from the list's
 // index (k_index), and only those are walked (whole blocks of FFTs, so a few beside them too).
-// Peak lists that are not in FFT order inside a bin read whole bins.  The windows of up to `batch`
+// Peak lists that are not in FFT order inside a bin read their copy by blocks of FFTs, or whole bins
+// where the list has none.  The windows of up to `batch`
 // bins at a time are laid end to end, two pieces per bin: ent[] = {end of the piece in that order,
 // where its peaks lie in the list less its begin}.  Each warp walks one contiguous part, 32 peaks at
 // a time whatever bins they are of.  A tile that no edge meets holds one number and needs no sums.
@@ -397,12 +464,13 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
     // flag and is not drawn)
     const bool fits = md.csr[bin0 + nbw] - pb <= (int64_t)0x7fffffff - (1 << 20);
     if (!fits && tid == 0) atomicOr(flag, GFH_FLAG_CAPACITY);
-    const uint32_t* const fl = fft_idx + pb;
+    const bool copied = (state & (kListFftUnsorted | kListNoCopy)) == kListFftUnsorted;
+    const uint32_t* const fl = copied ? md.copy + (pb - *md.csr_list) : fft_idx + pb;
     const uint32_t nfft = (uint32_t)md.n_fft;
     const FftRow* const SD = md.SD;
     const int64_t* const Bt = md.B;
     const longlong2* const UP = md.UP + bin0;
-    const bool window = !(state & kListFftUnsorted);
+    const bool window = copied || !(state & kListFftUnsorted);
     for (int q0 = 0; q0 < (fits ? nbw : 0); q0 += batch) {
       const int nq = min(batch, nbw - q0);
       // per bin (one thread each): its peaks that have an edge in the tile, in one or two pieces
@@ -416,7 +484,7 @@ __device__ __forceinline__ void hough_tile(const MapDev* __restrict__ maps, cons
           const longlong2 up = __ldg(UP + q);
           const int32_t* const blk = md.blk + (int64_t)(bin0 + q) * md.nb1;
           const int n = cnt1;
-          // indices past the table are flagged; they end the bin and are drawn nowhere
+          // indices past the table are flagged and drawn nowhere; the last is the largest
           const bool past = __ldg(fl + st1 + n - 1) >= nfft;
           if (past) atomicOr(flag, GFH_FLAG_FFT_RANGE);
           // first peaks of the FFT block that holds FFT i, and of the first block that starts there
@@ -1017,8 +1085,8 @@ static int launch_prologue(gfh_plan* p, const gfh_peaks* peaks) {
                                          p->d_list_state, p->n_list_states);
     GFH_CUDA_TRY(cudaGetLastError());
   }
-  k_index<<<(p->csr_entries + 7) / 8, 256, 0, st>>>(p->d_lists, p->d_csr_list, p->csr_entries,
-                                                    peaks->bin, peaks->fft_idx, peaks->offsets);
+  k_index<<<(p->csr_entries + kIndexWarps - 1) / kIndexWarps, kIndexWarps * kLane, 0, st>>>(
+      p->d_lists, p->d_csr_list, p->csr_entries, peaks->bin, peaks->fft_idx, peaks->offsets, p->d_list_state);
   GFH_CUDA_TRY(cudaGetLastError());
   return GFH_OK;
 }

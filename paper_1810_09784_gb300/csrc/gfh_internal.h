@@ -180,6 +180,8 @@ struct MapDev {
   const int64_t* csr;       // J + 1 entries: first peak (absolute index) of bins bin_lo .. bin_hi+1
   const int32_t* blk;       // [J][nb1]: offset in a bin's peaks of its first of FFT >= 2^shift b
   int32_t nb1, shift;
+  const int64_t* csr_list;  // first peak of the list's first indexed bin
+  const uint32_t* copy;     // the list's FFT indices from there, by blocks (lists out of FFT order)
   unsigned long long* keys; // n_bands
   unsigned long long* sums; // 2: sum, sum of squares
   gfh_candidate* cands;     // n_bands (may be null)
@@ -196,12 +198,17 @@ struct MapDev {
   ShiftLine line;           // a bin's windows of FFTs
 };
 
+// FFT blocks of a bin, at most.
+constexpr int kMaxFftBlocks = 256;
+
 // The index of one peak list, over the bins that some map reads (built per execute, k_index).
 struct ListDev {
   int64_t* csr;             // n_bins + 1
   int32_t* blk;             // [n_bins][nb1]
   int32_t list, bin_lo, n_bins, nb1, shift;
   int32_t entry0;           // its first bin in the plan-wide numbering
+  uint32_t* copy;           // room for the FFT indices of `cap` peaks
+  int64_t cap;
 };
 
 // One tile of the accumulation kernel: k rows [row0, row0+nrows) x columns [col0, col0+ncols).
