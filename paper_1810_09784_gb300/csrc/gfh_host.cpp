@@ -18,8 +18,6 @@ namespace {
 
 int64_t fixed_floor(double v) { return (int64_t)std::floor(std::ldexp(v, GFH_FRAC_BITS)); }
 
-int64_t floor_shift(int64_t v) { return v >> GFH_FRAC_BITS; }  // arithmetic shift = floor
-
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // n = 0 selects the original FrequencyHough (Sec. III Eq. fdotslope): x = -f, x0 = -f0 and
@@ -438,22 +436,24 @@ void tile_bins(const gfh_grid& g, const HostMap& hm, int64_t s_min, int64_t s_ma
                int64_t c1, int32_t* ja, int32_t* jb) {
   const int J = g.bin_hi - g.bin_lo + 1;
   if (c0 > g.n_x0 - 1) { *ja = 1; *jb = 0; return; }
-  // smallest jl with floor((U[jl+1]-s_max)) <= c1-1
-  int lo = 0, hi = J;  // answer in [0, J]; J means none
-  while (lo < hi) {
-    int mid = (lo + hi) / 2;
-    if (floor_shift(hm.U[mid + 1] - s_max) <= c1 - 1) hi = mid; else lo = mid + 1;
+  // (selected and not branched to: a plan makes thousands of tiles, and half the branches of a bisection
+  // are mispredicted)
+  const int64_t right = c1 << GFH_FRAC_BITS, left = c0 << GFH_FRAC_BITS;
+  int a = 0, b = 0;                      // first bins with U[jl+1] - s_max < right, U[jl] - s_min <= left
+  for (int n = J; n > 0;) {
+    const int half = n / 2;
+    const bool more = hm.U[a + half + 1] - s_max >= right;
+    a = more ? a + half + 1 : a;
+    n = more ? n - half - 1 : half;
   }
-  const int a = lo;
-  // largest jl with floor((U[jl]-s_min-1)) >= c0
-  lo = -1; hi = J - 1;  // answer in [-1, J-1]
-  while (lo < hi) {
-    int mid = (lo + hi + 1) / 2;
-    if (floor_shift(hm.U[mid] - s_min - 1) >= c0) lo = mid; else hi = mid - 1;
+  for (int n = J; n > 0;) {
+    const int half = n / 2;
+    const bool more = hm.U[b + half] - s_min - 1 >= left;
+    b = more ? b + half + 1 : b;
+    n = more ? n - half - 1 : half;
   }
-  const int b = lo;
   *ja = g.bin_lo + a;
-  *jb = g.bin_lo + b;
+  *jb = g.bin_lo + b - 1;
 }
 
 // Candidate bands of columns [c0, c1) (bands follow the columns): lo > hi when there is none.
@@ -509,33 +509,34 @@ double tile_work(const gfh_grid& g, const HostMap& hm, const TileDev& t) {
   const double e0 = (double)(hm.B[n - 1] + r0 * hm.S[n - 1]) * one,
                e1 = (double)(hm.B[n - 1] + r1 * hm.S[n - 1]) * one;
   const double s0 = n > 1 ? (e0 - b0) / (n - 1) : 0.0, s1 = n > 1 ? (e1 - b1) / (n - 1) : 0.0;
+  const double inv0 = s0 != 0.0 ? 1.0 / s0 : 0.0, inv1 = s1 != 0.0 ? 1.0 / s1 : 0.0;
   const int samples = std::min(nb, 8);
+  const double apart = samples > 1 ? (double)(nb - 1) / (samples - 1) : 0.0;
   double ffts = 0.0, moved = 0.0;
   for (int q = 0; q < samples; ++q) {
-    const int jl = t.bin_a - g.bin_lo + (int)((int64_t)q * (nb - 1) / std::max(1, samples - 1));
+    const int jl = t.bin_a - g.bin_lo + (int)(q * apart);
     const double hi_x = (double)hm.U[jl] * one - (double)t.col0;              // right edge
     const double lo_x = (double)hm.U[jl + 1] * one - (double)t.col0;          // left edge
     double lo = 0.0, hi = n;
-    auto at_most = [&](double x, double b, double s) {                        // b + i s <= x
-      if (s > 0.0) hi = std::min(hi, (x - b) / s);
-      else if (s < 0.0) lo = std::max(lo, (x - b) / s);
+    auto at_most = [&](double x, double b, double inv) {                      // b + i / inv <= x
+      if (inv > 0.0) hi = std::min(hi, (x - b) * inv);
+      else if (inv < 0.0) lo = std::max(lo, (x - b) * inv);
       else if (b > x) hi = lo;
     };
-    at_most(hi_x, b0, s0);                                                    // reaches the first column
-    at_most(-(lo_x - t.ncols), -b1, -s1);                                     // not past the last
+    at_most(hi_x, b0, inv0);                                                  // reaches the first column
+    at_most(-(lo_x - t.ncols), -b1, -inv1);                                   // not past the last
     double len = std::max(0.0, hi - lo);
     const double mid = 0.5 * (lo + hi);
     if (hi_x - lo_x > t.ncols && len > 0.0) {                                 // FFTs that cover the tile
       lo = 0.0;
       hi = n;
-      at_most(-(lo_x - 1.0), -b0, -s0);
-      at_most(hi_x - t.ncols, b1, s1);
+      at_most(-(lo_x - 1.0), -b0, -inv0);
+      at_most(hi_x - t.ncols, b1, inv1);
       len = std::max(0.0, len - std::max(0.0, hi - lo));
     }
     const double i = std::min(std::max(mid, 0.0), (double)(n - 1));
-    const double shift = t.nrows > 1 ? ((b1 - b0) + i * (s1 - s0)) / (t.nrows - 1) : 0.0;
     ffts += len;
-    moved += len * shift * (t.nrows - 1);
+    moved += len * ((b1 - b0) + i * (s1 - s0));
   }
   const double runs = kNoisePeaks / 32.0 * nb / samples;
   if (ffts <= 0.0) return fill;
@@ -582,6 +583,37 @@ void map_tiles(const gfh_grid& g, const HostMap& hm, int m, int64_t room, int r0
       tiles.insert(tiles.end(), best.begin(), best.end());
     }
   }
+}
+
+// One shape for all of map m, by the estimated time of a few sampled tiles of each: for a plan that is
+// executed once (map_tiles and balance_tiles take a few hundred us, more than they save one search).
+void sampled_tiles(const gfh_grid& g, const HostMap& hm, int m, int64_t room, int blocks,
+                   std::vector<TileDev>& tiles) {
+  const int64_t words = hm.one ? room : room / 2;
+  const int K = g.n_k;
+  int best_rows = 0, best_cols = 0;
+  double best = 0.0;
+  for (int rows = 8; rows <= 128; rows *= 2) {
+    const int nr = std::min(rows, K), most = cols_for(rows, words);
+    for (int cols = most; cols >= std::max(32, most / 4); cols = cols / 2 & ~3) {
+      const int64_t W = g.ld_x0, down = (K + nr - 1) / nr, across = (W + cols - 1) / cols;
+      double sum = 0.0, longest = 0.0;
+      int n = 0;
+      for (int64_t i = 0; i < std::min<int64_t>(down, 4); ++i)
+        for (int64_t j = 0; j < std::min<int64_t>(across, 4); ++j, ++n) {
+          const int64_t r = down > 1 ? i * (down - 1) / (std::min<int64_t>(down, 4) - 1) * nr : 0;
+          const int64_t c = across > 1 ? j * (across - 1) / (std::min<int64_t>(across, 4) - 1) * cols : 0;
+          const double w = tile_work(g, hm, make_tile(g, hm, m, (int)r, (int)std::min<int64_t>(nr, K - r), c,
+                                                      (int)std::min<int64_t>(cols, W - c)));
+          sum += w;
+          longest = std::max(longest, w);
+        }
+      const double time = sum / n * (double)(down * across) / blocks + 0.5 * longest;
+      if (best_rows == 0 || time < best) { best = time; best_rows = nr; best_cols = cols; }
+    }
+    if (rows >= K) break;
+  }
+  cut_tiles(g, hm, m, 0, K, 0, g.ld_x0, best_rows, best_cols, tiles);
 }
 
 // Halves the tiles that hold more than `most` work, across columns or rows as makes the least of it.
@@ -631,23 +663,29 @@ void balance_tiles(const std::vector<gfh_grid>& grids, const std::vector<HostMap
                    std::vector<TileDev>& tiles, std::vector<double>& work) {
   if (tiles.empty()) return;
   // work per block, and half of the longest tile for the last wave
-  auto time = [&](double* longest) {
-    *longest = *std::max_element(work.begin(), work.end());
-    return std::accumulate(work.begin(), work.end(), 0.0) / blocks + 0.5 * *longest;
+  double all, longest;
+  auto time = [&]() {
+    all = std::accumulate(work.begin(), work.end(), 0.0);
+    longest = *std::max_element(work.begin(), work.end());
+    return all / blocks + 0.5 * longest;
   };
-  const double least = std::max(std::accumulate(work.begin(), work.end(), 0.0) / (3.0 * blocks), 12000.0);
-  double longest, best = time(&longest);
+  double best = time();
+  const double least = std::max(all / (3.0 * blocks), 12000.0);
   std::vector<TileDev> best_tiles = tiles;
   std::vector<double> best_work = work;
-  for (double most = longest; most > least;) {
+  // (a split only adds work: done once no longest tile could make up for what the splits so far added)
+  int worse = 0;
+  for (double most = longest; most > least && worse < 2 && all / blocks + 0.5 * least < best;) {
     most = std::max(0.7 * most, least);
     split_tiles(grids, hms, most, tiles, work);
-    const double now = time(&longest);
+    const double now = time();
+    ++worse;
     if (now < best) {
       best = now;
       best_tiles = tiles;
       best_work = work;
-    } else if (now > 1.2 * best) {
+      worse = 0;
+    } else if (now > 1.05 * best) {
       break;
     }
   }
@@ -718,6 +756,12 @@ SmShare sm_share(const gfh_tile_config& tc) {
   return SmShare{tc.threads, blocks, kRoom[blocks]};
 }
 
+// Whether two shapes make the same plan.  (The default's coarse tiles have a share of their own.)
+bool same_share(const gfh_tile_config& a, const gfh_tile_config& b) {
+  const SmShare x = sm_share(a), y = sm_share(b);
+  return x.threads == y.threads && x.blocks == y.blocks;
+}
+
 }  // namespace
 
 extern "C" int gfh_plan_destroy(gfh_plan* p) {
@@ -736,6 +780,12 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
                                int32_t* const* h_maps, gfh_candidate* const* h_cands,
                                gfh_map_stats* d_stats, const gfh_tile_config* cfg,
                                gfh_plan** out) {
+  return gfh_make_plan(ctx, n_maps, grids, h_maps, h_cands, d_stats, cfg, false, out);
+}
+
+int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* const* h_maps,
+                  gfh_candidate* const* h_cands, gfh_map_stats* d_stats, const gfh_tile_config* cfg,
+                  bool once, gfh_plan** out) {
   if (!ctx || !out || n_maps < 1 || !grids || !h_maps) return GFH_ERR_ARG;
   *out = nullptr;
   gfh_tile_config tc;
@@ -780,6 +830,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
       cfg_bands = std::max(cfg_bands, hi - lo + 1);
     }
     if (map_xd[m]) cells_xd += (double)g.n_k * (double)g.ld_x0;
+    else if (once) sampled_tiles(g, hm, m, share.room, share.blocks * ctx->num_sms, tiles);
     else map_tiles(g, hm, m, share.room, 0, g.n_k, 0, g.ld_x0, tiles);
   }
   // x-direction tiles: uniform strips of 8 rows, four and more to each block of three per SM as far as
@@ -802,7 +853,7 @@ extern "C" int gfh_plan_create(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* gri
   for (size_t q = 0; q < tiles.size(); ++q) work[q] = tile_work(grids[tiles[q].map], hms[tiles[q].map], tiles[q]);
   for (size_t q = 0; q < tiles_x.size(); ++q)
     work_x[q] = (double)std::max(0, tiles_x[q].bin_b - tiles_x[q].bin_a + 1) * tiles_x[q].nrows;
-  balance_tiles(std::vector<gfh_grid>(grids, grids + n_maps), hms, share.blocks * ctx->num_sms, tiles, work);
+  if (!once) balance_tiles(std::vector<gfh_grid>(grids, grids + n_maps), hms, share.blocks * ctx->num_sms, tiles, work);
   sort_tiles(tiles, work);
   sort_tiles(tiles_x, work_x);
   const size_t cells = tile_bytes(tiles, 0, &max_tile_bands);
@@ -1198,8 +1249,10 @@ extern "C" int gfh_plan_autotune(gfh_plan* p, const gfh_peaks* peaks, int32_t re
   }
   rc = time_plan(p, peaks, reps, &best_ms);
   if (rc) return rc;
+  std::vector<gfh_tile_config> tried{p->cfg};
   auto try_shape = [&](const gfh_tile_config& cfg) -> int {
-    if (same_shape(cfg, p->cfg)) return GFH_OK;
+    for (const gfh_tile_config& c : tried)
+      if (same_share(c, cfg)) return GFH_OK;
     gfh_plan* q = nullptr;
     gfh_tile_config c = cfg;
     const int crc = gfh_plan_create(p->ctx, p->n_maps, p->grids.data(), p->h_maps.data(),
@@ -1207,6 +1260,7 @@ extern "C" int gfh_plan_autotune(gfh_plan* p, const gfh_peaks* peaks, int32_t re
                                     &c, &q);
     if (crc == GFH_ERR_SIZE || crc == GFH_ERR_ARG) return GFH_OK;   // shape does not fit
     if (crc) return crc;
+    tried.push_back(cfg);
     float ms = 0.f;
     const int trc = time_plan(q, peaks, reps, &ms);
     gfh_plan_destroy(q);

@@ -1141,7 +1141,7 @@ extern "C" int gfh_hough(gfh_ctx* ctx, const uint32_t* d_fft_idx, const uint32_t
   gfh_plan* p = nullptr;
   int32_t* maps[1] = {d_map};
   gfh_candidate* cands[1] = {d_cands};
-  int rc = gfh_plan_create(ctx, 1, &g1, maps, d_cands ? cands : nullptr, d_stats, nullptr, &p);
+  int rc = gfh_make_plan(ctx, 1, &g1, maps, d_cands ? cands : nullptr, d_stats, nullptr, true, &p);
   if (rc) return rc;
   k_set_offsets<<<1, 32, 0, ctx->stream>>>(p->d_offsets_single, n_peaks);
   rc = cudaGetLastError() == cudaSuccess ? GFH_OK : GFH_ERR_CUDA;

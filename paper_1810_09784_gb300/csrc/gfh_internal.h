@@ -276,6 +276,11 @@ int gfh_host_tables(const gfh_grid* g, std::vector<int64_t>& U, std::vector<int6
 int gfh_host_columns(const gfh_grid* g, std::vector<int32_t>& band, std::vector<double>& f0,
                      std::vector<double>& f0n);
 
+// gfh_plan_create; once: for a single execution, planned in less time.
+int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* const* h_maps,
+                  gfh_candidate* const* h_cands, gfh_map_stats* d_stats, const gfh_tile_config* cfg,
+                  bool once, gfh_plan** out);
+
 // The context's scratch buffer (gfh_peakmap.cu), grown on demand.
 int ensure_scratch(gfh_ctx* c, size_t bytes);
 // Equaliser + peak test + compaction on band spectra d_x [n_fft][ld] holding bins j0 .. j0+ld-1

@@ -3,10 +3,12 @@
 // cover of the tile where they are none.  Cases on stdin, one per line:
 //   n df bin_lo bin_hi n_fft t_first n_k k_min_rows dk_cols rows cols
 // (dk_cols: x0 columns that the last FFT moves per k row; rows = 0: planned tiles, two blocks on each
-// of 152 SMs.)  Prints per case: tiles, FFTs that meet a tile, missed ones, false covers, covers.
+// of 152 SMs; rows = -1: those of a plan that is executed once.)  Prints per case: tiles, FFTs that meet a tile, missed ones, false covers, covers.
 #include "../paper_1810_09784_gb300/csrc/gfh_host.cpp"
 
 #include <cstdio>
+
+static int64_t floor_shift(int64_t v) { return v >> GFH_FRAC_BITS; }
 
 int main() {
   gfh_grid g{};
@@ -30,7 +32,9 @@ int main() {
     find_analysis_columns(hm);
     std::vector<TileDev> tiles;
     hm.one = sparse_map(g, false);
-    if (rows > 0) {
+    if (rows < 0) {
+      sampled_tiles(g, hm, 0, kRoom[2], 304, tiles);
+    } else if (rows > 0) {
       cut_tiles(g, hm, 0, 0, g.n_k, 0, g.ld_x0, rows, cols, tiles);
     } else {
       map_tiles(g, hm, 0, kRoom[2], 0, g.n_k, 0, g.ld_x0, tiles);
@@ -43,7 +47,10 @@ int main() {
     for (const TileDev& t : tiles) {
       const int ub = std::min<int64_t>(t.ncols - 1, g.n_x0 - 1 - t.col0);
       const TileLine line = tile_line(sl, t.row0, (int64_t)t.row0 + t.nrows - 1);
-      for (int j = t.bin_a; j <= t.bin_b; ++j) {
+      // the tile's bins, and the next on either side, of which no FFT may meet it
+      const bool none = t.bin_a > t.bin_b;
+      for (int j = none ? g.bin_lo : std::max(g.bin_lo, t.bin_a - 1); j <= (none ? g.bin_hi : std::min(g.bin_hi, t.bin_b + 1)); ++j) {
+        const bool read = j >= t.bin_a && j <= t.bin_b;
         const int64_t left = hm.U[j - g.bin_lo + 1], right = hm.U[j - g.bin_lo] - 1;
         const BinFfts w = bin_ffts(line, left, right, t.col0, ub, ub == t.ncols - 1, g.n_fft);
         for (int i = 0; i < g.n_fft; ++i) {
@@ -53,7 +60,7 @@ int main() {
           const bool cover = floor_shift(left - first) <= 0 && floor_shift(right - last) >= ub;
           const bool counted = i >= w.lo && i <= w.hi && i > w.c_lo && i < w.c_hi;
           meet += in;
-          missed += in && (i < w.lo || i > w.hi);
+          missed += in && (!read || i < w.lo || i > w.hi);
           covers += counted;
           wrong += counted && !cover;
         }
