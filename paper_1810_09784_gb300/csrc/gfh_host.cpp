@@ -797,8 +797,6 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
   std::vector<char> map_xd(n_maps, 0);
   double cells_xd = 0.0;
   int max_tile_bands = 1, cfg_bands = 1;
-  std::map<int, ListDev> by_list;           // per list read: the bins and FFTs that its maps cover
-  std::map<int, int> list_ffts;
   for (int m = 0; m < n_maps; ++m) {
     const gfh_grid& g = grids[m];
     if (!grid_made(&g) || !h_maps[m]) return GFH_ERR_ARG;
@@ -812,11 +810,6 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
     int64_t ana_cols = 0;
     for (int64_t c = 0; c < g.n_x0; ++c) ana_cols += hm.band[c] >= 0;
     hm.cells = ana_cols * g.n_k;
-    auto ins = by_list.insert({g.list, ListDev{nullptr, nullptr, g.list, g.bin_lo, g.bin_hi + 1, 0, 0, 0, nullptr, 0}});
-    ListDev& ld = ins.first->second;             // n_bins holds the end of the bins for now
-    ld.bin_lo = std::min(ld.bin_lo, g.bin_lo);
-    ld.n_bins = std::max(ld.n_bins, g.bin_hi + 1);
-    list_ffts[g.list] = std::max(list_ffts[g.list], g.n_fft);
     if (((uintptr_t)h_maps[m]) % 16) return GFH_ERR_ARG;  // 16-byte vector stores
     // A line moving more than two columns per k row (coarse k steps, e.g. Eq. dkeqn's) costs
     // fewer events differenced along x0 on every row (2 per row) than along k (the columns it
@@ -861,26 +854,42 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
   const int n_tiles_k = (int)tiles.size();
   tiles.insert(tiles.end(), tiles_x.begin(), tiles_x.end());
 
-  // FFT blocks of 16 to 64, as fine as one per lane of the warp that looks a bin's up allows (a window's
-  // ends are read by whole blocks: 2118 rows x 2540 columns of 652 FFTs 75 -> 71 us); longer ones only
-  // so that a bin has at most 256.
+  // The index: per list the runs of bins that its maps cover, overlapping or adjacent maps in one run.
+  std::vector<int> order(n_maps), run_of(n_maps);
+  std::iota(order.begin(), order.end(), 0);
+  std::sort(order.begin(), order.end(), [&](int a, int b) {
+    return std::make_pair(grids[a].list, grids[a].bin_lo) < std::make_pair(grids[b].list, grids[b].bin_lo);
+  });
   std::vector<ListDev> lists;
-  std::map<int, int> list_at;
+  std::vector<int> ffts;
+  for (int m : order) {
+    const gfh_grid& g = grids[m];
+    const bool joins = !lists.empty() && lists.back().list == g.list &&
+                       g.bin_lo - lists.back().bin_lo <= lists.back().n_bins;
+    if (!joins) {
+      lists.push_back(ListDev{nullptr, nullptr, g.list, g.bin_lo, 0, 0, 0, 0, nullptr, 0});
+      ffts.push_back(0);
+    }
+    ListDev& ld = lists.back();
+    ld.n_bins = std::max(ld.n_bins, g.bin_hi - ld.bin_lo + 1);
+    ffts.back() = std::max(ffts.back(), g.n_fft);
+    run_of[m] = (int)lists.size() - 1;
+  }
   int64_t csr_entries = 0, copy_words = 0;
-  for (auto& kv : by_list) {
-    ListDev ld = kv.second;
-    ld.n_bins -= ld.bin_lo;
+  for (size_t l = 0; l < lists.size(); ++l) {
+    ListDev& ld = lists[l];
+    // FFT blocks of 16 to 64, as fine as one per lane of the warp that looks a bin's up allows (a
+    // window's ends are read by whole blocks: 2118 rows x 2540 columns of 652 FFTs 75 -> 71 us); longer
+    // ones only so that a bin has at most 256.
     ld.shift = 4;
-    while (((list_ffts[kv.first] - 1) >> ld.shift) + 1 > (ld.shift < 6 ? 32 : kMaxFftBlocks)) ++ld.shift;
-    ld.nb1 = ((list_ffts[kv.first] - 1) >> ld.shift) + 2;
+    while (((ffts[l] - 1) >> ld.shift) + 1 > (ld.shift < 6 ? 32 : kMaxFftBlocks)) ++ld.shift;
+    ld.nb1 = ((ffts[l] - 1) >> ld.shift) + 2;
     if (csr_entries + ld.n_bins > INT32_MAX) return GFH_ERR_SIZE;
     ld.entry0 = (int32_t)csr_entries;
     csr_entries += ld.n_bins;
     // room to order a list out of FFT order: an eighth of its (FFT, bin) pairs, noise peaks and more
-    ld.cap = (int64_t)ld.n_bins * list_ffts[kv.first] / 8 + 1024;
+    ld.cap = (int64_t)ld.n_bins * ffts[l] / 8 + 1024;
     copy_words += ld.cap;
-    list_at[kv.first] = (int)lists.size();
-    lists.push_back(ld);
   }
 
   // One device buffer: map descriptors | tiles | lists | index list of each bin | keys | per-map tables.
@@ -961,7 +970,7 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
     md.col_band = (const int32_t*)(base + o_band[m]);
     md.f0c = (const double*)(base + o_f0[m]);
     md.f0n = (const double*)(base + o_f0n[m]);
-    const ListDev& ld = lists[list_at[g.list]];
+    const ListDev& ld = lists[run_of[m]];
     md.csr = ld.csr + (g.bin_lo - ld.bin_lo);
     md.blk = ld.blk + (size_t)(g.bin_lo - ld.bin_lo) * ld.nb1;
     md.csr_list = ld.csr;

@@ -180,7 +180,7 @@ struct MapDev {
   const int64_t* csr;       // J + 1 entries: first peak (absolute index) of bins bin_lo .. bin_hi+1
   const int32_t* blk;       // [J][nb1]: offset in a bin's peaks of its first of FFT >= 2^shift b
   int32_t nb1, shift;
-  const int64_t* csr_list;  // first peak of the list's first indexed bin
+  const int64_t* csr_list;  // first peak of the run's first bin
   const uint32_t* copy;     // the list's FFT indices from there, by blocks (lists out of FFT order)
   unsigned long long* keys; // n_bands
   unsigned long long* sums; // 2: sum, sum of squares
@@ -201,7 +201,7 @@ struct MapDev {
 // FFT blocks of a bin, at most.
 constexpr int kMaxFftBlocks = 256;
 
-// The index of one peak list, over the bins that some map reads (built per execute, k_index).
+// The index of a peak list over a run of bins that maps read (built per execute, k_index).
 struct ListDev {
   int64_t* csr;             // n_bins + 1
   int32_t* blk;             // [n_bins][nb1]
@@ -251,7 +251,7 @@ struct gfh_plan {
   int n_list_states = 0;                  // largest list index + 1
   int* d_next = nullptr;
   int* d_sel_count = nullptr;
-  ListDev* d_lists = nullptr;             // the peak lists that maps read
+  ListDev* d_lists = nullptr;             // the runs of bins that maps read
   int32_t csr_entries = 0;                // their bins in all
   int32_t* d_csr_list = nullptr;          // per bin: its entry of d_lists
   bool select = false;
