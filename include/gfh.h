@@ -303,9 +303,9 @@ int gfh_plan_execute(gfh_plan* plan, const gfh_peaks* peaks);
  * Autotuner: times gfh_plan_execute on these peaks (reps runs each, CUDA events on the context's
  * stream) for the current tile shape and for every shape of rows {4, 8, 16} x cols {1024, 2048,
  * 3072, 4096} x threads {256, 512} (and 1024 threads for 16 rows) that fits in shared memory and
- * makes another plan (other threads or blocks per SM), and rebuilds the plan with the fastest.  The
- * results are unchanged by the shape (the maps are exact).  Synchronises; writes the bound outputs.
- * h_best / h_best_ms (may be NULL) receive the
+ * makes another plan (other threads or blocks per SM), and rebuilds the plan with the fastest, if it
+ * is faster than the current one by more than 2 %.  The results are unchanged by the shape (the maps
+ * are exact).  Synchronises; writes the bound outputs.  h_best / h_best_ms (may be NULL) receive the
  * chosen shape and its time.
  * The choice is cached for the life of the process, keyed by the plan's signature: the device
  * (compute capability, SM count), whether candidates are selected, and per map its k rows, x0
