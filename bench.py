@@ -860,9 +860,7 @@ def _roofline_of(ctx, stream, updates, map_bytes, ms):
 
 def measure_batched_n(ctx, stream, steps, warmup, tile=(16, 3072, 1024, 1)):
     """Config 3: the plain_small peakmap at 51 braking indices, one launch (CUDA graph), against
-    one plan per braking index run one after another.  The tile draws one form per warp (form 1):
-    measured 20.3 ms against 21.1 ms with each peak in its own form, maps identical (the tall
-    low-n maps mix interior and edge peaks in many warps)."""
+    one plan per braking index run one after another."""
     import torch
     from paper_1810_09784_gb300 import gfh
     spec, pm, grid_fields = workloads.batched_n(seed=ranks.rank_seed(1, 0))
@@ -1308,7 +1306,7 @@ def run_proposer(args):
         "data": res["data"], "config": {"workload": res["workload"], "checkpoint": res["checkpoint"]},
         "proposer": res, "speedup_vs_full_exact": res["speedup_vs_full_exact"],
         "recall": res["recall"], "operating_point": res["operating_point"],
-        "roofline": {"bound": "tensor", "kernel": "network forward (k_conv_fwd_tc, 5 layers)",
+        "roofline": {"bound": "tensor", "kernel": "network forward (k_conv_tma, 5 layers)",
                      "achieved": NET_FWD_FLOP * 51 / (res["network_forward_ms_51_maps"] * 1e-3) / 1e12,
                      "peak": PEAKS.get("bf16_tflops"), "unit": "TFLOP/s",
                      "frac": (NET_FWD_FLOP * 51 / (res["network_forward_ms_51_maps"] * 1e-3) / 1e12

@@ -643,7 +643,7 @@ __device__ __forceinline__ void async_proxy_fence() {
 // wait is bounded and a wait that runs out raises the timeout flag and ends the block's loop.
 // Input views for the copies (NHWC bf16, fully packed): S = 1: (CIN, W, H, B); S = 2: (CIN, 2, W/2,
 // H, B), whose parity coordinate picks the even or odd input columns, so entry j of parity 0 is
-// column 2 (x0 + j) - 1 and of parity 1 column 2 (x0 + j), as in k_conv_fwd_tc.
+// column 2 (x0 + j) - 1 and of parity 1 column 2 (x0 + j).
 // MODE 2, the input gradient of a stride-2 layer, is split by output parity instead of running on
 // inserted zeros: din[y][x] = sum over taps (dy, dx) with y + dy - 1 and x + dx - 1 even of
 // G[(y + dy - 1) / 2][(x + dx - 1) / 2] Wf[dy][dx] (Wf the flipped, transposed weights of MODE 1).

@@ -943,7 +943,6 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
     for (ListDev& ld : lists) ld.cap = 0;
     if (cudaMalloc(&p->d_buf, total) != cudaSuccess) { delete p; return GFH_ERR_NOMEM; }
   }
-  p->buf_bytes = total;
   char* base = (char*)p->d_buf;
   std::vector<char> h(total, 0);
   std::vector<MapDev> mds(n_maps);
@@ -1063,7 +1062,7 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
   std::vector<TileDev> fine;
   std::vector<int32_t> first;
   first.reserve((size_t)p->n_maps * (nct + 1) + 1);
-  int max_fine = 0, max_bands = p->max_tile_bands;
+  int max_bands = p->max_tile_bands;
   size_t worst = 0;                        // longest gathered list: every map at its largest
   for (int m = 0; m < p->n_maps; ++m) {
     const gfh_grid& g = p->grids[m];
@@ -1100,7 +1099,6 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
           map_tiles(g, hm, m, p->list_room, r0, r1, c_lo, c_hi, fine);
         }
         const int cnt = (int)(fine.size() - before);
-        max_fine = std::max(max_fine, cnt);
         sizes.push_back(cnt);
       }
     }
@@ -1142,7 +1140,6 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
   p->coarse_k = coarse_k;
   p->coarse_x = coarse_x;
   p->max_sel = max_sel;
-  p->max_fine = max_fine;
   p->max_tile_bands = max_bands;
   p->cells_list = cells_list;
   return GFH_OK;

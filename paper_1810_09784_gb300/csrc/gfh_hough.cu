@@ -254,8 +254,9 @@ __device__ __forceinline__ void events(uint64_t& v1, uint64_t& v2, uint64_t D, u
 // position p on row 0, f = frac(p), crosses its (e+1)-th column boundary (e = 0, 1, ...) at the
 // first row r with r s > f + e 2^32, so r = floor(x_e) + 1 with x_e = (f + e 2^32) / s.  x_e is kept
 // in rows of 2^-57 and stepped by D = ceil(2^89 / s), the rows per column (a table entry per FFT):
-// every rounding is upwards and below 130 units of 2^-57 in all, while an x_e that is no integer
-// lies at least 1/s >= 2^-33 below the next one, so floor() is exact.  The left edge enters a
+// every rounding is upwards and below 256 units of 2^-57 in all (at most 254 steps: two columns on each
+// of 127 rows), while an x_e that is no integer lies at least 1/s >= 2^-33 below the next one, so
+// floor() is exact.  The left edge enters a
 // column at its event (one lower each event), the right edge leaves one.
 // Lanes of a warp hold neighbouring FFTs of one bin, whose s, and so whose event counts, are nearly
 // alike: the loop runs to the warp's largest count.
@@ -407,8 +408,7 @@ __device__ __forceinline__ void fill_tile(const MapDev& md, const TileDev& t, in
 // a time whatever bins they are of.  A tile that no edge meets holds one number and needs no sums.
 //
 // What bounds it: on dense maps (20 sub-band maps of 2000 rows, 226M cells, 8.8e9 peak rows) the
-// events' integer instructions, about 7 per event, and the increments' bank conflicts (2.4 wavefronts
-// each): 4.68 ms against 7.56 ms for the row-by-row form on flat 16 x 3072 tiles.  On sparse maps
+// events' integer instructions and the increments' bank conflicts: 4.63 ms against 7.56 ms for the row-by-row form on flat 16 x 3072 tiles.  On sparse maps
 // (11 braking indices, 1.76e9 cells, 1.3 peak rows per cell) the tiles' chain of dependent loads and
 // barriers: with one count per cell 4.04 against 5.67 ms, five maps of 228-1858 rows x 85,654-164,343
 // columns 1.10 against 1.46 ms.  Small maps gain from the planned tiles (whole calls): 500 rows x 51,695

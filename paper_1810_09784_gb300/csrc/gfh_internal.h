@@ -235,7 +235,6 @@ struct gfh_plan {
   size_t cells = 0, cells_x = 0, cells_list = 0;   // shared memory of the largest tile's counts: full
                                                    // search's two lists, coarse tiles
   void* d_buf = nullptr;       // tables, map descriptors, tiles
-  size_t buf_bytes = 0;
   MapDev* d_maps = nullptr;
   TileDev* d_tiles = nullptr;          // tiles of x-direction maps follow the others
   int n_tiles = 0;                     // tiles differenced along k (rows > 0)
@@ -262,7 +261,7 @@ struct gfh_plan {
   gfh_map_stats* d_stats = nullptr;
   // coarse tiles (gfh_plan_set_coarse): per (map, coarse tile) the fine tiles that cover it
   // (group coarse_k * coarse_x of a map = all of the map's tiles, for a full search)
-  int coarse_k = 0, coarse_x = 0, max_sel = 0, max_fine = 0;
+  int coarse_k = 0, coarse_x = 0, max_sel = 0;
   void* d_coarse_buf = nullptr;
   TileDev* d_fine = nullptr;           // fine tiles, grouped by (map, coarse tile)
   int32_t* d_coarse_first = nullptr;   // n_maps * (coarse_k * coarse_x + 1) + 1 group offsets
@@ -298,4 +297,3 @@ int gfh_launch_plan(gfh_plan* plan, const gfh_peaks* peaks);
 int gfh_launch_plan_tiles(gfh_plan* plan, const gfh_peaks* peaks, const int32_t* d_coarse,
                           int n_sel, const int32_t* d_full);
 int gfh_prepare_plan(gfh_plan* plan);   // one-time kernel attributes (outside any capture)
-int gfh_launch_select(gfh_ctx* ctx, const int32_t* d_map, const MapDev& md, void* d_scratch);
