@@ -906,7 +906,7 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
   }
   size_t key_words = 0;
   for (int m = 0; m < n_maps; ++m) key_words += grids[m].n_bands + 2;
-  // (a launch takes at most 65535 lists)
+  // (an execution takes at most 65535 lists)
   int n_lists = 1;
   for (int m = 0; m < n_maps; ++m) n_lists = std::max(n_lists, std::min(grids[m].list, 65535) + 1);
   const size_t zeroed = sizeof(unsigned long long) * key_words + sizeof(int) * ((size_t)n_lists + 4);

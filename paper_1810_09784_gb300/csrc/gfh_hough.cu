@@ -59,26 +59,42 @@ __device__ __forceinline__ unsigned long long cand_key(int count, uint32_t lin) 
 // Order of each peak list (state[l], l < n_states, zeroed before): kListUnsorted when its bins are not ascending
 // (also flagged; such a list is not drawn), kListFftUnsorted when some bin's peaks are not in FFT
 // order (k_index then copies them by blocks of FFTs).
+//
+// The blocks share out the peaks of all lists evenly, whatever the lists' lengths.  Bound by its 8 bytes
+// per peak; with 8 blocks for each of 256 lists of 18 thousand to 18 million peaks it took 8 ms, the
+// longest list's, where the bytes take 0.6.
 __global__ void k_check_sorted(const uint32_t* __restrict__ bins, const uint32_t* __restrict__ fft,
-                               const int64_t* __restrict__ off, unsigned int* flag,
+                               const int64_t* __restrict__ off, int n_lists, unsigned int* flag,
                                int* __restrict__ state, int n_states) {
-  const int l = blockIdx.y;
-  const int64_t b = off[l], e = off[l + 1];
-  int bad = 0;
-  // four independent pairs per turn
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t p0 = b + 1 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p0 < e; p0 += 4 * step) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int64_t p = p0 + q * step;
-      if (p >= e) continue;
-      const uint32_t j1 = bins[p], j0 = bins[p - 1], f1 = fft[p], f0 = fft[p - 1];
-      if (j1 < j0) bad |= kListUnsorted;
-      else if (j1 == j0 && f1 < f0) bad |= kListFftUnsorted;
-    }
+  const int64_t begin = off[0], total = off[n_lists] - begin;
+  const int64_t part = ((total + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
+  const int64_t c0 = begin + blockIdx.x * part, c1 = min(c0 + part, begin + total);
+  if (c0 >= c1) return;
+  int l = 0;                                       // last list that begins at or before c0
+  for (int hi = n_lists - 1; l < hi;) {
+    const int mid = (l + hi + 1) / 2;
+    if (off[mid] <= c0) l = mid; else hi = mid - 1;
   }
-  if (bad & kListUnsorted) atomicOr(flag, GFH_FLAG_UNSORTED);
-  if (bad && l < n_states) atomicOr(&state[l], bad);
+  for (; l < n_lists && off[l] < c1; ++l) {
+    const int64_t b = max(off[l] + 1, c0), e = min(off[l + 1], c1);
+    int bad = 0;
+    // four independent pairs per turn
+    for (int64_t p0 = b + threadIdx.x; p0 < e; p0 += 4 * blockDim.x) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t p = p0 + q * blockDim.x;
+        if (p >= e) continue;
+        const uint32_t j1 = bins[p], j0 = bins[p - 1], f1 = fft[p], f0 = fft[p - 1];
+        if (j1 < j0) bad |= kListUnsorted;
+        else if (j1 == j0 && f1 < f0) bad |= kListFftUnsorted;
+      }
+    }
+    // one lane per warp, and only what is not known yet
+    bad = (int)__reduce_or_sync(0xffffffffu, (unsigned)bad);
+    if (threadIdx.x % kLane) continue;
+    if (bad & kListUnsorted) atomicOr(flag, GFH_FLAG_UNSORTED);
+    if (l < n_states && (bad & ~*reinterpret_cast<volatile int*>(&state[l]))) atomicOr(&state[l], bad);
+  }
 }
 
 // First of the list's peaks [lo, hi) with bin >= key, by the whole warp (a 32-way search, five bits a
@@ -1077,14 +1093,11 @@ int gfh_prepare_plan(gfh_plan* p) {
 static int launch_prologue(gfh_plan* p, const gfh_peaks* peaks) {
   gfh_ctx* ctx = p->ctx;
   cudaStream_t st = ctx->stream;
+  if (peaks->n_lists > 65535) return GFH_ERR_CUDA;   // (the lists' states, and other launches, stop there)
   GFH_CUDA_TRY(cudaMemsetAsync(p->d_zeroed, 0, p->zeroed_bytes, st));
-  {
-    // a few blocks per SM in all, at least 8 per list
-    dim3 grid(std::max(8, 4 * ctx->num_sms / peaks->n_lists), peaks->n_lists);
-    k_check_sorted<<<grid, 256, 0, st>>>(peaks->bin, peaks->fft_idx, peaks->offsets, ctx->d_flag,
-                                         p->d_list_state, p->n_list_states);
-    GFH_CUDA_TRY(cudaGetLastError());
-  }
+  k_check_sorted<<<4 * ctx->num_sms, 256, 0, st>>>(peaks->bin, peaks->fft_idx, peaks->offsets, peaks->n_lists,
+                                                   ctx->d_flag, p->d_list_state, p->n_list_states);
+  GFH_CUDA_TRY(cudaGetLastError());
   k_index<<<(p->csr_entries + kIndexWarps - 1) / kIndexWarps, kIndexWarps * kLane, 0, st>>>(
       p->d_lists, p->d_csr_list, p->csr_entries, peaks->bin, peaks->fft_idx, peaks->offsets, p->d_list_state);
   GFH_CUDA_TRY(cudaGetLastError());
