@@ -423,13 +423,16 @@ __device__ __forceinline__ void fill_tile(const MapDev& md, const TileDev& t, in
 // where its peaks lie in the list less its begin}.  Each warp walks one contiguous part, 32 peaks at
 // a time whatever bins they are of.  A tile that no edge meets holds one number and needs no sums.
 //
-// What bounds it: on dense maps (20 sub-band maps of 2000 rows, 226M cells, 8.8e9 peak rows) the
-// events' integer instructions and the increments' bank conflicts: 4.63 ms against 7.56 ms for the row-by-row form on flat 16 x 3072 tiles.  On sparse maps
-// (11 braking indices, 1.76e9 cells, 1.3 peak rows per cell) the tiles' chain of dependent loads and
-// barriers: with one count per cell 4.04 against 5.67 ms, five maps of 228-1858 rows x 85,654-164,343
-// columns 1.10 against 1.46 ms.  Small maps gain from the planned tiles (whole calls): 500 rows x 51,695
-// columns 134 against 234 us, the 32 rows of a followed-up candidate 42 against 86 us, 12 uneven
-// peakmaps 0.49 against 1.42 ms.
+// What bounds it: on dense maps (20 sub-band maps of 2000 rows, 226M cells, 9.0e9 peak rows) the
+// events' integer instructions (0.48 warp instructions per peak row in all, about 70 % of the issue slots) and
+// the increments' bank conflicts (2.43 wavefronts each): 4.64 ms against 7.56 ms for the row-by-row form
+// on flat 16 x 3072 tiles.  On sparse maps (11 braking indices, 1.76e9 cells, 1.3 peak rows per cell)
+// the tiles' chain of dependent loads and barriers (44 % of the issue slots): with one count per cell
+// 4.04 against 5.67 ms, five maps of 228-1858 rows x 85,654-164,343 columns 1.10 against 1.46 ms.  Small
+// maps gain from the planned tiles (whole calls): 500 rows x 51,695 columns 102 against 234 us, the 32
+// rows of a followed-up candidate 41 against 86 us, 12 uneven peakmaps 0.48 against 1.42 ms.  Tall maps of
+// a few hundred FFTs can be the slower ones by up to a tenth (2118 rows x 2540 columns of 652 FFTs 70
+// against 65 us): their windows are a few peaks of many bins.
 //
 // Shared memory: tot[32] row-0 chunk sums | spare words | skey[bands] candidate keys | sums per warp
 // | ent[2 batch] | G.
