@@ -417,16 +417,22 @@ void find_analysis_columns(HostMap& hm) {
 constexpr double kNoisePeaks = 0.0755;
 
 // Whether a map is drawn with one count per cell (+1 and -1) and not with two (+1 each).  Two halve a
-// tile, one makes lanes that leave the same column wait for each other.  Tiles of a map with few peaks
-// per column cost what their cells and chains of loads cost: fewer, larger ones are faster below two
-// (x0 columns counted, each peak of the band on each of them once): 51 half-hour maps (0.85) 7.00 ->
-// 4.73 ms, 11 braking indices (1.3) 5.78 -> 3.83 ms, one half-hour map (1.6) 138 -> 105 us.  Above,
-// 0.81 to 0.92 of the speed at 2.9 to 3.1, half at 50 (75 drawn plans, 12 uneven peakmaps).
+// tile, one makes lanes that leave the same column wait for each other.  With few peaks per x0 column a
+// tile costs what its cells and chains of loads cost, and fewer, larger ones are faster: 51 half-hour
+// maps (0.85 peaks per column) 7.00 -> 4.73 ms, 11 braking indices (0.15 to 12.7) 5.78 -> 4.04 ms, one
+// half-hour map (1.6) 138 -> 102 us.  The line lies at two peaks per column where neighbouring peaks of a
+// bin, on the map's middle row, lie two columns apart (at 2.9 to 3.1 peaks 0.81 to 0.92 of the speed, at
+// 50 half of it), and falls to one where they share a column (at 1.1 to 1.6 peaks 0.85 of the speed, at
+// 0.6 to 0.75 1.44 of it).
 // The x-direction form counts a left column on every row, so there the line lies at one: half-hour map
 // at 3 and 12 columns per row (1.6) 238 -> 176 and 202 -> 186 us with two counts, 11 braking indices at 4
-// columns (0.15 to 12.7) 2.90 -> 2.55 ms with one for the maps below one.
-bool sparse_map(const gfh_grid& g, bool xd) {
-  return kNoisePeaks * g.n_fft * (double)(g.bin_hi - g.bin_lo + 1) < (xd ? 1.0 : 2.0) * (double)g.n_x0;
+// columns 2.90 -> 2.55 ms with one for the maps below one.
+bool sparse_map(const gfh_grid& g, const HostMap& hm, bool xd) {
+  const double per_column = kNoisePeaks * g.n_fft * (double)(g.bin_hi - g.bin_lo + 1) / (double)g.n_x0;
+  if (xd) return per_column < 1.0;
+  const double shift = (double)(hm.B.back() - hm.B[0]) + 0.5 * g.n_k * (double)(hm.S.back() - hm.S[0]);
+  const double apart = std::fabs(shift) / 4294967296.0 / std::max(1, g.n_fft - 1) / kNoisePeaks;
+  return per_column < 1.0 + std::min(1.0, 0.5 * apart);
 }
 
 // Bin range [ja, jb] of the peaks that can touch columns [c0, c1) on rows [r0, r1) (tile planning).
@@ -795,7 +801,7 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
   std::vector<HostMap> hms(n_maps);
   std::vector<TileDev> tiles, tiles_x;
   std::vector<char> map_xd(n_maps, 0);
-  double cells_xd = 0.0;
+  double cells_k = 0.0, cells_xd = 0.0;
   int max_tile_bands = 1, cfg_bands = 1;
   for (int m = 0; m < n_maps; ++m) {
     const gfh_grid& g = grids[m];
@@ -815,16 +821,24 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
     // fewer events differenced along x0 on every row (2 per row) than along k (the columns it
     // crosses): such maps use the x-direction form.
     map_xd[m] = hm.S[g.n_fft - 1] > (int64_t(2) << GFH_FRAC_BITS);
-    hm.one = sparse_map(g, map_xd[m]);
+    hm.one = sparse_map(g, hm, map_xd[m]);
+    (map_xd[m] ? cells_xd : cells_k) += (double)g.n_k * (double)g.ld_x0;
     find_analysis_columns(hm);
     for (int64_t c = 0; c < g.ld_x0; c += tc.cols) {
       int32_t lo, hi;
       column_bands(hm, c, std::min<int64_t>(c + tc.cols, g.ld_x0), &lo, &hi);
       cfg_bands = std::max(cfg_bands, hi - lo + 1);
     }
-    if (map_xd[m]) cells_xd += (double)g.n_k * (double)g.ld_x0;
-    else if (once) sampled_tiles(g, hm, m, share.room, share.blocks * ctx->num_sms, tiles);
-    else map_tiles(g, hm, m, share.room, 0, g.n_k, 0, g.ld_x0, tiles);
+  }
+  // Twice the cells per tile are of no use where two counts make no more tiles than one and a half for
+  // each block (2 to 7 Mcells: 0.90 to 1.19 of the speed with one).
+  const bool few = cells_k < 1.5 * 0.5 * (double)share.room * share.blocks * ctx->num_sms;
+  for (int m = 0; m < n_maps; ++m) {
+    if (map_xd[m]) continue;
+    HostMap& hm = hms[m];
+    hm.one = hm.one && !few;
+    if (once) sampled_tiles(grids[m], hm, m, share.room, share.blocks * ctx->num_sms, tiles);
+    else map_tiles(grids[m], hm, m, share.room, 0, grids[m].n_k, 0, grids[m].ld_x0, tiles);
   }
   // x-direction tiles: uniform strips of 8 rows, four and more to each block of three per SM as far as
   // 256 columns allow.  (Tiles of 16 rows keep 16 carries in registers and fill an SM with one block,
@@ -1017,6 +1031,7 @@ int gfh_make_plan(gfh_ctx* ctx, int32_t n_maps, const gfh_grid* grids, int32_t* 
   p->n_tiles = n_tiles_k;
   p->n_tiles_x = (int)tiles.size() - n_tiles_k;
   p->map_xd = map_xd;
+  for (const HostMap& hm : hms) p->map_one.push_back(hm.one);
   p->max_tile_bands = max_tile_bands;
   p->d_zeroed = base + o_keys;
   p->zeroed_bytes = zeroed;
@@ -1071,7 +1086,7 @@ extern "C" int gfh_plan_set_coarse(gfh_plan* p, int32_t coarse_k, int32_t coarse
     if (rc) return rc;
     rc = gfh_host_columns(&g, hm.band, hm.f0, hm.f0n);
     if (rc) return rc;
-    hm.one = sparse_map(g, false);
+    hm.one = p->map_one[m];
     find_analysis_columns(hm);
     // columns of each f0 tile: analysis columns only; f0 falls with the column, so each range is
     // contiguous

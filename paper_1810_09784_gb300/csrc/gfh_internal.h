@@ -239,7 +239,7 @@ struct gfh_plan {
   TileDev* d_tiles = nullptr;          // tiles of x-direction maps follow the others
   int n_tiles = 0;                     // tiles differenced along k (rows > 0)
   int n_tiles_x = 0;                   // tiles of maps moving > 2 columns per k row: along x0
-  std::vector<char> map_xd;            // per map: drawn in the x-direction form
+  std::vector<char> map_xd, map_one;   // per map: drawn in the x-direction form, with one count per cell
   int max_tile_bands = 0;
   // zeroed per execute, in one piece: all maps' keys and sums, the lists' order states, the tile
   // counters (full search's two launches; coarse-tile list length and next tile)

@@ -31,7 +31,7 @@ int main() {
     if (gfh_host_tables(&g, hm.U, hm.B, hm.S) || gfh_host_columns(&g, hm.band, hm.f0, hm.f0n)) return 1;
     find_analysis_columns(hm);
     std::vector<TileDev> tiles;
-    hm.one = sparse_map(g, false);
+    hm.one = sparse_map(g, hm, false);
     if (rows < 0) {
       sampled_tiles(g, hm, 0, kRoom[2], 304, tiles);
     } else if (rows > 0) {

@@ -27,9 +27,12 @@ CASES = {
     "t0_zero": fields_of(5.0, 150, 300, 24, 9, t_first=0.0),
 }
 DENSE = fields_of(5.0, 200, 150, 200, 60)
+# small plans take two counts whatever their maps: a map of 8 million cells without peaks beside them
+LARGE = fields_of(7.0, 140, 420, 60, 20)
 
 
 def check(gfh, ctx, fields, tile, seed=11):
+    fields = fields + [dict(LARGE, list=len(fields))]
     grids = [gfh.grid_make(gfh.Grid(**f)) for f in fields]
     maps = [torch.full((g.n_k, g.ld_x0), -7, dtype=torch.int32, device="cuda") for g in grids]
     cands = [torch.zeros(g.n_bands * 64, dtype=torch.uint8, device="cuda") for g in grids]
@@ -37,13 +40,15 @@ def check(gfh, ctx, fields, tile, seed=11):
     plan = gfh.Plan(ctx, grids, maps, cands, stats, tile=tile)
     lists = [synth.random_peaklist(f["n_fft"], f["bin_lo"] - 2, f["bin_hi"] + 2, 0.08, seed + i)
              for i, f in enumerate(fields)]
+    lists[-1] = tuple(x[:0] for x in lists[-1])
     off = np.cumsum([0] + [len(l[0]) for l in lists]).astype(np.int64)
     plan.execute(*(to_dev(torch, np.concatenate([l[k] for l in lists])) for k in (0, 1)), to_dev(torch, off),
                  len(lists))
     torch.cuda.synchronize()
     assert ctx.check() == gfh.GFH_OK
     st = read_stats(gfh, stats)
-    for i, (f, g) in enumerate(zip(fields, grids)):
+    assert not maps.pop().any()
+    for i, (f, g) in enumerate(zip(fields[:-1], grids)):
         ref = O.hough_map(oracle_grid(f), *lists[i])
         got = maps[i].cpu().numpy()
         assert np.array_equal(got[:, : g.n_x0], ref)
