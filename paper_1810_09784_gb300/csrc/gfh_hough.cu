@@ -63,26 +63,28 @@ __device__ __forceinline__ unsigned long long cand_key(int count, uint32_t lin) 
 // The blocks share out the peaks of all lists evenly, whatever the lists' lengths.  Bound by its 8 bytes
 // per peak; with 8 blocks for each of 256 lists of 18 thousand to 18 million peaks it took 8 ms, the
 // longest list's, where the bytes take 0.6.
-__global__ void k_check_sorted(const uint32_t* __restrict__ bins, const uint32_t* __restrict__ fft,
-                               const int64_t* __restrict__ off, int n_lists, unsigned int* flag,
-                               int* __restrict__ state, int n_states) {
-  const int64_t begin = off[0], total = off[n_lists] - begin;
-  const int64_t part = ((total + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
-  const int64_t c0 = begin + blockIdx.x * part, c1 = min(c0 + part, begin + total);
+__global__ void __launch_bounds__(256) k_check_sorted(const uint32_t* __restrict__ bins, const uint32_t* __restrict__ fft,
+                               const int64_t* __restrict__ off, int n_lists, float per_block,
+                               unsigned int* flag, int* __restrict__ state, int n_states) {
+  const int64_t begin = off[0], end = off[n_lists];
+  // an equal part, a little more for float32's rounding, of at least a pair per thread
+  const int64_t part = max((int64_t)((float)(end - begin) * per_block) + 32, (int64_t)256) & ~(int64_t)31;
+  const int64_t c0 = begin + blockIdx.x * part, c1 = min(c0 + part, end);
   if (c0 >= c1) return;
   int l = 0;                                       // last list that begins at or before c0
   for (int hi = n_lists - 1; l < hi;) {
     const int mid = (l + hi + 1) / 2;
     if (off[mid] <= c0) l = mid; else hi = mid - 1;
   }
-  for (; l < n_lists && off[l] < c1; ++l) {
-    const int64_t b = max(off[l] + 1, c0), e = min(off[l + 1], c1);
+  for (int64_t first = n_lists == 1 ? begin : off[l]; first < c1;) {
+    const int64_t next = n_lists == 1 ? end : off[l + 1];
+    const int64_t b = max(first + 1, c0), e = min(next, c1);
     int bad = 0;
     // four independent pairs per turn
-    for (int64_t p0 = b + threadIdx.x; p0 < e; p0 += 4 * blockDim.x) {
+    for (int64_t p0 = b + threadIdx.x; p0 < e; p0 += 4 * 256) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int64_t p = p0 + q * blockDim.x;
+        const int64_t p = p0 + q * 256;
         if (p >= e) continue;
         const uint32_t j1 = bins[p], j0 = bins[p - 1], f1 = fft[p], f0 = fft[p - 1];
         if (j1 < j0) bad |= kListUnsorted;
@@ -91,9 +93,12 @@ __global__ void k_check_sorted(const uint32_t* __restrict__ bins, const uint32_t
     }
     // one lane per warp, and only what is not known yet
     bad = (int)__reduce_or_sync(0xffffffffu, (unsigned)bad);
-    if (threadIdx.x % kLane) continue;
-    if (bad & kListUnsorted) atomicOr(flag, GFH_FLAG_UNSORTED);
-    if (l < n_states && (bad & ~*reinterpret_cast<volatile int*>(&state[l]))) atomicOr(&state[l], bad);
+    if (bad && threadIdx.x % kLane == 0) {
+      if (bad & kListUnsorted) atomicOr(flag, GFH_FLAG_UNSORTED);
+      if (l < n_states && (bad & ~*reinterpret_cast<volatile int*>(&state[l]))) atomicOr(&state[l], bad);
+    }
+    if (++l >= n_lists) break;
+    first = next;
   }
 }
 
@@ -161,6 +166,7 @@ k_index(const ListDev* __restrict__ lists, const int32_t* __restrict__ entry_lis
   if (e >= n_entries) return;
   const ListDev& ld = lists[entry_list[e]];
   const int jl = e - ld.entry0;
+  const int st = state[ld.list];
   // first peaks with bin >= key and >= key + 1
   int64_t lo[2], hi[2];
 #pragma unroll
@@ -186,7 +192,6 @@ k_index(const ListDev* __restrict__ lists, const int32_t* __restrict__ entry_lis
   }
   const int n = (int)(lo[1] - lo[0]);
   int32_t* const begin = ld.blk + (int64_t)jl * ld.nb1;
-  const int st = state[ld.list];
   if ((st & kListFftUnsorted) && !(st & kListUnsorted)) {
     const int64_t at = lo[0] - first_of_bin(bins, off[ld.list], off[ld.list + 1], (uint32_t)ld.bin_lo, lane);
     if (at + n <= ld.cap)
@@ -1098,8 +1103,10 @@ static int launch_prologue(gfh_plan* p, const gfh_peaks* peaks) {
   cudaStream_t st = ctx->stream;
   if (peaks->n_lists > 65535) return GFH_ERR_CUDA;   // (the lists' states, and other launches, stop there)
   GFH_CUDA_TRY(cudaMemsetAsync(p->d_zeroed, 0, p->zeroed_bytes, st));
-  k_check_sorted<<<4 * ctx->num_sms, 256, 0, st>>>(peaks->bin, peaks->fft_idx, peaks->offsets, peaks->n_lists,
-                                                   ctx->d_flag, p->d_list_state, p->n_list_states);
+  const int check_blocks = 4 * ctx->num_sms;
+  k_check_sorted<<<check_blocks, 256, 0, st>>>(peaks->bin, peaks->fft_idx, peaks->offsets, peaks->n_lists,
+                                               (1.f + 0x1p-20f) / check_blocks, ctx->d_flag, p->d_list_state,
+                                               p->n_list_states);
   GFH_CUDA_TRY(cudaGetLastError());
   k_index<<<(p->csr_entries + kIndexWarps - 1) / kIndexWarps, kIndexWarps * kLane, 0, st>>>(
       p->d_lists, p->d_csr_list, p->csr_entries, peaks->bin, peaks->fft_idx, peaks->offsets, p->d_list_state);
