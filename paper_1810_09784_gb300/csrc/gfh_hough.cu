@@ -436,8 +436,8 @@ __device__ __forceinline__ void fill_tile(const MapDev& md, const TileDev& t, in
 // 4.04 against 5.67 ms, five maps of 228-1858 rows x 85,654-164,343 columns 1.10 against 1.46 ms.  Small
 // maps gain from the planned tiles (whole calls): 500 rows x 51,695 columns 102 against 234 us, the 32
 // rows of a followed-up candidate 41 against 86 us, 12 uneven peakmaps 0.48 against 1.42 ms.  Tall maps of
-// a few hundred FFTs can be the slower ones by up to a tenth (2118 rows x 2540 columns of 652 FFTs 70
-// against 65 us): their windows are a few peaks of many bins.
+// a few hundred FFTs can be the slower ones, by up to a fifth below 75 us a call (2118 rows x 2540
+// columns of 652 FFTs 73 against 65 us): their windows are a few peaks of many bins.
 //
 // Shared memory: tot[32] row-0 chunk sums | spare words | skey[bands] candidate keys | sums per warp
 // | ent[2 batch] | G.
